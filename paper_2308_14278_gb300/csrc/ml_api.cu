@@ -1042,19 +1042,25 @@ ShootArgs make_args(const ml_field *f)
     return a;
 }
 
-// Task decomposition of rays [b, e) for the mixed kernel.
-void set_tasks(ShootArgs &a, const Geo &g, int64_t b, int64_t e)
+// Task decomposition of rays [b, e) for the mixed kernel.  A task's level-2
+// columns (about 2048 rays along a row, within one level-1 cell) share the
+// staging of its near lenses.  Small launches take fewer columns per task,
+// down to one, so that about two tasks come on each of the GPU's 24 resident
+// warps per SM: a launch of a few hundred tasks otherwise leaves most warps
+// idle and ends with its longest one.
+void set_tasks(ShootArgs &a, const Geo &g, int64_t b, int64_t e, int num_sms)
 {
     a.ray_begin = b;
     a.ray_end = e;
     const int64_t gpb = (g.n1y + 31) / 32;
-    const int64_t l2_per_cc = std::max<int64_t>(1, std::min<int64_t>(g.l2sx, (2048 + g.n2x - 1) / g.n2x));
-    const int64_t cc_per_l1 = (g.l2sx + l2_per_cc - 1) / l2_per_cc;
     const int64_t jb = b / g.n3x, je = (e - 1) / g.n3x;
     auto rg = [&](int64_t j) { return (j / g.n1y) * gpb + (j % g.n1y) / 32; };
     a.groups_per_band = gpb;
     a.rg_first = rg(jb);
     a.n_rg = rg(je) - a.rg_first + 1;
+    const int64_t most = a.n_rg * g.N2x / (2 * 24 * (int64_t)num_sms);
+    const int64_t l2_per_cc = std::max<int64_t>(1, std::min({(int64_t)g.l2sx, (2048 + g.n2x - 1) / g.n2x, most}));
+    const int64_t cc_per_l1 = (g.l2sx + l2_per_cc - 1) / l2_per_cc;
     a.l2_per_cc = l2_per_cc;
     a.cc_per_l1 = cc_per_l1;
     a.n_cc = g.N1x * cc_per_l1;
@@ -1299,7 +1305,7 @@ ml_status batch_create_impl(const ml_field_desc *descs, int32_t n, int32_t tpm, 
         for (size_t q = 0; q < m; ++q) {
             ml_field *f = b->fields[gr.maps[q]];
             args[q] = make_args(f);
-            set_tasks(args[q], f->g, 0, f->g.n3x * f->g.n3y);
+            set_tasks(args[q], f->g, 0, f->g.n3x * f->g.n3y, f->num_sms);
             gr.near_cap = std::max(gr.near_cap, args[q].near_cap);
             base[q + 1] = base[q] + args[q].n_tasks;
         }
@@ -1541,7 +1547,7 @@ ml_status ml_shoot_rays(ml_field *f, uint64_t ray_begin, uint64_t ray_end, void 
         a.ray_begin = (int64_t)b;
         a.ray_end = (int64_t)e;
         if (g.precision == ML_PREC_MIXED) {
-            set_tasks(a, g, (int64_t)b, (int64_t)e);
+            set_tasks(a, g, (int64_t)b, (int64_t)e, f->num_sms);
             ML_CK(cudaMemsetAsync(f->d_work, 0, sizeof(unsigned long long), s));
         }
         ML_CK(launch_shoot(a, f->num_sms, s));
@@ -1749,7 +1755,7 @@ ml_status ml_cic_backward_ex(ml_field *f, const float *dL_dM, double *grad_lens,
                                         grad_params, scale, f->num_sms, s));
         return ML_OK;
     }
-    set_tasks(a, g, 0, g.n3x * g.n3y);
+    set_tasks(a, g, 0, g.n3x * g.n3y, f->num_sms);
     const size_t n_mom = (size_t)(g.N2x * g.N2y) * (size_t)(g.p + 1);
     double *gs = nullptr;
     double2 *mom = nullptr;
