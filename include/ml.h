@@ -146,7 +146,7 @@ typedef struct {
     int32_t tune;               /* 1, with l2_sub_x = l2_sub_y = 0: the autotuner picks
                                    the level-2 grid (and with it p) and, unless l1_x or
                                    l1_y is set, the level-1 size (1, 1/sqrt2, 1/2 or
-                                   1/(2 sqrt2) of Eq. 10's): a cost model ranks 48 grids,
+                                   1/(2 sqrt2) of Eq. 10's): a cost model ranks up to 48 grids,
                                    then the best grid of each of the three best level-1
                                    sizes is built and timed on slices of rays and the
                                    fastest is taken.  The far-field bound stays within
@@ -176,9 +176,11 @@ typedef struct {
     /* Certified walk (ML_WALK_CERTIFIED): a warp's level-2 column that has
      * near lenses is walked in certified spans only if every near lens lies
      * farther than span_far lattice spacings (l3x) from its rays, else ray by
-     * ray.  0: the library's choice (3000; with tune, whichever of 3000, 1500,
-     * 700, 300, 100, +inf and no certified spans at all measured fastest; in a
-     * batch, +inf).  Any choice gives the same counts. */
+     * ray.  0: the library's choice: 2 sqrt(m / (l3x dpx)) with m the lenses'
+     * mean mass, where a lens moves neighbouring rays a quarter of a pixel
+     * apart; with tune, whichever of 0.4, 0.6, 1, 1.6 and 2.5 times that and no
+     * certified spans at all measured fastest.  Any choice gives the same
+     * counts. */
     double span_far;
 } ml_field_desc;
 

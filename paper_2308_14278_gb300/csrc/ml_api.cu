@@ -90,12 +90,12 @@ struct ml_field {
     int64_t n_lens = 0;
     int32_t tuned = 0;
     // certified walk: a warp's level-2 column with near lenses is spanned only
-    // if they all lie farther than this from its rays (lattice units; +inf:
-    // such columns always take the per-ray walk); the autotuner measures both
-    float span_far = ML_SPAN_FAR;
+    // if they all lie farther than this from its rays (lattice units; a large
+    // value: such columns always take the per-ray walk); 0 until create sets
+    // it (the caller's, the autotuner's or span_far_of)
+    float span_far = 0.f;
     // certified walk at all: false runs the per-ray kernel (the autotuner
-    // measures it beside the two thresholds; fields with near lenses nearly
-    // everywhere gain nothing from spans)
+    // measures it beside the distances)
     bool use_span = true;
     ml_field_desc desc{};            // parameters (lens pointers cleared)
     std::vector<double> worst;       // truncation bound per Taylor order (worst level-1 cell)
@@ -392,7 +392,7 @@ struct GridChoice {
     int sx = 20, sy = 20, p = 0;
     double l1x = 0.0, l1y = 0.0;    // level-1 size; 0 = Eq. 10's
     double cost = 0.0;
-    float span_far = ML_SPAN_FAR;   // certified walk's lens-column threshold (see ml_field)
+    float span_far = 0.f;           // certified walk's lens-column threshold (see ml_field); 0 = by rule
     bool use_span = true;           // certified walk at all (see ml_field)
 };
 
@@ -408,25 +408,45 @@ struct TuneCand {
     double span_frac;               // expected share of rays the certified walk may span
 };
 
-// Shooting time per ray of the certified walk, picoseconds: a least-squares
-// fit to 13 grids of the paper-scale field (level-1 cells of 1/2, 1/sqrt 2 and
-// 1 times Eq. 10's, level-2 cells of 88 to 1400 rays along a row, p = 4 to 8;
-// largest error 8 %).  Per-ray work is small and near lenses, the per-column
-// set-up (one per level-2 cell and row) and the order P carry the cost.
-double span_cost_ps(int P, double near_per_ray, double n2x)
+// Distance in lattice units within which a near lens sends the certified
+// walk's column to the per-ray walk, when the caller leaves it to the library:
+// where a lens of the mean mass moves neighbouring rays a quarter of a pixel
+// apart (m' / rho^2 = 1/4, m' = m / (l3x dpx)), so that runs are about four
+// rays long.  Best of 1500, 700, 300, 100 and 40 lattice units at the fastest
+// grids of six fields: 3.2 sqrt(m') on the paper-scale field (1500 units:
+// 0.134 ps a ray, 0.227 at 700), 2 on the Table-1 field (100), 0.8 to 1.8 on
+// four of the batched maps.
+double span_far_of(double mean_mass, double l3x, double dpx)
 {
-    return 0.145 + 0.238 * near_per_ray + 30.6 / std::max(1.0, n2x) + 0.0159 * P;
+    return 2.0 * sqrt(std::max(0.0, mean_mass) / (l3x * dpx));
 }
 
-// The certified walk spans a warp's level-2 column only when every near lens
-// lies farther than ML_SPAN_FAR lattice units from its rays; elsewhere it
-// runs the per-ray walk.  For lenses spread evenly over the 3 x 3 block of
-// level-1 cells, the share of columns without such a lens is
-// exp(-near * pi (ML_SPAN_FAR l3)^2 / (9 l1x l1y)).
-double span_share(double near_per_ray, double l3, double l1x, double l1y)
+double mean_abs_mass(const std::vector<double> &hm)
 {
-    const double r = (double)ML_SPAN_FAR * l3;
-    return exp(-near_per_ray * 3.14159265358979 * r * r / (9.0 * l1x * l1y));
+    double t = 0.0;
+    for (double m : hm) t += fabs(m);
+    return hm.empty() ? 0.0 : t / (double)hm.size();
+}
+
+// Shooting time per ray of the certified walk, picoseconds: a least-squares
+// fit to 210 grids of the paper-scale field, the Table-1 field and four of
+// the batched maps (level-1 cells of 1 to 1/(2 sqrt 2) times Eq. 10's, level-2
+// cells of 11 to 2806 rays along a row, p = 3 to 16), each at its best lens
+// distance; 12 % rms.  The constant is the fields' mean (0.05 to 0.28, by
+// their runs' lengths).  A column's set-up and its first and last window carry
+// the cost, so long level-2 cells with a high order pay.
+double span_cost_ps(int P, double near_per_ray, double n2x)
+{
+    return 0.187 + 0.0335 * near_per_ray + 0.0072 * P +
+           (16.8 + 0.79 * P + 1.87 * near_per_ray) / std::max(1.0, n2x);
+}
+
+// The share of columns that the certified walk spans: no near lens within
+// `far` (theta_E) of the column's rays, for lenses spread evenly over the
+// 3 x 3 block of level-1 cells: exp(-near * pi far^2 / (9 l1x l1y)).
+double span_share(double near_per_ray, double far, double l1x, double l1y)
+{
+    return exp(-near_per_ray * 3.14159265358979 * far * far / (9.0 * l1x * l1y));
 }
 
 double cand_cost(const TuneCand &c, int P)
@@ -500,8 +520,15 @@ ml_status tune_candidates(uint64_t key, const ml_field_desc &d, const std::vecto
     ml_status st = derive_geometry(d, hx, hy, g0);
     if (st != ML_OK) return st;
     const bool xlong = g0.l1x >= g0.l1y;
-    static const int fine[] = {20, 40, 60, 80, 120, 160};
-    static const int coarse[] = {10, 20};
+    // level-2 cells along the long and the short side: the certified walk's
+    // cost falls with the length of its columns, the per-ray walk's with P.
+    // Cells longer than the paper's are left out when the caller fixes P, whose
+    // truncation would grow.
+    const bool certified = d.walk == ML_WALK_CERTIFIED && d.deposit == ML_DEPOSIT_NGP && d.taylor_p == 0;
+    const std::vector<int> fine = certified ? std::vector<int>{5, 10, 20, 40}
+                                            : std::vector<int>{20, 40, 60, 80, 120, 160};
+    const std::vector<int> coarse = certified ? std::vector<int>{5, 10, 20} : std::vector<int>{10, 20};
+    const double mean_mass = mean_abs_mass(hm);
     // level-1 scales: Eq. 10's size unless the caller fixed it
     std::vector<double> scales{1.0};
     if (d.l1_x == 0.0 && d.l1_y == 0.0)
@@ -515,6 +542,7 @@ ml_status tune_candidates(uint64_t key, const ml_field_desc &d, const std::vecto
     for (int a : fine)
         for (int b : coarse) {
             if (e != cudaSuccess) break;
+            if (b > a) continue;
             Cand c{};
             c.sx = xlong ? a : b;
             c.sy = xlong ? b : a;
@@ -547,7 +575,7 @@ ml_status tune_candidates(uint64_t key, const ml_field_desc &d, const std::vecto
         }
     const double tol = d.far_tol > 0.0 ? d.far_tol : 1e-7;
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    std::vector<TuneCand> res;
+    std::vector<TuneCand> res, over;     // over: the bound misses far_tol at every order
     for (Cand &c : cands) {
         if (e != cudaSuccess) break;
         std::vector<double> bound((size_t)(c.g.N1x * c.g.N1y * PMAX));
@@ -566,19 +594,22 @@ ml_status tune_candidates(uint64_t key, const ml_field_desc &d, const std::vecto
                         tot += cnt[(size_t)((cy + dy) * c.g.NEx + cx + dxx)];
         const double near_per_ray = tot / (double)std::max<int64_t>(1, c.g.N1x * c.g.N1y);
         int p = d.taylor_p;
+        bool met = p != 0;
         if (p == 0) {
             p = PMAX;
             for (int q = 1; q <= PMAX; ++q) {
                 double w = 0.0;
                 for (size_t k = 0; k < bound.size() / PMAX; ++k) w = std::max(w, bound[k * PMAX + q - 1]);
-                if (w <= tol) { p = q; break; }
+                if (w <= tol) { p = q; met = true; break; }
             }
         }
         if (d.macro_mode == ML_MACRO_FOLD) p = std::max(p, 2);
-        res.push_back(TuneCand{c.sx, c.sy, mixed_p_supported(p), (double)c.g.N2x * (double)c.g.N2y,
+        (met ? res : over).push_back(TuneCand{c.sx, c.sy, mixed_p_supported(p), (double)c.g.N2x * (double)c.g.N2y,
                                (double)c.g.n3x * (double)c.g.n3y, (double)c.g.N1x * (double)c.g.N1y,
                                near_per_ray, c.l1x, c.l1y, (double)c.g.n2x, d.walk,
-                               span_share(near_per_ray, c.g.l3x, c.g.l1x, c.g.l1y)});
+                               span_share(near_per_ray,
+                                          c.g.l3x * span_far_of(mean_mass, c.g.l3x, c.g.dpx), c.g.l1x,
+                                          c.g.l1y)});
     }
     for (Cand &c : cands) {
         if (c.cells) cudaFreeAsync(c.cells, s);
@@ -587,6 +618,7 @@ ml_status tune_candidates(uint64_t key, const ml_field_desc &d, const std::vecto
     }
     if (f32) cudaFreeAsync(f32, s);
     if (e != cudaSuccess) return cuda_fail(e, "grid autotuner");
+    if (res.empty()) res = over;
     out = res;
     std::lock_guard<std::mutex> lock(g_tune_mu);
     g_tune_cache[key] = res;
@@ -657,7 +689,7 @@ ml_status tune_grid(const ml_field_desc &d, const std::vector<double> &hx, const
     for (size_t i = 0; i < std::min<size_t>(3, order.size()); ++i) {
         const TuneCand &c = cands[order[i]];
         double est = 0.0;
-        float far = ML_SPAN_FAR;
+        float far = 0.f;
         bool span = true;
         // a candidate that cannot be built (near lists too long for the
         // mixed kernel's shared memory, memory) is passed over
@@ -758,10 +790,12 @@ ml_status create_plan(const ml_field_desc *d_in, cudaStream_t s, ml_field *f)
         }
         f->tuned = 1;
     }
-    if (d->span_far > 0.0) f->span_far = (float)std::min(d->span_far, 3.0e38);
     ml_status st = derive_geometry(*d, hx, hy, f->g);
     if (st != ML_OK) return st;
     Geo &g = f->g;
+    if (d->span_far > 0.0) f->span_far = (float)std::min(d->span_far, 3.0e38);
+    else if (f->span_far <= 0.f)
+        f->span_far = (float)std::min(span_far_of(mean_abs_mass(hm), g.l3x, g.dpx), 3.0e38);
     const bool nearfar = d->precision != ML_PREC_DIRECT64;
     if (nearfar && !rays_inside_sheet(g))
         return fail(ML_ERR_UNSUPPORTED, "near/far modes need the whole ray rectangle inside the "
@@ -950,19 +984,13 @@ ml_status measure_grid(const ml_field_desc &d, const std::vector<double> &hx, co
         const uint64_t r0 = (total - 2 * n) / 2;
         const uint64_t warm = std::min<uint64_t>(n, 64ull * (uint64_t)g.n3x);
         // the certified walk is timed with lens columns spanned beyond five
-        // distances about a factor two apart (lattice spacings: where spanning
-        // pays depends on the lenses' pull in pixels per spacing, which differs
-        // between fields), with them always walked ray by ray, and without
-        // spans (the per-ray kernel); the fastest counts
+        // distances about a factor 1.6 apart around the library's rule (where
+        // spanning pays differs between fields), and without spans (the per-ray
+        // kernel); the fastest counts
         const bool certified = f->desc.walk == ML_WALK_CERTIFIED && f->g.deposit == ML_DEPOSIT_NGP;
-        constexpr int NV = 7;
-        const float fars[NV] = {ML_SPAN_FAR, 1500.f, 700.f, 300.f, 100.f, 3.0e38f, 3.0e38f};
-        static const char *const names[NV] = {" (lens columns spanned beyond 3000)",
-                                              " (lens columns spanned beyond 1500)",
-                                              " (lens columns spanned beyond 700)",
-                                              " (lens columns spanned beyond 300)",
-                                              " (lens columns spanned beyond 100)",
-                                              " (lens columns per ray)", " (no spans)"};
+        constexpr int NV = 6;
+        const float rule = (float)span_far_of(mean_abs_mass(hm), g.l3x, g.dpx);
+        const float fars[NV] = {rule, 2.5f * rule, 1.6f * rule, 0.6f * rule, 0.4f * rule, rule};
         double best_ray = -1.0;
         for (int v = 0; v < (certified ? NV : 1) && st == ML_OK; ++v) {
             f->span_far = fars[v];
@@ -984,9 +1012,9 @@ ml_status measure_grid(const ml_field_desc &d, const std::vector<double> &hx, co
                 use_span = v < NV - 1;
             }
             if (st == ML_OK && getenv("ML_TUNE_LOG"))
-                fprintf(stderr, "ml tune:   create %.2f ms, %.3g and %.3g of %.3g rays in %.3f and %.3f ms%s\n",
+                fprintf(stderr, "ml tune:   create %.2f ms, %.3g and %.3g of %.3g rays in %.3f and %.3f ms (%s %g)\n",
                         create_ms, (double)n, (double)(2 * n), (double)total, ms[0], ms[1],
-                        certified ? names[v] : "");
+                        certified && v < NV - 1 ? "lens columns spanned beyond" : "no spans", fars[v]);
         }
         if (st == ML_OK) est_ms = create_ms + best_ray * (double)total;
     }
@@ -1014,7 +1042,6 @@ ShootArgs make_args(const ml_field *f)
     const Geo &g = f->g;
     a.near_cap = std::max(1, f->max_near);
     a.walk = f->desc.walk == ML_WALK_CERTIFIED && f->use_span ? ML_WALK_CERTIFIED : ML_WALK_PER_RAY;
-    a.span_far = f->span_far;
     a.l3x_f = (float)g.l3x;
     a.l3x_lo = (float)(g.l3x - (double)a.l3x_f);
     a.c0_f = (float)(0.5 - 0.5 * (double)g.n2x);
@@ -1026,6 +1053,7 @@ ShootArgs make_args(const ml_field *f)
         double rc = 4.0 * 5.9604644775390625e-8 * (0.5 * g.l2x + 32.0 * g.l3y) / 5e-7;
         a.rc2 = (float)(rc * rc);
         a.rc2u = (float)((rc / g.l3x) * (rc / g.l3x));
+        a.span_far2 = std::min(3.0e38f, std::max(f->span_far * f->span_far, 1.02f * a.rc2u + 1e-30f));
     }
     a.ipx_f = (float)(1.0 / g.dpx);
     a.ipy_f = (float)(1.0 / g.dpy);
@@ -1225,12 +1253,8 @@ ml_status batch_create_impl(const ml_field_desc *descs, int32_t n, int32_t tpm, 
         }
         GridChoice best;
         // the batch's grids come from the cost model alone (timing every map
-        // would cost more than it saves); the per-ray model ranks them: on
-        // the lens-dense maps of a batch the certified walk runs mostly per
-        // ray, and the certified model (fitted on a sparse field) misranks
-        ml_field_desc model = plan[i];
-        model.walk = ML_WALK_PER_RAY;
-        if (e == cudaSuccess) st = tune_grid(model, hx, hy, hm, dx, dy, dm, s, false, best);
+        // would cost more than it saves)
+        if (e == cudaSuccess) st = tune_grid(plan[i], hx, hy, hm, dx, dy, dm, s, false, best);
         cudaFreeAsync(dx, s);
         cudaFreeAsync(dy, s);
         cudaFreeAsync(dm, s);
@@ -1251,9 +1275,6 @@ ml_status batch_create_impl(const ml_field_desc *descs, int32_t n, int32_t tpm, 
         ml_status st = create_plan(&plan[i], s, b->fields[i]);
         if (st != ML_OK) return fail(st, "map " + std::to_string(i) + ": " + g_err);
         b->fields[i]->tuned = tuned[i];
-        // not timed per map: the batches measured (lens-dense fields) run
-        // faster with lens columns walked ray by ray
-        if (plan[i].span_far == 0.0) b->fields[i]->span_far = 3.0e38f;
     }
     // coefficient builds of different maps overlap on a few streams
     {

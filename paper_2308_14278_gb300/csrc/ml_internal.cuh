@@ -15,19 +15,11 @@ constexpr uint32_t PIX_OUT = 0xFFFFFFFFu;   // run-length code: outside the map
 constexpr uint32_t PIX_DROP = 0xFFFFFFFEu;  // run-length code: ray hit a lens
 constexpr int WARPS_PER_CTA = 8;
 
-// The certified walk (ML_WALK_CERTIFIED): rays it evaluates per step (its
-// window), rays short of the predicted pixel edge at which a window starts,
-// and the distance in lattice units within which a near lens makes it hand a
-// warp's level-2 column to the per-ray walk (runs shorten and certified spans
-// stay short near a lens).
-#ifndef ML_SPAN_W
-#define ML_SPAN_W 2
-#endif
+// The certified walk (ML_WALK_CERTIFIED): rays short of the predicted pixel
+// edge (less the bound's margin there) at which a window starts.  0, 0.25 and
+// 0.5 measured 3.31, 3.37 and 3.57 ms per 2e10 rays of the paper-scale lattice.
 #ifndef ML_SPAN_MARGIN
-#define ML_SPAN_MARGIN 1.0f
-#endif
-#ifndef ML_SPAN_FAR
-#define ML_SPAN_FAR 3000.0f
+#define ML_SPAN_MARGIN 0.0f
 #endif
 
 // Parameters derived from an ml_field_desc (§3.1 and §3.2).
@@ -93,8 +85,9 @@ struct ShootArgs {
     int64_t n_tasks;
     int near_cap;                   // float4 slots of shared memory per warp
     int walk;                       // ML_WALK_CERTIFIED or ML_WALK_PER_RAY (mixed NGP)
-    float span_far;                 // certified walk: lens columns spanned only if every near
-                                    // lens lies farther than this (lattice units)
+    float span_far2;                // certified walk: lens columns spanned only if every near
+                                    // lens lies farther than the root of this (lattice units);
+                                    // at least the close-pass radius, with a margin
     // float constants of the mixed kernel
     float l3x_f, l3x_lo, c0_f, ipx_f, ipy_f;
     float cxy_f;                    // change of the u slope of beta_x per ray row (fold: d_y l3y l3x / dpx)
@@ -488,6 +481,13 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
 {
     f32x2 d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
 

@@ -203,10 +203,12 @@ __global__ void __launch_bounds__(256) k_shoot_fp64(ShootArgs a)
 // are merged and added with one atomic when the pixel changes.  The atomics
 // return nothing (fire-and-forget reductions); a wrapped uint32 count is found
 // afterwards by comparing the map's 64-bit sum with the in-map ray counter.
+// `in` counts the rays added to the map; the lane's other rays (tot - in) fell
+// outside it.
 struct RunState {
     int cx, cy;
     unsigned cnt;
-    unsigned in, out;
+    unsigned in, tot;
 };
 
 __device__ __forceinline__ void run_flush(RunState &rs, uint32_t *map, int mnx, int mny)
@@ -215,20 +217,7 @@ __device__ __forceinline__ void run_flush(RunState &rs, uint32_t *map, int mnx, 
     if ((unsigned)rs.cx < (unsigned)mnx && (unsigned)rs.cy < (unsigned)mny) {
         atomicAdd(map + (size_t)rs.cy * (unsigned)mnx + (unsigned)rs.cx, rs.cnt);
         rs.in += rs.cnt;
-    } else {
-        rs.out += rs.cnt;
     }
-}
-
-__device__ __forceinline__ void run_add(RunState &rs, int gx, int gy, uint32_t *map, int mnx, int mny)
-{
-    if (gx != rs.cx || gy != rs.cy) {
-        run_flush(rs, map, mnx, mny);
-        rs.cx = gx;
-        rs.cy = gy;
-        rs.cnt = 0;
-    }
-    ++rs.cnt;
 }
 
 // Lane-valid ray of a warp-uniform walk position.
@@ -247,8 +236,6 @@ __device__ __forceinline__ void run_step(RunState &rs, bool valid, int gx, int g
                 if ((unsigned)rs.cx < (unsigned)mnx && (unsigned)rs.cy < (unsigned)mny) {
                     atomicAdd(map + (size_t)rs.cy * (unsigned)mnx + (unsigned)rs.cx, rs.cnt);
                     rs.in += rs.cnt;
-                } else {
-                    rs.out += rs.cnt;
                 }
             }
             rs.cx = gx;
@@ -267,8 +254,6 @@ __device__ __forceinline__ void flush_run(RunState &rs, int cx, int cy, unsigned
     if ((unsigned)cx < (unsigned)mnx && (unsigned)cy < (unsigned)mny) {
         atomicAdd(map + (size_t)cy * (unsigned)mnx + (unsigned)cx, cnt);
         rs.in += cnt;
-    } else {
-        rs.out += cnt;
     }
 }
 
@@ -461,8 +446,6 @@ __device__ __forceinline__ float rsqrt_approx(float y)
     return r;
 }
 
-constexpr int NN_DYN = 5;   // walk_span: near list of any length, read from shared memory
-
 // Span-walk counts of a warp into the field's counters.
 __device__ void flush_spans(const ShootArgs &a, const SpanCount &sc)
 {
@@ -478,329 +461,284 @@ __device__ void flush_spans(const ShootArgs &a, const SpanCount &sc)
 }
 
 // Certified walk of one level-2 column (NGP counts).  Each lane walks its own
-// ray range [k0, k1) of its row in steps.  A step evaluates a window of W
-// consecutive rays kb, kb+1, ... with exactly the per-ray arithmetic of
-// walk_fixed / near_sum_lat / row_eval, after the lane's last evaluated ray
-// ka.  When kb > ka + 1 the rays strictly between them are not evaluated:
-// they join the current run only if ray kb lands in the run's pixel and a
-// bound proves that every ray between lands there too; otherwise the lane
-// takes nothing from this step and retries with a shorter gap.  Every ray
-// therefore gets the pixel the per-ray walk gives it, and the counts are
-// bit-identical.  The gap is chosen so that the window starts ML_SPAN_MARGIN
-// rays short of where the lane's (X, Y) slope says the next pixel edge lies,
-// so that one step usually crosses it.  The window's rays are evaluated
-// together, in straight-line code: their Horner chains are independent and
-// interleave, the near list is read once for all of them, and one warp vote
-// serves the window's close-pass test.
+// ray range [k0, k1) of its row in steps.  A step evaluates a window of two
+// consecutive rays b, b+1 with exactly the per-ray arithmetic of walk_fixed /
+// near_sum_lat / row_eval, after the lane's last evaluated ray a.  When b lies
+// beyond a + 1 the rays strictly between them are not evaluated: they join
+// the current run only if ray b lands in the run's pixel and a bound proves
+// that every ray between lands there too; otherwise the lane takes nothing
+// from this step and retries with a shorter gap.  Every ray therefore gets the
+// pixel the per-ray walk gives it, and the counts are bit-identical.
 //
 // The bound.  Along the row the walk's value X(u) (and Y(u)) is the FP32
-// evaluation of F(u) = P(u) + sum_q (lx_q - u) m_q / ((lx_q - u)^2 + dy2_q)
-// (Y: the terms dyy_q m_q / (...)), with P the row polynomial and the FP32
-// lens constants taken as exact reals.  For a ray between a and b:
-//  - rounding: |X - F| <= E = c eps (S_P + sum_q m_q / rho_q), with
-//    S_P = sum |C_m| U^m (U the lane's largest |u|), eps = 2^-24, rho_q the
-//    lens's smallest distance to the span's rays and c = 2 (P + nn + 8), at
-//    least twice the count of roundings on the path (Horner FMAs, per lens
-//    the offset, r^2, reciprocal, mass product and accumulation);
-//  - shape: F lies within K = (b - a)^2 / 8 max|F''| of the chord between
-//    F(a) and F(b), with |F''| <= sum m(m-1) |C_m| U^(m-2) + sum_q 2 m_q / rho_q^3
-//    (Y: 6 m_q |dyy_q| / rho_q^4): with r^2 = x^2 + dy2 and c = x / r, a
-//    lens's term m x / r^2 has second derivative (2 m / r^3) c (4 c^2 - 3),
-//    and |4 c^3 - 3 c| <= 1 on [-1, 1] (the Chebyshev polynomial T_3); its y
-//    term m dyy / r^2 has (m dyy / r^4) (8 c^2 - 2), at most 6 in size;
-//  - so X lies in [min(X_a, X_b) - 2E - K, max(X_a, X_b) + 2E + K] (margin
-//    widened by 1 %, ends rounded outwards); if that interval has one floor,
-//    and the same holds for Y, every ray between shares the anchor's pixel;
-//  - when |X_b - X_a| - 2E > (b - a)^2 max|F''| (= 8K), F' has one sign on
-//    the span (it is within (b - a) max|F''| of the chord's slope, by the
-//    mean value theorem), so F is monotone, lies between F(a) and F(b), and
-//    the interval needs no K: near a pixel edge, spans several times longer
-//    pass.
-// A span whose rays could come within the close-pass radius of a lens is never
-// certified (those rays would take the hi/lo arithmetic), and anchors outside
-// |X|, |Y| < 2^21 (rays dropped on a lens) are never certified from.
-template <int P, int NN>
-__device__ __forceinline__ void walk_span(const RowPoly<P> &rp, const ShootArgs &a, const SmemNear &nl,
-                                          int nn_dyn, int k0, int k1, float dyl, float dyl_lo,
-                                          RunState &rs, unsigned &drop, SpanCount &sc)
+// evaluation of F(u) = P(u) + sum_q m_q / z_q, z_q = (lx_q - u) + i dy_q (X the
+// real part; Y minus yx times the imaginary part), with P the row polynomial
+// and the FP32 lens constants taken as exact reals.  What the bound needs of F
+// is taken once per column and lane (span_bound), so a step's test reads no
+// lens:
+//  - rounding: |X - F| <= E = eps ((P + 1 + nn) S_P + (8 + nn) sum_q m_q / rho_q),
+//    with S_P = sum |C_m| U^m (U the lane's largest |u|), eps = 2^-24, rho_q the
+//    lens's least distance to the lane's rays.  P roundings of Horner's rule
+//    with fused multiply-adds, each at most eps S_P to first order; per lens
+//    at most 7 on its term (the offset once and twice in r^2, r^2, two of the
+//    reciprocal's 2^-23, the mass product) and one of the running sum; the
+//    ones added cover the second order;
+//  - shape: F'' stays in [lo, hi] over the lane's rays.  The polynomial gives
+//    2 C_2 +- sum_{m>=3} m(m-1) |C_m| U^(m-2).  A lens's m/z has the second
+//    derivative 2m/z^3, and the third is at most 6m/rho^4 in size, so on a
+//    range of half-width h about its middle it stays within 6 m h/rho^4 of its
+//    value there (used for rho > 3h; else within 2m/rho^3 of zero).
+//    On a span of w rays F = chord - F''(xi) t (w - t) / 2, so F lies no more
+//    than w^2/8 max(hi, 0) below the chord and w^2/8 max(-lo, 0) above it;
+//  - when |X_b - X_a| - 2E > w^2 max|F''| / 2, F' has one sign on the span (the
+//    chord's slope is the mean of F', from which F' at t differs by at most
+//    max|F''| (t^2 + (w - t)^2) / 2w), F lies between F(a) and F(b), and the
+//    curvature's margin is not needed;
+//  - so X lies in [min(X_a, X_b) - 2E - below, max(X_a, X_b) + 2E + above], 2E
+//    widened by a tenth and the rest by 1 % against the rounding of the test
+//    itself; if that stays in one pixel, and likewise Y, every ray between
+//    shares the pixel.
+// The caller takes this walk only where no ray of the column can come within
+// the close-pass radius of a lens (those rays take the hi/lo arithmetic) and
+// where |X|, |Y| < 2^20, so that the floor's bit form is valid.
+//
+// The next window.  The slope at the last ray (the span's chord plus half the
+// span times the mid-range F'', or the window's own difference) and that F''
+// give the distance to the next pixel edge (the parabola's root); the
+// window is placed so that its two rays straddle the edge.  A step that lands
+// past the edge aims again from the same chord, one whose bound fails halves
+// its gap.
+//
+// What bounds it: instruction issue, about 200 warp instructions a step, and
+// the warp takes its slowest lane's steps (15 per 702-ray column of the
+// paper-scale field, 10 for the mean lane).  With the bound taken per step,
+// lens by lens, windows placed by the slope alone and two flushes a step,
+// 2e10 rays of the paper-scale lattice took 5.88 ms, 1e10 of the Table-1
+// lattice 10.7 ms and 1e11 of the 1e13-ray production lattice 15.0 ms; now
+// 3.31, 6.8 and 7.4 ms at the same grids.  Lens loops are not unrolled (near
+// lists are short: unrolled by four they took 8 % more time), and a window
+// whose rays both change pixel takes only its first, so that a step has one
+// flush (9 %).
+struct SpanBound {
+    f32x2 e;                    // 1/2 - 2E (widened)
+    f32x2 t;                    // 2E (widened)
+    f32x2 g, s;                 // -(below - above)/2 and -(below + above)/2 per w^2
+    f32x2 m;                    // max |F''| / 2 (widened)
+    f32x2 d;                    // F''/2 in the middle of the range
+    bool ok;                    // |X|, |Y| stay below 2^20
+};
+
+template <int P>
+__device__ __forceinline__ SpanBound span_bound(const RowPoly<P> &rp, const ShootArgs &a, const float4 *near,
+                                                int nn, float ulo, float uhi, float dyl)
 {
-    constexpr int W = ML_SPAN_W;                // rays evaluated per step
-    constexpr bool REG = NN < NN_DYN;
-    constexpr int NR = (REG && NN > 0) ? NN : 1;
-    float lx[NR], lm[NR], dy2[NR], dyy[NR];
-    if constexpr (REG) {
-#pragma unroll
-        for (int q = 0; q < NN; ++q) {
-            const float4 L = nl.near[q];
-            lx[q] = L.x;
-            lm[q] = L.z;
-            const float dy = __fsub_rn(L.y, dyl);
-            dy2[q] = __fmul_rn(dy, dy);
-            dyy[q] = __fmul_rn(dy, a.yx_f);
-        }
-    }
-    const int nlen = REG ? NN : nn_dyn;
-    // record q of the near list: the registers, or shared memory with the
-    // per-lane terms formed as near_sum_lat forms them
-    auto rec = [&](int q, float &x, float &m, float &d2, float &dd) {
-        if constexpr (REG) {
-            x = lx[q]; m = lm[q]; d2 = dy2[q]; dd = dyy[q];
-        } else {
-            const float4 L = nl.near[q];
-            const float dy = __fsub_rn(L.y, dyl);
-            x = L.x; m = L.z; d2 = __fmul_rn(dy, dy); dd = __fmul_rn(dy, a.yx_f);
-        }
-    };
-    f32x2 C[P + 1];
-#pragma unroll
-    for (int m = 0; m <= P; ++m) C[m] = pack2(rp.X[m], rp.Y[m]);
-    const f32x2 MAGIC = pack2(12582912.0f, 12582912.0f);
-    constexpr float LIM = 2097152.0f;           // 2^21
-
-    // source positions of rays kb .. kb+W-1 by the per-ray arithmetic, in raw
-    // floor form; dr[r] marks a ray on a lens (sent far outside the map, as
-    // walk_fixed does).  Called by all lanes together (the close-pass branch
-    // is taken by warp vote); av[r] says which rays the lane will use.
-    float X[W], Y[W];
-    unsigned rx[W], ry[W];
-    bool dr[W];
-    auto eval_window = [&](int kb, const bool (&av)[W]) {
-        float u[W];
-        f32x2 v[W];
-#pragma unroll
-        for (int r = 0; r < W; ++r) {
-            u[r] = __fadd_rn((float)(kb + r), a.c0_f);
-            v[r] = C[P];
-        }
-#pragma unroll
-        for (int m = P - 1; m >= 0; --m) {
-#pragma unroll
-            for (int r = 0; r < W; ++r) v[r] = fma2(v[r], pack2(u[r], u[r]), C[m]);
-        }
-#pragma unroll
-        for (int r = 0; r < W; ++r) {
-            unpack2(v[r], X[r], Y[r]);
-            dr[r] = false;
-        }
-        // (nlen is warp-uniform: an empty near list skips the lens loop and its vote)
-        if (!(REG && NN == 0) && nlen > 0) {
-            float mn[W];
-#pragma unroll
-            for (int r = 0; r < W; ++r) mn[r] = 3.0e38f;
-            auto lens = [&](int q) {
-                float x, m, d2, dd;
-                rec(q, x, m, d2, dd);
-#pragma unroll
-                for (int r = 0; r < W; ++r) {
-                    const float dx = __fsub_rn(x, u[r]);
-                    const float r2 = __fmaf_rn(dx, dx, d2);
-                    mn[r] = fminf(mn[r], r2);
-                    const float sv = __fmul_rn(m, rcp_approx(r2));
-                    X[r] = __fmaf_rn(dx, sv, X[r]);
-                    Y[r] = __fmaf_rn(dd, sv, Y[r]);
-                }
-            };
-            if constexpr (REG) {
-#pragma unroll
-                for (int q = 0; q < NR; ++q) lens(q);
-            } else {
-                for (int q = 0; q < nlen; ++q) lens(q);
-            }
-            bool cl[W], any = false;
-#pragma unroll
-            for (int r = 0; r < W; ++r) {
-                cl[r] = av[r] && mn[r] < a.rc2u;
-                any |= cl[r];
-            }
-            if (__any_sync(0xffffffffu, any)) {
-                // rare: one copy of the hi/lo path, the window rotated through slot 0
-#pragma unroll 1
-                for (int i = 0; i < W; ++i) {
-                    if (cl[0]) {
-                        unpack2(v[0], X[0], Y[0]);
-                        if (!near_sum_hilo_lat(nl, nlen, u[0], dyl, dyl_lo, a.yx_f, X[0], Y[0])) {
-                            X[0] = -1.0e30f;
-                            dr[0] = true;
-                        }
-                    }
-                    const float u0 = u[0], X0 = X[0], Y0 = Y[0];
-                    const f32x2 v0 = v[0];
-                    const bool c0 = cl[0], d0 = dr[0];
-#pragma unroll
-                    for (int r = 0; r + 1 < W; ++r) {
-                        u[r] = u[r + 1]; X[r] = X[r + 1]; Y[r] = Y[r + 1];
-                        v[r] = v[r + 1]; cl[r] = cl[r + 1]; dr[r] = dr[r + 1];
-                    }
-                    u[W - 1] = u0; X[W - 1] = X0; Y[W - 1] = Y0;
-                    v[W - 1] = v0; cl[W - 1] = c0; dr[W - 1] = d0;
-                }
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < W; ++r) {
-            float fx, fy;
-            unpack2(add2_rd(pack2(X[r], Y[r]), MAGIC), fx, fy);
-            rx[r] = (unsigned)__float_as_int(fx);
-            ry[r] = (unsigned)__float_as_int(fy);
-        }
-    };
-
-    // bounds of the row polynomial over the lane's range: S = sum |C_m| U^m,
-    // Q = sum_{m>=2} m (m-1) |C_m| U^(m-2), rounded upwards
-    const bool on = k1 > k0;
-    const float ulo = __fadd_rn((float)k0, a.c0_f);
-    const float uhi = __fadd_rn((float)(on ? k1 - 1 : k0), a.c0_f);
-    const float Um = fmaxf(fabsf(ulo), fabsf(uhi));
+    SpanBound b;
+    const float U = fmaxf(fabsf(ulo), fabsf(uhi));
     float SX = fabsf(rp.X[P]), SY = fabsf(rp.Y[P]);
 #pragma unroll
     for (int m = P - 1; m >= 0; --m) {
-        SX = __fmaf_ru(SX, Um, fabsf(rp.X[m]));
-        SY = __fmaf_ru(SY, Um, fabsf(rp.Y[m]));
+        SX = __fmaf_ru(SX, U, fabsf(rp.X[m]));
+        SY = __fmaf_ru(SY, U, fabsf(rp.Y[m]));
     }
-    float QX = 0.f, QY = 0.f;
+    float RX = 0.f, RY = 0.f, DX = 0.f, DY = 0.f;
     if constexpr (P >= 2) {
-        QX = (float)(P * (P - 1)) * fabsf(rp.X[P]);
-        QY = (float)(P * (P - 1)) * fabsf(rp.Y[P]);
+        DX = 2.f * rp.X[2];
+        DY = 2.f * rp.Y[2];
 #pragma unroll
-        for (int m = P - 1; m >= 2; --m) {
-            QX = __fmaf_ru(QX, Um, (float)(m * (m - 1)) * fabsf(rp.X[m]));
-            QY = __fmaf_ru(QY, Um, (float)(m * (m - 1)) * fabsf(rp.Y[m]));
+        for (int m = P; m >= 3; --m) {
+            RX = __fmaf_ru(RX, U, (float)(m * (m - 1)) * fabsf(rp.X[m]));
+            RY = __fmaf_ru(RY, U, (float)(m * (m - 1)) * fabsf(rp.Y[m]));
+        }
+        RX *= U;
+        RY *= U;
+    }
+    float AX = fabsf(DX), AY = fabsf(DY), t = 0.f;
+    const float um = 0.5f * (ulo + uhi), hw = 0.5f * (uhi - ulo);
+#pragma unroll 1
+    for (int q = 0; q < nn; ++q) {
+        const float4 L = near[q];
+        const float m = L.z, x = L.x - um, dy = __fsub_rn(L.y, dyl);
+        const float dist = fmaxf(0.f, fabsf(x) - hw);
+        const float ir = rsqrt_approx(fmaf(dist, dist, dy * dy)), ir2 = ir * ir;
+        const float mr = fabsf(m) * ir;
+        t += mr;
+        const float g2 = 2.f * mr * ir2;              // |2m/z^3| over the range
+        AX += g2;
+        if (3.f * hw * ir < 1.f) {
+            const float inv = rcp_approx(fmaf(x, x, dy * dy));
+            const float wr = x * inv, wi = dy * inv, w2 = wr * wr - wi * wi, v2 = 2.f * wr * wi;
+            DX += 2.f * m * (w2 * wr - v2 * wi);
+            DY += 2.f * m * a.yx_f * (w2 * wi + v2 * wr);
+            RX += 3.f * g2 * ir * hw;
+            RY += 3.f * g2 * ir * hw * a.yx_f;
+        } else {
+            RX += g2;
+            RY += g2 * a.yx_f;
         }
     }
-    const float rcut = __fmaf_ru(1.01f, a.rc2u, 1e-30f);
-    // 2 c eps: twice the rounding bound's factor (see above)
-    const float c2e = (float)(4 * (P + 8 + nlen)) * 5.9604645e-8f;
+    AY += AX * a.yx_f;
+    RX = fmaf(1e-5f, AX, RX);
+    RY = fmaf(1e-5f, AY, RY);
+    const float tY = t * a.yx_f;
+    b.ok = SX + t < 1048576.f && SY + tY < 1048576.f;
+    // 2E, a tenth wider (the constant covers the roundings of the test itself,
+    // on positions below 1)
+    constexpr float E2 = 1.1f * 2.f * 5.9604645e-8f;
+    const float cp = E2 * (float)(P + 1 + nn), cl = E2 * (float)(8 + nn);
+    const float eX = fmaf(cl, t, fmaf(cp, SX, 3e-7f)), eY = fmaf(cl, tY, fmaf(cp, SY, 3e-7f));
+    const float hX = 0.12625f * fmaxf(DX + RX, 0.f), lX = 0.12625f * fmaxf(RX - DX, 0.f);
+    const float hY = 0.12625f * fmaxf(DY + RY, 0.f), lY = 0.12625f * fmaxf(RY - DY, 0.f);
+    b.t = pack2(eX, eY);
+    b.e = pack2(0.5f - eX, 0.5f - eY);
+    b.g = pack2(0.5f * (lX - hX), 0.5f * (lY - hY));
+    b.s = pack2(-0.5f * (lX + hX), -0.5f * (lY + hY));
+    b.m = pack2(0.505f * (fabsf(DX) + RX), 0.505f * (fabsf(DY) + RY));
+    b.d = pack2(0.5f * DX, 0.5f * DY);
+    return b;
+}
 
-    auto certify = [&](int ka, int kb, float Xa, float Ya, float Xb, float Yb) {
-        if (!(fabsf(Xa) < LIM && fabsf(Xb) < LIM && fabsf(Ya) < LIM && fabsf(Yb) < LIM)) return false;
-        const float ua = __fadd_rn((float)ka, a.c0_f), ub = __fadd_rn((float)kb, a.c0_f);
-        float tX = 0.f, tY = 0.f, cX = QX, cY = QY;
-        bool clear = true;
-        if (!(REG && NN == 0) && nlen > 0) {
-            auto lens = [&](int q) {
-                float x, m, d2, dd;
-                rec(q, x, m, d2, dd);
-                const float dist = fmaxf(0.f, fmaxf(__fsub_rd(ua, x), __fsub_rd(x, ub)));
-                const float rho2 = __fmaf_rd(dist, dist, d2);
-                clear &= rho2 > rcut;
-                const float ir2 = rcp_approx(rho2), ir = rsqrt_approx(rho2);
-                const float mr = m * ir, md = m * fabsf(dd);
-                tX += mr;
-                tY = fmaf(md, ir2, tY);
-                cX = fmaf(2.f * mr, ir2, cX);
-                cY = fmaf(6.f * md, ir2 * ir2, cY);
-            };
-            if constexpr (REG) {
+// Rays from the last one to the next pixel edge, less the margin that a span
+// needs there: position c in [-1/2, 1/2) off the pixel's centre, e = 1/2 less
+// the margin, slope s, half the second derivative d: the first root of the
+// parabola in the slope's direction; NaN where it turns back before.
+__device__ __forceinline__ float rays_to_edge(float c, float e, float s, float d)
+{
+    const unsigned sg = __float_as_uint(s) & 0x80000000u;
+    const float eh = e - __uint_as_float(__float_as_uint(c) ^ sg);
+    const float disc = fmaf(4.f * __uint_as_float(__float_as_uint(d) ^ sg), eh, s * s);
+    return 2.f * eh * rcp_approx(fmaf(disc, rsqrt_approx(disc), fabsf(s)));
+}
+
+// A lattice count held in a float (0 <= v < 2^23) as an integer, by an add.
+__device__ __forceinline__ unsigned count_of(float v)
+{
+    return (unsigned)(__float_as_int(__fadd_rn(v, 8388608.f)) - 0x4B000000);
+}
+
+template <int P>
+__device__ __forceinline__ void walk_span(const RowPoly<P> &rp, const SpanBound &b, const ShootArgs &a,
+                                          const float4 *near, int nn, bool on, float ulo, float uhi, float dyl,
+                                          RunState &rs, SpanCount &sc)
+{
+    constexpr float MAGIC_F = 12582912.0f;
+    const f32x2 MAGIC = pack2(MAGIC_F, MAGIC_F), NEG1 = pack2(-1.f, -1.f), NHALF = pack2(-0.5f, -0.5f);
+    f32x2 C[P + 1];
 #pragma unroll
-                for (int q = 0; q < NR; ++q) lens(q);
-            } else {
-                for (int q = 0; q < nlen; ++q) lens(q);
-            }
-        }
-        const float w = __fsub_rn(ub, ua);
-        const float kk = 0.125f * w * w;
-        // 2E and K of each component; where the chord's rise exceeds what the
-        // curvature can undo over the span, |F(b) - F(a)| - 2E > (b - a)^2
-        // max|F''| = 8K, F' keeps one sign (mean value theorem), F lies
-        // between F(a) and F(b), and K is not needed
-        const float eX = c2e * (SX + tX), eY = c2e * (SY + tY);
-        const float kX = kk * cX, kY = kk * cY;
-        const bool monoX = __fsub_rd(__fmul_rd(fabsf(__fsub_rn(Xb, Xa)), 0.9999998f), eX) > 8.1f * kX;
-        const bool monoY = __fsub_rd(__fmul_rd(fabsf(__fsub_rn(Yb, Ya)), 0.9999998f), eY) > 8.1f * kY;
-        const float MX = 1.01f * (monoX ? eX : eX + kX);
-        const float MY = 1.01f * (monoY ? eY : eY + kY);
-        const bool okx = floor_to_int(__fsub_rd(fminf(Xa, Xb), MX)) == floor_to_int(__fadd_ru(fmaxf(Xa, Xb), MX));
-        const bool oky = floor_to_int(__fsub_rd(fminf(Ya, Yb), MY)) == floor_to_int(__fadd_ru(fmaxf(Ya, Yb), MY));
-        return clear && okx && oky;
-    };
-
-    const Geo &g = a.g;
+    for (int m = 0; m <= P; ++m) C[m] = pack2(rp.X[m], rp.Y[m]);
     const unsigned offx = (unsigned)rp.bx - 0x4B400000u, offy = (unsigned)rp.by - 0x4B400000u;
-    unsigned rcx = (unsigned)rs.cx - offx, rcy = (unsigned)rs.cy - offy;   // run pixel, raw form
-    int kst = k0;                 // first ray of the current run in this walk
-    int ka = k0 - 1;              // last evaluated ray (none yet)
-    float Xa = 0.f, Ya = 0.f;
-    int gap = 1;                  // next window at ka + gap
-    unsigned ev = 0, spn = 0;     // this column's evaluations and certified spans
-    for (;;) {
-        const bool act = on && ka + 1 < k1;
-        if (!__any_sync(0xffffffffu, act)) break;
-        const int kb = act ? min(ka + gap, k1 - 1) : ka + 1;
-        const bool span = act && kb > ka + 1;
-        bool av[W];
-#pragma unroll
-        for (int r = 0; r < W; ++r) av[r] = act && kb + r < k1;
-        eval_window(kb, av);
-        bool ok = act;
-        if (span) {
-            const bool same = rx[0] == rcx && ry[0] == rcy;
-            ok = same && certify(ka, kb, Xa, Ya, X[0], Y[0]);
-            spn += ok ? 1u : 0u;
-            if (!ok) {
-                ++ev;
-                // ray kb is past a pixel edge: the next window starts where the
-                // chord from ka crosses it; otherwise the bound failed, and the
-                // gap halves
-                int g2 = (kb - ka) >> 1;
-                if (!same && fabsf(Xa) < LIM && fabsf(X[0]) < LIM && fabsf(Ya) < LIM && fabsf(Y[0]) < LIM) {
-                    float t = 1.f;
-                    const float fa = __fsub_rn(__int_as_float((int)rcx), 12582912.0f);
-                    const float ga = __fsub_rn(__int_as_float((int)rcy), 12582912.0f);
-                    if (rx[0] != rcx) {
-                        const float e = X[0] > Xa ? __fadd_rn(fa, 1.f) : fa;
-                        t = fminf(t, __fsub_rn(e, Xa) * rcp_approx(__fsub_rn(X[0], Xa)));
-                    }
-                    if (ry[0] != rcy) {
-                        const float e = Y[0] > Ya ? __fadd_rn(ga, 1.f) : ga;
-                        t = fminf(t, __fsub_rn(e, Ya) * rcp_approx(__fsub_rn(Y[0], Ya)));
-                    }
-                    g2 = floor_to_int(fmaxf(t, 0.f) * (float)(kb - ka) - ML_SPAN_MARGIN);
-                }
-                gap = max(1, min(g2, kb - ka - 1));
-            }
-        }
-        if (ok) {
-            // slope baseline: the last evaluated ray, or at the column's start
-            // the window's first ray
-            const int kp = ka < k0 ? kb : ka;
-            const float Xp = ka < k0 ? X[0] : Xa, Yp = ka < k0 ? Y[0] : Ya;
-#pragma unroll
-            for (int r = 0; r < W; ++r) {
-                if (av[r]) {
-                    ++ev;
-                    if (dr[r]) ++drop;
-                    if (rx[r] != rcx || ry[r] != rcy) {
-                        flush_run(rs, (int)(rcx + offx), (int)(rcy + offy), rs.cnt + (unsigned)(kb + r - kst),
-                                  a.map_u32, g.mnx, g.mny);
-                        rs.cnt = 0;
-                        kst = kb + r;
-                        rcx = rx[r];
-                        rcy = ry[r];
-                    }
-                    ka = kb + r;
-                    Xa = X[r];
-                    Ya = Y[r];
-                }
-            }
-            // rays to the next pixel edge along the slope since the baseline;
-            // the next window starts ML_SPAN_MARGIN rays before it
-            gap = 1;
-            if (ka > kp && fabsf(Xa) < LIM && fabsf(Ya) < LIM && fabsf(Xp) < LIM && fabsf(Yp) < LIM) {
-                // (one reciprocal per component on the step's critical path)
-                const float fk = (float)(ka - kp);
-                const float dX = __fsub_rn(Xa, Xp), dY = __fsub_rn(Ya, Yp);
-                const float fX = __fsub_rn(Xa, __fsub_rn(__int_as_float((int)rcx), 12582912.0f));
-                const float fY = __fsub_rn(Ya, __fsub_rn(__int_as_float((int)rcy), 12582912.0f));
-                const float gX = (dX > 0.f ? __fsub_rn(1.f, fX) : fX) * fk;
-                const float gY = (dY > 0.f ? __fsub_rn(1.f, fY) : fY) * fk;
-                const float n = fminf(fminf(gX * rcp_approx(fabsf(dX)), gY * rcp_approx(fabsf(dY))), 1048576.f);
-                gap = max(1, floor_to_int(n - ML_SPAN_MARGIN));
-            }
-        }
+    // the run's pixel in raw floor form (the bits of floor + 1.5 2^23)
+    f32x2 R = pack2(__int_as_float((int)((unsigned)rs.cx - offx)), __int_as_float((int)((unsigned)rs.cy - offy)));
+    f32x2 pa = 0;                 // the last evaluated ray, off its pixel's centre
+    // the current run's first ray, as if all its rays lay in this column (an
+    // exact float: counts this long are flushed first)
+    if (rs.cnt > 1048576u) {
+        run_flush(rs, a.map_u32, a.g.mnx, a.g.mny);
+        rs.cnt = 0;
     }
-    if (on) rs.cnt += (unsigned)(k1 - kst);
-    rs.cx = (int)(rcx + offx);
-    rs.cy = (int)(rcy + offy);
+    float ust = ulo - (float)rs.cnt;
+    float ua = ulo - 1.f;         // last evaluated ray (none yet)
+    float gap = 1.f;
+    unsigned ev = 0, spn = 0;
+    const unsigned mnx = (unsigned)a.g.mnx, mny = (unsigned)a.g.mny;
+    bool act = on;
+    while (__any_sync(0xffffffffu, act)) {
+        // the window's rays (one ray, taken twice, at the end of the range),
+        // by the per-ray arithmetic
+        const float ub = fminf(ua + gap, uhi), w = ub - ua;
+        float u1 = fminf(__fadd_rn(ub, 1.f), uhi);
+        const f32x2 U0 = pack2(ub, ub), U1 = pack2(u1, u1);
+        f32x2 v0 = C[P], v1 = C[P];
+#pragma unroll
+        for (int m = P - 1; m >= 0; --m) {
+            v0 = fma2(v0, U0, C[m]);
+            v1 = fma2(v1, U1, C[m]);
+        }
+        if (nn > 0) {
+            float X0, Y0, X1, Y1;
+            unpack2(v0, X0, Y0);
+            unpack2(v1, X1, Y1);
+#pragma unroll 1
+            for (int q = 0; q < nn; ++q) {
+                const float4 L = near[q];
+                const float dy = __fsub_rn(L.y, dyl);
+                const float dy2 = __fmul_rn(dy, dy), dyy = __fmul_rn(dy, a.yx_f);
+                const float dx0 = __fsub_rn(L.x, ub), dx1 = __fsub_rn(L.x, u1);
+                const float s0 = __fmul_rn(L.z, rcp_approx(__fmaf_rn(dx0, dx0, dy2)));
+                const float s1 = __fmul_rn(L.z, rcp_approx(__fmaf_rn(dx1, dx1, dy2)));
+                X0 = __fmaf_rn(dx0, s0, X0);
+                Y0 = __fmaf_rn(dyy, s0, Y0);
+                X1 = __fmaf_rn(dx1, s1, X1);
+                Y1 = __fmaf_rn(dyy, s1, Y1);
+            }
+            v0 = pack2(X0, Y0);
+            v1 = pack2(X1, Y1);
+        }
+        const f32x2 f0 = add2_rd(v0, MAGIC);
+        f32x2 f1 = add2_rd(v1, MAGIC);
+        const bool same0 = f0 == R;
+        // when both rays changed pixel only the first is taken: one flush a step
+        if (!same0 && f1 != f0) {
+            f1 = f0;
+            v1 = v0;
+            u1 = ub;
+        }
+        const bool span = w > 1.5f;
+        // the span's rays: mono drops the curvature's margin, then both ends
+        // must lie in the pixel's interior narrowed by the margins
+        const f32x2 p0 = add2(add2(v0, fma2(R, NEG1, MAGIC)), NHALF);
+        const f32x2 dp = fma2(pa, NEG1, p0);
+        const float w2 = w * w;
+        float dX, dY, tX, tY, hx, hy, ax, ay, bx, by;
+        unpack2(dp, dX, dY);
+        unpack2(fma2(b.m, pack2(w2, w2), b.t), tX, tY);
+        const f32x2 W2 = pack2(fabsf(dX) > tX ? 0.f : w2, fabsf(dY) > tY ? 0.f : w2);
+        unpack2(fma2(b.s, W2, b.e), hx, hy);
+        unpack2(fma2(b.g, W2, pa), ax, ay);
+        unpack2(fma2(b.g, W2, p0), bx, by);
+        const bool in = fabsf(ax) < hx && fabsf(bx) < hx && fabsf(ay) < hy && fabsf(by) < hy;
+        const bool ok = act && (!span || (same0 && in));
+        spn += ok && span ? 1u : 0u;
+        ev += act ? 1u : 0u;
+        ev += ok && u1 > ub ? 1u : 0u;
+        // the run ends before ray b (ray b changed pixel) or after it
+        const bool chg = ok && f1 != R;
+        float rx, ry;
+        unpack2(R, rx, ry);
+        const unsigned cx = (unsigned)__float_as_int(rx) + offx, cy = (unsigned)__float_as_int(ry) + offy;
+        const unsigned n = count_of((same0 ? u1 : ub) - ust);
+        if (chg && cx < mnx && cy < mny) {
+            atomicAdd(a.map_u32 + (size_t)cy * mnx + cx, n);
+            rs.in += n;
+        }
+        if (chg) ust = same0 ? u1 : ub;
+        // slope at the last ray (of this window, or the old one when nothing
+        // was taken), and the next window
+        float d1x, d1y, sX, sY, cX, cY, DX, DY, eX, eY;
+        unpack2(fma2(v0, NEG1, v1), d1x, d1y);
+        const float rw = rcp_approx(w), h = ok ? (span ? w + 2.f : 1.f) : -w;
+        const f32x2 num = pack2(span ? dX : d1x, span ? dY : d1y);
+        unpack2(fma2(b.d, pack2(h, h), mul2(num, pack2(rw, rw))), sX, sY);
+        if (ok) {
+            R = f1;
+            pa = add2(add2(v1, fma2(f1, NEG1, MAGIC)), NHALF);
+            ua = u1;
+        }
+        unpack2(pa, cX, cY);
+        unpack2(b.d, DX, DY);
+        unpack2(b.e, eX, eY);
+        const float ne = fminf(fminf(rays_to_edge(cX, eX, sX, DX), rays_to_edge(cY, eY, sY, DY)), 1048576.f);
+        gap = __fsub_rn(__fadd_rd(ne - ML_SPAN_MARGIN, MAGIC_F), MAGIC_F);
+        // half the span when its bound failed, and when the parabola puts the
+        // edge near or past a ray that lies beyond it
+        if (!ok && (same0 || gap > 0.9f * w)) gap = __fsub_rn(__fadd_rd(0.5f * w, MAGIC_F), MAGIC_F);
+        gap = fmaxf(gap, 1.f);
+        act = act && ua < uhi;
+    }
+    if (on) rs.cnt = count_of(uhi + 1.f - ust);
+    float rx, ry;
+    unpack2(R, rx, ry);
+    rs.cx = __float_as_int(rx) + (int)offx;
+    rs.cy = __float_as_int(ry) + (int)offy;
     sc.evals += ev;
     sc.spans += spn;
 }
@@ -817,9 +755,8 @@ __device__ __forceinline__ float pin(float v)
 // One warp task of the mixed kernel (NGP deposit): stage the near list, then
 // walk each level-2 column of the task.  Shared by the single-map and the
 // batched persistent kernels.
-// SPAN: 0 the per-ray walk only; 1 the certified walk in one copy for every
-// near-list length; 2 the same with a second copy for empty near lists.
-template <int P, int SPAN>
+// SPAN: the certified walk where it pays, else the per-ray walk only.
+template <int P, bool SPAN>
 __device__ __forceinline__ void shoot_task(const ShootArgs &a, int64_t t, float4 *near, float2 *nlo,
                                            int lane, float dyl, float dyl_lo, RunState &rs,
                                            unsigned &drop, unsigned long long &pairs,
@@ -854,35 +791,28 @@ __device__ __forceinline__ void shoot_task(const ShootArgs &a, int64_t t, float4
         RowPoly<P> rp;
         row_setup<P>(a.nodes + (min(c2y, g.N2y - 1) * g.N2x + c2x) * node_stride(P), q, ry, a, rp);
         pairs += (unsigned long long)nn * (unsigned long long)(k1 - k0);
+        rs.tot += (unsigned)(k1 - k0);
         if constexpr (SPAN) {
             // the certified walk where runs are long: no near lens, or every
-            // near lens farther than a.span_far lattice units from every ray
-            // of the warp's walk; elsewhere the per-ray walk
-            bool far = true;
-            if (nn > 0) {
-                bool close = false;
-                if (k1 > k0) {
-                    const float ulo = __fadd_rn((float)k0, a.c0_f), uhi = __fadd_rn((float)(k1 - 1), a.c0_f);
-                    for (int q = 0; q < nn; ++q) {
-                        const float4 L = near[q];
-                        const float dy = __fsub_rn(L.y, dyl);
-                        const float dx = fmaxf(0.f, fmaxf(ulo - L.x, L.x - uhi));
-                        close |= __fmaf_rn(dx, dx, dy * dy) < a.span_far * a.span_far;
-                    }
-                }
-                far = !__any_sync(0xffffffffu, close);
+            // near lens farther than the field's span_far (and the
+            // close-pass radius) from every ray of the warp's walk; elsewhere
+            // the per-ray walk
+            const bool on = k1 > k0;
+            const float ulo = __fadd_rn((float)k0, a.c0_f), uhi = __fadd_rn((float)(on ? k1 - 1 : k0), a.c0_f);
+            bool close = false;
+#pragma unroll 1
+            for (int q = 0; q < nn; ++q) {
+                const float4 L = near[q];
+                const float dy = __fsub_rn(L.y, dyl);
+                const float dx = fmaxf(0.f, fmaxf(ulo - L.x, L.x - uhi));
+                close |= __fmaf_rn(dx, dx, dy * dy) < a.span_far2;
             }
-            if (far) {
-                // one copy of the walk for every near-list length (its lens loops
-                // run from shared memory) in the single-map kernel, where a second
-                // copy for empty lists measured slower, its code competing for the
-                // instruction cache; the batch kernel, whose lens-dense maps walk
-                // most lens columns ray by ray, measured faster with it
-                if (SPAN == 2 && nn == 0)
-                    walk_span<P, 0>(rp, a, nl, nn, k0, k1, dyl, dyl_lo, rs, drop, sc);
-                else
-                    walk_span<P, NN_DYN>(rp, a, nl, nn, k0, k1, dyl, dyl_lo, rs, drop, sc);
-                continue;
+            if (!__any_sync(0xffffffffu, on && close)) {
+                const SpanBound sb = span_bound<P>(rp, a, near, nn, ulo, uhi, dyl);
+                if (!__any_sync(0xffffffffu, on && !sb.ok)) {
+                    walk_span<P>(rp, sb, a, near, nn, on, ulo, uhi, dyl, rs, sc);
+                    continue;
+                }
             }
         }
         {
@@ -954,11 +884,11 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, ML_MIN_BLOCKS) k_shoot_mix
         bool stop;
         const int64_t t = fetch_task(a, lane, stop);
         if (stop || t >= a.n_tasks) break;
-        shoot_task<P, SPAN ? 1 : 0>(a, t, near, nlo, lane, dyl, dyl_lo, rs, drop, pairs, tasks, sc);
+        shoot_task<P, SPAN>(a, t, near, nlo, lane, dyl, dyl_lo, rs, drop, pairs, tasks, sc);
     }
     run_flush(rs, a.map_u32, a.g.mnx, a.g.mny);
     // dropped rays were sent far outside the map and counted as out above
-    flush_stats(a, rs.in, rs.out - drop, drop, pairs, lane == 0 ? tasks : 0, 0u);
+    flush_stats(a, rs.in, rs.tot - rs.in - drop, drop, pairs, lane == 0 ? tasks : 0, 0u);
     flush_spans(a, sc);
 }
 
@@ -1003,7 +933,7 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, ML_MIN_BLOCKS) k_shoot_bat
             if (cur >= 0) {
                 const ShootArgs &ac = b.args[cur];
                 run_flush(rs, ac.map_u32, ac.g.mnx, ac.g.mny);
-                flush_stats(ac, rs.in, rs.out - drop, drop, pairs, lane == 0 ? tasks : 0, 0u);
+                flush_stats(ac, rs.in, rs.tot - rs.in - drop, drop, pairs, lane == 0 ? tasks : 0, 0u);
                 flush_spans(ac, sc);
                 rs = RunState{-1, -1, 0u, 0u, 0u};
                 drop = 0;
@@ -1014,13 +944,13 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, ML_MIN_BLOCKS) k_shoot_bat
             cur = lo;
             lane_dy(b.args[cur].l3yx, lane, dyl, dyl_lo);
         }
-        shoot_task<P, SPAN ? 2 : 0>(b.args[cur], t - b.task_base[cur], near, nlo, lane, dyl, dyl_lo, rs,
+        shoot_task<P, SPAN>(b.args[cur], t - b.task_base[cur], near, nlo, lane, dyl, dyl_lo, rs,
                                     drop, pairs, tasks, sc);
     }
     if (cur >= 0) {
         const ShootArgs &ac = b.args[cur];
         run_flush(rs, ac.map_u32, ac.g.mnx, ac.g.mny);
-        flush_stats(ac, rs.in, rs.out - drop, drop, pairs, lane == 0 ? tasks : 0, 0u);
+        flush_stats(ac, rs.in, rs.tot - rs.in - drop, drop, pairs, lane == 0 ? tasks : 0, 0u);
         flush_spans(ac, sc);
     }
 }

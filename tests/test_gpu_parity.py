@@ -358,6 +358,33 @@ def test_certified_walk_equals_per_ray_walk(ml, case):
     fp.close()
 
 
+@pytest.mark.parametrize("l2_sub", [(5, 5), (10, 5), (40, 20)])
+@pytest.mark.parametrize("span_far", [0.0, 1.0, 60.0, 1e9])
+def test_certified_walk_at_any_grid_and_lens_distance(ml, l2_sub, span_far):
+    """Long and short level-2 columns, and lens columns spanned from the
+    close-pass radius outwards up to not at all, on a lattice dense enough
+    for long runs (9e7 rays on 200 x 150 pixels): always the per-ray counts."""
+    w = _mixed_case(seed=11, n_av=3000)
+    fc = _field(ml, w, precision=ml.PREC_MIXED, l2_sub=l2_sub, span_far=span_far)
+    fp = _field(ml, w, precision=ml.PREC_MIXED, l2_sub=l2_sub, walk=ml.WALK_PER_RAY)
+    nx3, n = fc.info["n_rays_x"], fc.n_rays
+    for r0, r1 in ((0, n), (3 * nx3 + 11, 40 * nx3 + 5), (9 * nx3 + 100, 9 * nx3 + 103)):
+        for f in (fc, fp):
+            f.clear()
+            f.shoot(r0, r1)
+        a, b = fc.counts().cpu().numpy(), fp.counts().cpu().numpy()
+        assert np.array_equal(a, b), int(np.abs(a.astype(np.int64) - b.astype(np.int64)).sum())
+        sa, sb = fc.stats(), fp.stats()
+        for k in ("rays_in", "rays_out", "rays_dropped", "near_pairs"):
+            assert sa[k] == sb[k], k
+    if span_far == 0.0:
+        fc.clear()
+        fc.shoot()
+        assert fc.stats()["spans"] > 0 and fc.stats()["rays_evaluated"] < n
+    fc.close()
+    fp.close()
+
+
 def test_mixed_map_matches_oracle_and_split_invariance(ml):
     w = _mixed_case(6)
     f = _field(ml, w, precision=ml.PREC_MIXED)
