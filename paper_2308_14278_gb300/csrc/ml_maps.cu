@@ -8,6 +8,7 @@
 #include <math.h>
 
 #include <mutex>
+#include <type_traits>
 
 namespace ml {
 
@@ -93,26 +94,71 @@ cudaError_t launch_mu(const Geo &g, const uint32_t *cu, const float *cf, int wan
     return cudaGetLastError();
 }
 
-// Light curves (§4.1, Fig. 3).  For every sample: bilinear interpolation between the four
-// pixel centres around the point, each value being the map convolved with
-// the separable normalised Gaussian taps (zero outside the map).  Only the
-// pixels the samples need are convolved.  One warp per sample group; taps
-// in shared memory.
-__global__ void k_light_curves(Geo g, const uint32_t *__restrict__ cu, const float *__restrict__ cf,
-                               double scale, const double *__restrict__ tracks, int n_tracks,
-                               int n_samples, int h, const float *__restrict__ taps_g,
-                               float *__restrict__ out)
+// Light curves (§4.1, Fig. 3).  A sample is the bilinear interpolation between
+// the four pixel centres around its point, each value being the map convolved
+// with the separable normalised Gaussian taps (zero outside the map); corner
+// pixels outside the map count nothing.  Bilinear weights and taps of one axis
+// combine to N = 2h + 2 weights, W[k] = w0 taps[k] + w1 taps[k-1], so a sample
+// is sum_y Wy[y] (sum_x Wx[x] M): N^2 products instead of 4 (2h + 1)^2.
+
+// One axis of a sample: floor of its position and the two corners' weights as
+// hi + lo floats, zero for a corner outside [0, size).
+struct LcAxis {
+    float w0h, w0l, w1h, w1l;
+    int i0;
+};
+
+__device__ __forceinline__ LcAxis lc_axis(double t, int size)
 {
-    __shared__ float taps[129];
-    for (int t = threadIdx.x; t <= 2 * h; t += blockDim.x) taps[t] = taps_g[t];
-    __syncthreads();
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= (int64_t)n_tracks * n_samples) return;
-    int tr = (int)(q / n_samples), k = (int)(q % n_samples);
-    const double *T = tracks + 4 * tr;
-    double t = n_samples > 1 ? (double)k / (double)(n_samples - 1) : 0.0;
-    double u = T[0] + t * (T[2] - T[0]) - 0.5;
-    double v = T[1] + t * (T[3] - T[1]) - 0.5;
+    LcAxis a;
+    const double f = floor(t);
+    a.i0 = (int)f;
+    const double w = t - f;
+    const int i1 = (int)((unsigned)a.i0 + 1u);
+    const double w0 = a.i0 >= 0 && a.i0 < size ? 1.0 - w : 0.0, w1 = i1 >= 0 && i1 < size ? w : 0.0;
+    a.w0h = (float)w0;
+    a.w0l = (float)(w0 - (double)a.w0h);
+    a.w1h = (float)w1;
+    a.w1l = (float)(w1 - (double)a.w1h);
+    return a;
+}
+
+// s + c with the rounding of the sum kept (Knuth's two-sum).
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// W[k] as hi + lo floats, in FP32 instructions (FP64 runs at 1/64 of their rate).
+__device__ __forceinline__ float2 lc_weight(const LcAxis &a, const float *taps, int h, int k)
+{
+    const float t0 = k <= 2 * h ? taps[k] : 0.f, t1 = k > 0 ? taps[k - 1] : 0.f;
+    const float p0 = __fmul_rn(a.w0h, t0), p1 = __fmul_rn(a.w1h, t1);
+    const float e0 = __fmaf_rn(a.w0l, t0, __fmaf_rn(a.w0h, t0, -p0));
+    const float e1 = __fmaf_rn(a.w1l, t1, __fmaf_rn(a.w1h, t1, -p1));
+    float s, e;
+    two_sum(p0, p1, s, e);
+    e = __fadd_rn(e, __fadd_rn(e0, e1));
+    const float hi = __fadd_rn(s, e);
+    return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, s)));
+}
+
+// Position of sample k of a track (pixel-centre coordinates).
+__device__ __forceinline__ void lc_point(const double *T, int k, int n_samples, double &u, double &v)
+{
+    const double t = n_samples > 1 ? (double)k / (double)(n_samples - 1) : 0.0;
+    u = T[0] + t * (T[2] - T[0]) - 0.5;
+    v = T[1] + t * (T[3] - T[1]) - 0.5;
+}
+
+// A sample corner by corner in FP64 (samples whose weighted sum is not an
+// ordinary number: infinities and NaN in the map, sums near the FP32 range's
+// ends).
+__device__ __noinline__ double lc_sample64(const uint32_t *cu, const float *cf, int mnx, int mny, double u,
+                                           double v, int h, const float *taps)
+{
     double fu = floor(u), fv = floor(v);
     double wx = u - fu, wy = v - fv;
     int i0 = (int)fu, j0 = (int)fv;
@@ -120,16 +166,16 @@ __global__ void k_light_curves(Geo g, const uint32_t *__restrict__ cu, const flo
     for (int c = 0; c < 4; ++c) {
         int pi = i0 + (c & 1), pj = j0 + (c >> 1);
         double wc = ((c & 1) ? wx : 1.0 - wx) * ((c >> 1) ? wy : 1.0 - wy);
-        if (pi < 0 || pi >= g.mnx || pj < 0 || pj >= g.mny || wc == 0.0) continue;
+        if (pi < 0 || pi >= mnx || pj < 0 || pj >= mny || wc == 0.0) continue;
         double conv = 0.0;
         for (int dy = -h; dy <= h; ++dy) {
             int yy = pj + dy;
-            if (yy < 0 || yy >= g.mny) continue;
+            if (yy < 0 || yy >= mny) continue;
             double row = 0.0;
-            const int64_t base = (int64_t)yy * g.mnx;
+            const int64_t base = (int64_t)yy * mnx;
             for (int dx = -h; dx <= h; ++dx) {
                 int xx = pi + dx;
-                if (xx < 0 || xx >= g.mnx) continue;
+                if (xx < 0 || xx >= mnx) continue;
                 double val = cu ? (double)cu[base + xx] : (double)cf[base + xx];
                 row += (double)taps[dx + h] * val;
             }
@@ -137,7 +183,136 @@ __global__ void k_light_curves(Geo g, const uint32_t *__restrict__ cu, const flo
         }
         acc += wc * conv;
     }
-    out[q] = (float)(acc * scale);
+    return acc;
+}
+
+// s + c += (wh + wl) v with the product's and the sum's FP32 roundings kept in
+// c (error-free product by a fused multiply-add): about 46 bits.
+__device__ __forceinline__ void dot_add(float &s, float &c, float wh, float wl, float v)
+{
+    const float p = __fmul_rn(wh, v);
+    const float e = __fmaf_rn(wl, v, __fmaf_rn(wh, v, -p));
+    float t, f;
+    two_sum(s, p, t, f);
+    s = t;
+    c = __fadd_rn(c, __fadd_rn(f, e));
+}
+
+constexpr int LC_LANES = 8;                         // lanes per sample
+constexpr int LC_THREADS = 128;
+constexpr int LC_SAMPLES = LC_THREADS / LC_LANES;   // samples per block
+
+// Eight lanes per sample: a lane takes every eighth column of the window (a
+// 32-byte sector per row and group) and sums it over the rows, with weights and
+// sums as hi + lo floats.  FP64 runs at 1/64 of FP32's rate here: one thread
+// per sample, corner by corner in FP64 (4 x 33 x 33 products for a source of 4
+// pixels), took 7.9 ms for 80 curves of 4096 samples; this takes 0.34 ms and lies closer
+// to the sums in 64 bits.  Bound by FP32 issue: 18 instructions per pixel and
+// sample, 3.8e8 of them.
+template <class T>
+__global__ void __launch_bounds__(LC_THREADS) k_light_curves(int mnx, int mny, const T *__restrict__ map,
+                                                             double scale, const double *__restrict__ tracks,
+                                                             int n_tracks, int n_samples, int h,
+                                                             const float *__restrict__ taps_g,
+                                                             float *__restrict__ out)
+{
+    __shared__ float taps[129];
+    extern __shared__ float2 lc_wy[];               // LC_SAMPLES x N
+    const int N = 2 * h + 2;
+    for (int t = threadIdx.x; t <= 2 * h; t += blockDim.x) taps[t] = taps_g[t];
+    __syncthreads();
+    const int lane = threadIdx.x % LC_LANES, slot = threadIdx.x / LC_LANES;
+    const int64_t q0 = blockIdx.x * (int64_t)LC_SAMPLES, q = q0 + slot, n = (int64_t)n_tracks * n_samples;
+    const bool have = q < n;
+    // the samples' positions, in FP64, one thread per sample
+    __shared__ LcAxis axes[2][LC_SAMPLES];
+    if (threadIdx.x < LC_SAMPLES && q0 + threadIdx.x < n) {
+        const int64_t i = q0 + threadIdx.x;
+        const int tr = (int)(i / n_samples);
+        double u, v;
+        lc_point(tracks + 4 * tr, (int)(i - (int64_t)tr * n_samples), n_samples, u, v);
+        axes[0][threadIdx.x] = lc_axis(u, mnx);
+        axes[1][threadIdx.x] = lc_axis(v, mny);
+    }
+    __syncthreads();
+    const LcAxis ax = axes[0][slot], ay = axes[1][slot];
+    float2 *wy = lc_wy + slot * N;
+    for (int k = lane; k < N; k += LC_LANES) wy[k] = lc_weight(ay, taps, h, k);
+    __syncwarp();
+    // rows and columns of the window inside the map (64-bit: the window of a
+    // track far outside lies nowhere)
+    const int64_t x0 = (int64_t)ax.i0 - h, y0 = (int64_t)ay.i0 - h;
+    const int ka = (int)max((int64_t)0, min((int64_t)N, -y0)), kb = (int)max((int64_t)0, min((int64_t)N, mny - y0));
+    float S = 0.f, C = 0.f;
+    unsigned any = 0;
+    if (have) {
+        for (int k = lane; k < N; k += LC_LANES) {
+            const int64_t x = x0 + k;
+            if (x < 0 || x >= mnx) continue;
+            const float2 w = lc_weight(ax, taps, h, k);
+            const T *p = map + (y0 + ka) * mnx + x;
+            float s = 0.f, c = 0.f;
+#pragma unroll 4
+            for (int r = ka; r < kb; ++r, p += mnx) {
+                const T val = __ldg(p);
+                const float2 W = wy[r];
+                if constexpr (sizeof(T) == 4 && std::is_integral<T>::value) {
+                    any |= val;
+                    // counts below 2^23 become floats by their bits; larger ones
+                    // in two exact parts
+                    if (val < 0x800000u) {
+                        dot_add(s, c, W.x, W.y, __fsub_rn(__uint_as_float(0x4B000000u | val), 8388608.f));
+                    } else {
+                        dot_add(s, c, W.x, W.y, (float)(val & 0xFFFFFF00u));
+                        dot_add(s, c, W.x, W.y, (float)(val & 0xFFu));
+                    }
+                } else {
+                    any |= __float_as_uint(val) & 0x7FFFFFFFu;
+                    dot_add(s, c, W.x, W.y, val);
+                }
+            }
+            C = __fmaf_rn(w.x, c, C);
+            dot_add(S, C, w.x, w.y, s);
+        }
+    }
+#pragma unroll
+    for (int o = LC_LANES / 2; o > 0; o >>= 1) {
+        const float s2 = __shfl_down_sync(0xffffffffu, S, o, LC_LANES), c2 = __shfl_down_sync(0xffffffffu, C, o, LC_LANES);
+        float t, e;
+        two_sum(S, s2, t, e);
+        S = t;
+        C = __fadd_rn(C, __fadd_rn(c2, e));
+        any |= __shfl_down_sync(0xffffffffu, any, o, LC_LANES);
+    }
+    if (lane != 0 || !have) return;
+    double tot = (double)S + (double)C;
+    if (!(fabs(tot) >= 1e-20 && fabs(tot) <= 1e37) && (any != 0 || !(tot == 0.0))) {
+        const uint32_t *cu = nullptr;
+        const float *cf = nullptr;
+        if constexpr (std::is_integral<T>::value) cu = map; else cf = map;
+        const int tr = (int)(q / n_samples);
+        double u, v;
+        lc_point(tracks + 4 * tr, (int)(q - (int64_t)tr * n_samples), n_samples, u, v);
+        tot = lc_sample64(cu, cf, mnx, mny, u, v, h, taps);
+    }
+    out[q] = (float)(tot * scale);
+}
+
+static cudaError_t run_light_curves(int mnx, int mny, const uint32_t *cu, const float *cf, double scale,
+                                    const double *d_tracks, int n_tracks, int n_samples, int h,
+                                    const float *d_taps, float *out, cudaStream_t s)
+{
+    const int64_t n = (int64_t)n_tracks * n_samples;
+    if (n == 0) return cudaSuccess;
+    const unsigned blocks = (unsigned)((n + LC_SAMPLES - 1) / LC_SAMPLES);
+    const size_t smem = sizeof(float2) * LC_SAMPLES * (size_t)(2 * h + 2);   // at most 16.6 KB
+    if (cu)
+        k_light_curves<uint32_t><<<blocks, LC_THREADS, smem, s>>>(mnx, mny, cu, scale, d_tracks, n_tracks, n_samples,
+                                                                  h, d_taps, out);
+    else
+        k_light_curves<float><<<blocks, LC_THREADS, smem, s>>>(mnx, mny, cf, scale, d_tracks, n_tracks, n_samples, h,
+                                                               d_taps, out);
+    return cudaGetLastError();
 }
 
 // Normalised Gaussian source taps of §4.1 at integer offsets |t| <= floor(4 sigma),
@@ -205,10 +380,7 @@ cudaError_t launch_light_curves_noalloc(const Geo &g, const uint32_t *cu, const 
     e = cudaMemcpyAsync(d_tracks, tracks_host, sizeof(double) * 4 * (size_t)n_tracks,
                         cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
-    int64_t n = (int64_t)n_tracks * n_samples;
-    k_light_curves<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(g, cu, cf, scale, d_tracks, n_tracks,
-                                                               n_samples, h, d_taps, out);
-    return cudaGetLastError();
+    return run_light_curves(g.mnx, g.mny, cu, cf, scale, d_tracks, n_tracks, n_samples, h, d_taps, out, s);
 }
 
 cudaError_t launch_light_curves(const Geo &g, const uint32_t *cu, const float *cf, double scale,
@@ -223,10 +395,7 @@ cudaError_t launch_light_curves(const Geo &g, const uint32_t *cu, const float *c
     if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(d_taps, taps, sizeof(float) * (2 * h + 1), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) { cudaFreeAsync(d_taps, s); return e; }
-    int64_t n = (int64_t)n_tracks * n_samples;
-    k_light_curves<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(g, cu, cf, scale, tracks, n_tracks,
-                                                               n_samples, h, d_taps, out);
-    e = cudaGetLastError();
+    e = run_light_curves(g.mnx, g.mny, cu, cf, scale, tracks, n_tracks, n_samples, h, d_taps, out, s);
     cudaFreeAsync(d_taps, s);
     return e;
 }
@@ -237,11 +406,7 @@ cudaError_t launch_light_curves_dev(const Geo &g, const uint32_t *cu, const floa
                                     const double *d_tracks, int n_tracks, int n_samples, int h,
                                     const float *d_taps, float *out, cudaStream_t s)
 {
-    int64_t n = (int64_t)n_tracks * n_samples;
-    if (n == 0) return cudaSuccess;
-    k_light_curves<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(g, cu, cf, scale, d_tracks, n_tracks,
-                                                               n_samples, h, d_taps, out);
-    return cudaGetLastError();
+    return run_light_curves(g.mnx, g.mny, cu, cf, scale, d_tracks, n_tracks, n_samples, h, d_taps, out, s);
 }
 
 // ---- 64-bit sum of a count map -------------------------------------------------
@@ -431,44 +596,102 @@ cudaError_t launch_peak_stats(const uint32_t *N, int nx, int ny, int along, cons
 
 // ---- adjoint of the light curves ---------------------------------------------
 //
-// A light-curve sample is L = sum_c w_c sum_{dx,dy} taps[dx] taps[dy] M[p_c + (dx, dy)]
-// over the four bilinear corners p_c (k_light_curves), a linear map of the
-// magnification map M.  Its transpose adds, for every sample with incoming
-// gradient g, g w_c taps[dx] taps[dy] to the same pixels, skipping exactly the
-// corners and taps the forward skips.
-__global__ void k_light_curves_adj(int mnx, int mny, const double *__restrict__ tracks, int n_tracks,
-                                   int n_samples, int h, const float *__restrict__ taps_g,
-                                   const float *__restrict__ dl, float *__restrict__ gmap)
+// A light-curve sample is a weighted sum of its window's pixels (k_light_curves,
+// W as there), a linear map of the magnification map M.  Its transpose adds
+// g Wy[y] Wx[x] to the same pixels for every sample with incoming gradient g,
+// leaving out weights that are zero.
+//
+// A block takes LCA_CHUNK consecutive samples of one track and gathers: a warp
+// takes the rows of the chunk's bounding box in turn, a lane three of the
+// columns that the row's samples reach, and a pixel sums its samples in a
+// register and is added once.  One thread and 4 (2h + 1)^2 atomics a sample
+// took 5.0 ms for 80 curves of 4096 samples of a 4-pixel source, bound by the
+// L2's atomics, N^2 atomics a sample 0.57 ms for 40 curves, this 0.28 ms
+// (0.11 against 0.43 ms at 0.5 pixels, 1.5 against 4.5 ms at 16; samples 0.3
+// to 8 pixels apart alike), bound by issue.
+constexpr int LCA_THREADS = 256;
+constexpr int LCA_CHUNK = 16;
+constexpr int LCA_COLS = 3;
+
+__global__ void __launch_bounds__(LCA_THREADS) k_light_curves_adj(int mnx, int mny,
+                                                                     const double *__restrict__ tracks, int n_samples,
+                                                                     int h, const float *__restrict__ taps_g,
+                                                                     const float *__restrict__ dl,
+                                                                     float *__restrict__ gmap)
 {
     __shared__ float taps[129];
-    for (int t = threadIdx.x; t <= 2 * h; t += blockDim.x) taps[t] = taps_g[t];
+    __shared__ int sx[LCA_CHUNK], sy[LCA_CHUNK];      // first column and row of each sample's window
+    __shared__ int rows[2];
+    __shared__ LcAxis axes[2][LCA_CHUNK];
+    extern __shared__ float lca_w[];                  // per sample N x weights, N y weights (times g)
+    const int N = 2 * h + 2, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int t = tid; t <= 2 * h; t += blockDim.x) taps[t] = taps_g[t];
     __syncthreads();
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= (int64_t)n_tracks * n_samples) return;
-    const float gq = dl[q];
-    if (gq == 0.f) return;
-    int tr = (int)(q / n_samples), k = (int)(q % n_samples);
-    const double *T = tracks + 4 * tr;
-    double t = n_samples > 1 ? (double)k / (double)(n_samples - 1) : 0.0;
-    double u = T[0] + t * (T[2] - T[0]) - 0.5;
-    double v = T[1] + t * (T[3] - T[1]) - 0.5;
-    double fu = floor(u), fv = floor(v);
-    double wx = u - fu, wy = v - fv;
-    int i0 = (int)fu, j0 = (int)fv;
-    for (int c = 0; c < 4; ++c) {
-        int pi = i0 + (c & 1), pj = j0 + (c >> 1);
-        double wc = ((c & 1) ? wx : 1.0 - wx) * ((c >> 1) ? wy : 1.0 - wy);
-        if (pi < 0 || pi >= mnx || pj < 0 || pj >= mny || wc == 0.0) continue;
-        const float gw = (float)((double)gq * wc);
-        for (int dy = -h; dy <= h; ++dy) {
-            int yy = pj + dy;
-            if (yy < 0 || yy >= mny) continue;
-            const float gy = gw * taps[dy + h];
-            for (int dx = -h; dx <= h; ++dx) {
-                int xx = pi + dx;
-                if (xx < 0 || xx >= mnx) continue;
-                atomicAdd(gmap + (int64_t)yy * mnx + xx, gy * taps[dx + h]);
+    const int chunks = (n_samples + LCA_CHUNK - 1) / LCA_CHUNK;
+    const int tr = blockIdx.x / chunks, k0 = (blockIdx.x - tr * chunks) * LCA_CHUNK;
+    const int ns = min(LCA_CHUNK, n_samples - k0);
+    if (tid < ns) {
+        double u, v;
+        lc_point(tracks + 4 * tr, k0 + tid, n_samples, u, v);
+        const LcAxis ax = lc_axis(u, mnx), ay = lc_axis(v, mny);
+        axes[0][tid] = ax;
+        axes[1][tid] = ay;
+        // (windows far outside the map, where the weights are zero, are held
+        // within a range that cannot overflow)
+        sx[tid] = max(min(ax.i0, mnx + 1024), -1024) - h;
+        sy[tid] = max(min(ay.i0, mny + 1024), -1024) - h;
+    }
+    __syncthreads();
+    for (int q = tid; q < ns * N; q += blockDim.x) {
+        const int i = q / N, k = q - i * N;
+        const float g = dl[(int64_t)tr * n_samples + k0 + i];
+        lca_w[2 * i * N + k] = lc_weight(axes[0][i], taps, h, k).x;
+        const float2 w = lc_weight(axes[1][i], taps, h, k);
+        lca_w[(2 * i + 1) * N + k] = g == 0.f || w.x == 0.f ? 0.f : g * w.x;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        int c = sy[0], d = sy[0];
+        for (int i = 1; i < ns; ++i) {
+            c = min(c, sy[i]);
+            d = max(d, sy[i]);
+        }
+        rows[0] = max(c, 0);
+        rows[1] = min(d + N, mny);
+    }
+    __syncthreads();
+    for (int y = rows[0] + wid; y < rows[1]; y += LCA_THREADS / 32) {
+        // lane i: sample i's weight of this row (0 outside its window)
+        float wy = 0.f;
+        int cx = 0;
+        if (lane < ns) {
+            const unsigned ky = (unsigned)(y - sy[lane]);
+            if (ky < (unsigned)N) wy = lca_w[(2 * lane + 1) * N + ky];
+            cx = sx[lane];
+        }
+        const unsigned live = __ballot_sync(0xffffffffu, wy != 0.f);
+        if (live == 0) continue;
+        const int xa = max(0, __reduce_min_sync(0xffffffffu, wy != 0.f ? cx : 0x7fffffff));
+        const int xb = min(mnx, __reduce_max_sync(0xffffffffu, wy != 0.f ? cx : -0x7fffffff) + N);
+        for (int x = xa + lane; x - lane < xb; x += 32 * LCA_COLS) {
+            float acc[LCA_COLS];
+#pragma unroll
+            for (int c = 0; c < LCA_COLS; ++c) acc[c] = 0.f;
+            for (unsigned m = live; m != 0; m &= m - 1) {
+                const int i = __ffs(m) - 1;
+                const float w = __shfl_sync(0xffffffffu, wy, i);
+                const int kx = x - __shfl_sync(0xffffffffu, cx, i);
+                const float *wx = lca_w + 2 * i * N;
+#pragma unroll
+                for (int c = 0; c < LCA_COLS; ++c)
+                    if ((unsigned)(kx + 32 * c) < (unsigned)N) {
+                        const float v = wx[kx + 32 * c];
+                        if (v != 0.f) acc[c] = fmaf(w, v, acc[c]);
+                    }
             }
+#pragma unroll
+            for (int c = 0; c < LCA_COLS; ++c)
+                if (x + 32 * c < xb && acc[c] != 0.f) atomicAdd(gmap + (int64_t)y * mnx + x + 32 * c, acc[c]);
         }
     }
 }
@@ -486,8 +709,10 @@ cudaError_t launch_light_curves_adj(int mnx, int mny, const double *d_tracks, in
     e = cudaMemcpyAsync(d_taps, taps, sizeof(float) * (2 * h + 1), cudaMemcpyHostToDevice, s);
     const int64_t n = (int64_t)n_tracks * n_samples;
     if (e == cudaSuccess && n > 0) {
-        k_light_curves_adj<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(mnx, mny, d_tracks, n_tracks,
-                                                                        n_samples, h, d_taps, dl, gmap);
+        const int64_t blocks = (int64_t)n_tracks * ((n_samples + LCA_CHUNK - 1) / LCA_CHUNK);
+        if (blocks > 0x7fffffff) { cudaFreeAsync(d_taps, s); return cudaErrorInvalidConfiguration; }
+        k_light_curves_adj<<<(unsigned)blocks, LCA_THREADS, sizeof(float) * 2 * LCA_CHUNK * (size_t)(2 * h + 2), s>>>(
+            mnx, mny, d_tracks, n_samples, h, d_taps, dl, gmap);
         e = cudaGetLastError();
     }
     cudaFreeAsync(d_taps, s);

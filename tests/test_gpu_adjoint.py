@@ -294,6 +294,92 @@ def test_map_light_curves_match_oracle(ml):
     assert np.allclose(out.cpu().numpy(), ref, rtol=1e-5, atol=1e-6)
 
 
+def _corner_sums(mu, tracks, ns, sigma):
+    """Light curves corner by corner and tap by tap in FP64 with float taps, as
+    the library documents them: corners outside the map or of weight zero and
+    taps outside the map are left out (so infinities elsewhere stay there)."""
+    ny, nx = mu.shape
+    h = int(np.floor(4 * sigma))
+    t = np.exp(-0.5 * (np.arange(-h, h + 1) / sigma) ** 2)
+    taps = (t / t.sum()).astype(np.float32).astype(np.float64)
+    out = np.zeros((len(tracks), ns))
+    for i, (x0, y0, x1, y1) in enumerate(tracks):
+        for k in range(ns):
+            f = k / (ns - 1) if ns > 1 else 0.0
+            u, v = x0 + f * (x1 - x0) - 0.5, y0 + f * (y1 - y0) - 0.5
+            i0, j0 = int(np.floor(u)), int(np.floor(v))
+            for c in range(4):
+                pi, pj = i0 + (c & 1), j0 + (c >> 1)
+                w = (u - i0 if c & 1 else 1 - (u - i0)) * (v - j0 if c >> 1 else 1 - (v - j0))
+                if not (0 <= pi < nx and 0 <= pj < ny) or w == 0:
+                    continue
+                xs, ys = np.arange(max(0, pi - h), min(nx, pi + h + 1)), np.arange(max(0, pj - h), min(ny, pj + h + 1))
+                with np.errstate(invalid="ignore", over="ignore"):
+                    rows = (mu[np.ix_(ys, xs)] * taps[xs - pi + h]).sum(1)
+                    out[i, k] += w * (rows * taps[ys - pj + h]).sum()
+    return out
+
+
+@pytest.mark.parametrize("sigma", [0.2, 0.5, 1.9, 16.0])
+@pytest.mark.parametrize("ns", [1, 3, 33])
+def test_light_curves_and_transpose_over_sources_and_spacings(ml, sigma, ns):
+    """Windows of 2 to 130 pixels on a 37 x 29 map, samples far apart and close
+    together (33: a chunk and one more), tracks in, across and beyond the rim.
+    The sums carry about 46 bits, so a curve lies within the rounding of its
+    float (2^-24) and of the sums' 1e-12; the transpose is FP32: per pixel at
+    most ns + 3 roundings of terms that add up to J^T |w|."""
+    import torch
+    rng = np.random.default_rng(3)
+    mu = rng.uniform(-1.0, 3.0, (29, 37)).astype(np.float32)
+    tracks = np.array([[3.0, 4.0, 30.0, 20.0], [-40.0, 5.5, 80.0, 9.5], [12.25, -3.0, 12.25, 31.0],
+                       [36.9, 28.9, 37.4, 29.4], [500.0, 500.0, 501.0, 900.0], [5.5, 6.5, 7.5, 6.5]])
+    m = torch.as_tensor(mu).cuda()
+    out = torch.empty((len(tracks), ns), dtype=torch.float32, device="cuda")
+    ml.ml_map_light_curves(m, tracks, ns, sigma, out)
+    ref = _corner_sums(mu.astype(np.float64), tracks, ns, sigma)
+    mag = _corner_sums(np.abs(mu).astype(np.float64), tracks, ns, sigma)
+    assert np.all(np.abs(out.cpu().numpy() - ref) <= 2.0 ** -24 * np.abs(ref) + 1e-12 * mag + 1e-45)
+    w = rng.standard_normal((len(tracks), ns)).astype(np.float32)
+    w[0, 0] = 0.0
+    g = torch.empty((29, 37), dtype=torch.float32, device="cuda")
+    ml.ml_map_light_curves_backward(torch.as_tensor(w).cuda(), tracks, ns, sigma, g)
+    for _ in range(6):
+        # <J e, w> = <e, J^T w> on maps of a few random pixels
+        e = np.zeros((29, 37))
+        at = rng.integers(0, 29), rng.integers(0, 37)
+        e[at] = 1.0
+        col = _corner_sums(e, tracks, ns, sigma)
+        assert abs(g.cpu().numpy()[at] - (col * w).sum()) <= 2.0 ** -24 * (w.size + 3) * (col * np.abs(w)).sum() + 1e-45
+
+
+def test_light_curves_of_large_counts_and_unusual_maps(ml):
+    """Counts up to 2^32 - 1 (beyond 2^24 a float drops bits), and infinities,
+    NaN and values near the FP32 range's ends in a float map: as the corner
+    sums in FP64 give them."""
+    import torch
+    rng = np.random.default_rng(8)
+    tracks = np.array([[2.0, 2.0, 18.0, 14.0], [10.5, 1.5, 10.5, 14.5]])
+    w = inputs.Workload("counts", inputs.LensField(np.zeros(0), np.zeros(0), np.zeros(0)), 0.25, 0.25, 0.0,
+                        (0.0, 0.0, 100.0), (-1.0, -1.0, 1.0, 1.0), (20, 16), ray_box=(-2.0, -1.5, 2.0, 1.5),
+                        ray_n=(64, 48))
+    f = ml.Field(w, precision=ml.PREC_DIRECT64)
+    n = rng.integers(0, 2 ** 32, (16, 20)).astype(np.uint32)
+    n[5:9, 5:9] = rng.integers(0, 1 << 23, (4, 4))
+    ml.ml_field_set_counts(f.h, torch.as_tensor(n.view(np.int32)).cuda())
+    got = f.light_curves(tracks, 30, 0.7).cpu().numpy()
+    ref = _corner_sums(n.astype(np.float64), tracks, 30, 0.7) * f.info["mu_per_count"]
+    assert np.all(np.abs(got - ref) <= 2.0 ** -23 * np.abs(ref))
+    f.close()
+    for value in (np.inf, -np.inf, np.nan, 3e38, 1e-40, 2e-38):
+        mu = np.full((16, 20), value if abs(value) < 1e-30 else 1.0, np.float32)
+        mu[7, 10] = value
+        out = torch.empty((2, 30), dtype=torch.float32, device="cuda")
+        ml.ml_map_light_curves(torch.as_tensor(mu).cuda(), tracks, 30, 0.7, out)
+        with np.errstate(over="ignore"):
+            ref = _corner_sums(mu.astype(np.float64), tracks, 30, 0.7).astype(np.float32)
+        assert np.allclose(out.cpu().numpy(), ref, rtol=2.0 ** -22, atol=3e-45, equal_nan=True), value
+
+
 def test_light_curve_adjoint_is_the_transpose_of_the_oracle_operator(ml):
     """Brute force: the oracle's light-curve operator J (samples x pixels),
     column by column on unit maps; the GPU backward must return J^T w."""
