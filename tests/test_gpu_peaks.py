@@ -43,6 +43,40 @@ def test_synthetic_ridges_match_oracle(ml, along):
     f.close()
 
 
+@pytest.mark.parametrize("along", ["x", "y"])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (3, 3), (4, 2), (120, 33), (121, 8), (124, 9), (119, 70), (244, 31), (2, 300)])
+def test_peaks_at_strip_edges_match_oracle(ml, nx, ny, along):
+    """Maps around the kernel's strips of 120 columns and groups of 8 rows, of
+    widths that are and are not multiples of four, dense in ridges, with counts
+    from 0 to 2^25 and pixels exactly at the threshold."""
+    import torch
+    rng = np.random.default_rng(nx * 1000 + ny)
+    N = rng.integers(0, 3, (ny, nx)).astype(np.int64) * 40 + rng.integers(0, 9, (ny, nx))
+    N[:, ::5] += 300 * (rng.random((ny, (nx + 4) // 5)) < 0.7)
+    N[::4] += 300 * (rng.random(((ny + 3) // 4, nx)) < 0.4)
+    N[rng.random((ny, nx)) < 0.05] *= 1 << 16
+    if nx >= 3 and ny >= 3:
+        N[1, :3], N[:3, 1] = (0, 75, 0), (0, 75, 0)      # h^2 = 25 <N> exactly: (150)^2 = 75 * 300
+    f = _blank_field(ml, nx, ny)
+    ml.ml_field_set_counts(f.h, torch.as_tensor(N.astype(np.int32)).cuda())
+    a = ml.ALONG_X if along == "x" else ml.ALONG_Y
+    for nsigma in (5.0, 10.0, 0.5):
+        n, peaks, m = _gpu_peaks(ml, f, a, nsigma=nsigma, capacity=nx * ny)
+        ref = oracle.peaks(N, along, nsigma=nsigma)
+        assert np.array_equal(m, ref)
+        assert n == int((ref & 2).astype(bool).sum()) == len(peaks)
+        assert {tuple(p) for p in peaks} == {(x, y) for y, x in zip(*np.nonzero(ref & 2))}
+    edges = np.linspace(0.0, 3.0, 8)
+    got = ml.ml_peak_statistics(f.h, edges, a, 0.0, nsigma=0.5)
+    g = oracle.geometry_of(inputs.Workload("blank", inputs.LensField(np.zeros(0), np.zeros(0), np.zeros(0)), 0.25, 0.25,
+                                           0.0, (0.0, 0.0, 100.0), (-1.0, -1.0, 1.0, 1.0), (nx, ny),
+                                           ray_box=(-2.0, -1.5, 2.0, 1.5), ray_n=(64, 48)))
+    want = oracle.peak_statistics(N, ref, along, *_axis(g, along), 0.0, edges)
+    for x, y in zip(got, want):
+        assert np.array_equal(x, np.asarray(y).astype(np.uint64))
+    f.close()
+
+
 def test_peaks_of_a_shot_map_match_oracle(ml):
     """A fold-model map shot on the GPU: its own count map through both
     implementations (the oracle reads the GPU's counts: the check is of the
