@@ -382,11 +382,10 @@ double ray_cost_ps(int P, double near_per_ray)
     return (1.0 - f) * cost_row(r, q) + f * cost_row(r + 1, q);
 }
 // Field build, nanoseconds: per level-2 node and coefficient, and per
-// level-1 cell (truncation bound, box and sub-block series); measured as the
-// create time's growth with the node count at a fixed order and with the
-// level-1 cell count (paper-scale map and the Table-1 fold field alike).
-constexpr double kNodeCostNs = 0.12;
-constexpr double kCellCostNs = 400.0;
+// level-1 cell (truncation bound, box and sub-block series), from the Table-1
+// field's kernels (10.9M nodes of order 4 in 1.16 ms; 54,579 cells in 5.5 ms).
+constexpr double kNodeCostNs = 0.022;
+constexpr double kCellCostNs = 100.0;
 
 struct GridChoice {
     int sx = 20, sy = 20, p = 0;
@@ -899,27 +898,25 @@ ml_status create_finish(ml_field *f, int p, cudaStream_t s, bool sync = true)
         f->far_bound = f->worst[p - 1];
         const LensTable L = f->table();
         const int64_t nodes = g.N2x * g.N2y;
-        ML_CK(f->alloc(&f->d_coef64, (size_t)nodes * (p + 1) * 2, s));
-        f->build_used = ML_BUILD_DIRECT;
-        bool done = false;
-        if (d->build != ML_BUILD_DIRECT) {
-            size_t ns = hier_scratch_doubles(g);
-            if (ns > 0) {
-                double *scratch = nullptr;
-                ML_CK(ml_malloc_async((void **)&scratch, ns * sizeof(double), s));
-                cudaError_t e = launch_coeffs_hier(g, L, f->d_coef64, scratch, ns, s);
-                cudaFreeAsync(scratch, s);
-                if (e != cudaSuccess) return cuda_fail(e, "hierarchical coefficient build");
-                f->build_used = ML_BUILD_HIERARCHICAL;
-                done = true;
-            } else if (d->build == ML_BUILD_HIERARCHICAL) {
-                return fail(ML_ERR_UNSUPPORTED, "hierarchical build not available");
-            }
-        }
-        if (!done) ML_CK(launch_coeffs_direct(g, L, f->d_coef64, s));
-        if (d->precision == ML_PREC_MIXED) {
-            ML_CK(f->alloc(&f->d_nodes, (size_t)nodes * node_stride(p), s));
-            ML_CK(launch_node_finalize(g, f->d_coef64, f->d_nodes, s));
+        const bool mixed = d->precision == ML_PREC_MIXED;
+        const size_t ns = d->build != ML_BUILD_DIRECT ? hier_scratch_doubles(g) : 0;
+        if (ns == 0 && d->build == ML_BUILD_HIERARCHICAL)
+            return fail(ML_ERR_UNSUPPORTED, "hierarchical build not available");
+        // FP64 coefficients: the near/far mode's, and the direct build's on its
+        // way to the mixed mode's records
+        if (!mixed || ns == 0) ML_CK(f->alloc(&f->d_coef64, (size_t)nodes * (p + 1) * 2, s));
+        if (mixed) ML_CK(f->alloc(&f->d_nodes, (size_t)nodes * node_stride(p), s));
+        if (ns > 0) {
+            double *scratch = nullptr;
+            ML_CK(ml_malloc_async((void **)&scratch, ns * sizeof(double), s));
+            cudaError_t e = launch_coeffs_hier(g, L, f->d_coef64, f->d_nodes, scratch, ns, s);
+            cudaFreeAsync(scratch, s);
+            if (e != cudaSuccess) return cuda_fail(e, "hierarchical coefficient build");
+            f->build_used = ML_BUILD_HIERARCHICAL;
+        } else {
+            ML_CK(launch_coeffs_direct(g, L, f->d_coef64, s));
+            if (mixed) ML_CK(launch_node_finalize(g, f->d_coef64, f->d_nodes, s));
+            f->build_used = ML_BUILD_DIRECT;
         }
     } else {
         g.p = 0;
@@ -980,7 +977,10 @@ ml_status measure_grid(const ml_field_desc &d, const std::vector<double> &hx, co
         // cancels a launch's fixed start and tail
         const Geo &g = f->g;
         const uint64_t total = (uint64_t)g.n3x * (uint64_t)g.n3y;
-        const uint64_t n = std::min<uint64_t>(total / 2, std::max<uint64_t>(500000000ull, total / 100));
+        // (long enough that a launch's start and tail, some tens of microseconds,
+        // stay a few per cent of it)
+        const uint64_t n = std::min<uint64_t>(total / 2, std::max<uint64_t>({500000000ull, total / 100,
+                                                                             std::min<uint64_t>(total / 32, 4000000000ull)}));
         const uint64_t r0 = (total - 2 * n) / 2;
         const uint64_t warm = std::min<uint64_t>(n, 64ull * (uint64_t)g.n3x);
         // the certified walk is timed with lens columns spanned beyond five

@@ -296,11 +296,11 @@ __global__ void __launch_bounds__(ML_PB_THREADS) k_p_bound(Geo g, LensTable L, d
         // extended ids of the near block: rows c1y..c1y+2, columns c1x..c1x+2
         n0[i] = (int32_t)(c1y * g.NEx + c1x);
     }
-    float acc[PB_CELLS][PMAX];
+    f32x2 acc[PB_CELLS][PMAX / 2];         // orders in pairs, two-lane instructions
 #pragma unroll
     for (int i = 0; i < PB_CELLS; ++i)
 #pragma unroll
-        for (int q = 0; q < PMAX; ++q) acc[i][q] = 0.f;
+        for (int q = 0; q < PMAX / 2; ++q) acc[i][q] = 0;
     for (int64_t k = threadIdx.x; k < L.n; k += blockDim.x) {
         const int32_t cell = L.cell[k];
         const float xh = L.xh[k], xl = L.xl[k], yh = L.yh[k], yl = L.yl[k], mf = L.mf[k];
@@ -313,15 +313,18 @@ __global__ void __launch_bounds__(ML_PB_THREADS) k_p_bound(Geo g, LensTable L, d
             const float D = __fmul_rn(sqrt_approx(__fmaf_rn(dx, dx, __fmul_rn(dy, dy))), 1.f - 1e-6f);
             if (D <= rho) {
 #pragma unroll
-                for (int q = 0; q < PMAX; ++q) acc[i][q] = INFINITY;
+                for (int q = 0; q < PMAX / 2; ++q) acc[i][q] = pack2(INFINITY, INFINITY);
                 continue;
             }
             const float u = __fmul_rn(rho, rcp_approx(D));
-            float t = __fmul_rn(__fmul_rn(mf, u), rcp_approx(__fsub_rn(D, rho)));  // times u^{p} below
+            const float t1 = __fmul_rn(__fmul_rn(__fmul_rn(mf, u), rcp_approx(__fsub_rn(D, rho))), u);
+            const float u2 = __fmul_rn(u, u);
+            f32x2 t = pack2(t1, __fmul_rn(t1, u));
+            const f32x2 uu = pack2(u2, u2);
 #pragma unroll
-            for (int q = 0; q < PMAX; ++q) {
-                t = __fmul_rn(t, u);
-                acc[i][q] = __fadd_rn(acc[i][q], t);
+            for (int q = 0; q < PMAX / 2; ++q) {
+                acc[i][q] = add2(acc[i][q], t);
+                t = mul2(t, uu);
             }
         }
     }
@@ -331,7 +334,9 @@ __global__ void __launch_bounds__(ML_PB_THREADS) k_p_bound(Geo g, LensTable L, d
     for (int i = 0; i < PB_CELLS; ++i)
 #pragma unroll
         for (int q = 0; q < PMAX; ++q) {
-            float v = acc[i][q];
+            float a0, a1;
+            unpack2(acc[i][q / 2], a0, a1);
+            float v = q & 1 ? a1 : a0;
             for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
             if (lane == 0) red[i][q][wid] = v;
         }
@@ -509,6 +514,20 @@ struct BinomTableF {
 };
 __constant__ BinomTableF c_binomf = BinomTableF();
 
+// The exact table as hi + lo floats, in global memory (coalesced, as g_binom).
+struct BinomTableDf {
+    float2 v[(HP + 1) * (HP + 1)];
+    constexpr BinomTableDf() : v()
+    {
+        BinomTable b;
+        for (int i = 0; i < (HP + 1) * (HP + 1); ++i) {
+            v[i].x = (float)b.v[i];
+            v[i].y = (float)(b.v[i] - (double)v[i].x);
+        }
+    }
+};
+__device__ BinomTableDf g_binomdf = BinomTableDf();
+
 struct Hier {
     int64_t bxn, byn;                // level-1 cells per box side
     int64_t NBx, NBy;                // boxes across the level-1 grid
@@ -581,6 +600,144 @@ __device__ __forceinline__ void p2l_add(double m, double dx, double dy, double h
     }
 }
 
+// ---- the same sums in hi + lo floats -----------------------------------------
+//
+// The mixed mode rounds c_1..c_p and the node's position within its pixel to
+// FP32, so its series need not be carried in FP64, whose rate here is 1/64 of
+// FP32's: they run in pairs of floats (unevaluated sums h + l, about 46 bits;
+// Dekker 1971, Knuth's two-sum).  Orders HD and above are plain FP32: a lens's
+// term of order j is |w|^j < 0.6^j of its leading one, so their rounding is
+// below 2^-24 0.6^HD = 1.3e-10 of the nearest lenses' leading terms, 1e-8 of a
+// pixel at the tuned grids.  The FP64 near/far mode keeps the FP64 sums.
+constexpr int HD = 12;               // orders carried in pairs
+
+struct df {
+    float h, l;
+};
+
+__device__ __forceinline__ df df_of(double v)
+{
+    df r;
+    r.h = (float)v;
+    r.l = (float)(v - (double)r.h);
+    return r;
+}
+
+__device__ __forceinline__ df df_renorm(float s, float e)       // |e| <= |s| / 2 or so
+{
+    df r;
+    r.h = __fadd_rn(s, e);
+    r.l = __fsub_rn(e, __fsub_rn(r.h, s));
+    return r;
+}
+
+__device__ __forceinline__ void df_sum2(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+__device__ __forceinline__ df df_add(df a, df b)
+{
+    float s, e;
+    df_sum2(a.h, b.h, s, e);
+    return df_renorm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+
+__device__ __forceinline__ df df_neg(df a) { return df{-a.h, -a.l}; }
+
+// product as p + e without renormalisation
+__device__ __forceinline__ void df_prod(df a, df b, float &p, float &e)
+{
+    p = __fmul_rn(a.h, b.h);
+    e = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)));
+}
+
+__device__ __forceinline__ df df_mul(df a, df b)
+{
+    float p, e;
+    df_prod(a, b, p, e);
+    return df_renorm(p, e);
+}
+
+// a b + c d
+__device__ __forceinline__ df df_dot2(df a, df b, df c, df d)
+{
+    float p, e, q, f, s, t;
+    df_prod(a, b, p, e);
+    df_prod(c, d, q, f);
+    df_sum2(p, q, s, t);
+    return df_renorm(s, __fadd_rn(t, __fadd_rn(e, f)));
+}
+
+// p2l_add on pairs: dx, dy the lens's offset from the expansion's centre, h the
+// scale, ih = 1/h.
+struct PairSums {
+    df r[HD], i[HD];                 // orders 0..HD-1
+    float fr[HP + 1 - HD], fi[HP + 1 - HD];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int j = 0; j < HD; ++j) r[j] = i[j] = df{0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j <= HP - HD; ++j) fr[j] = fi[j] = 0.f;
+    }
+};
+
+__device__ __forceinline__ void p2l_add_df(double m, df dx, df dy, df h, df ih, PairSums &a)
+{
+    const df r2 = df_dot2(dx, dx, dy, dy);
+    df inv;                                            // h / r^2
+    if (r2.h > 1e-30f && r2.h < 1e30f) {
+        // reciprocal by one third-order Newton step on the residual
+        const float y = rcp_approx(r2.h);
+        const float e = __fmaf_rn(-r2.l, y, __fmaf_rn(-r2.h, y, 1.f));
+        inv = df_mul(h, df_renorm(y, __fmul_rn(y, __fmaf_rn(e, e, e))));
+    } else {
+        const double x = (double)dx.h + (double)dx.l, z = (double)dy.h + (double)dy.l;
+        inv = df_of(((double)h.h + (double)h.l) / (x * x + z * z));
+    }
+    const df wr = df_mul(dx, inv), wi = df_neg(df_mul(dy, inv));
+    const float lw = __logf(h.h * inv.h);
+    const int J = lw < -74.0f / (float)(HP + 1) ? (int)(-74.0f / lw) : HP;
+    const df mh = df_mul(df_of(m), ih);
+    df tr = df_neg(df_mul(mh, wr)), ti = df_neg(df_mul(mh, wi));
+#pragma unroll
+    for (int j = 0; j < HD; ++j) {
+        if (j > J) return;
+        float s, e;
+        df_sum2(a.r[j].h, tr.h, s, e);
+        a.r[j].h = s;
+        a.r[j].l = __fadd_rn(a.r[j].l, __fadd_rn(e, tr.l));
+        df_sum2(a.i[j].h, ti.h, s, e);
+        a.i[j].h = s;
+        a.i[j].l = __fadd_rn(a.i[j].l, __fadd_rn(e, ti.l));
+        const df nr = df_dot2(tr, wr, df_neg(ti), wi);
+        ti = df_dot2(tr, wi, ti, wr);
+        tr = nr;
+    }
+    float fr = tr.h, fi = ti.h;
+    const float vr = wr.h, vi = wi.h;
+#pragma unroll
+    for (int j = HD; j <= HP; ++j) {
+        if (j > J) return;
+        a.fr[j - HD] += fr;
+        a.fi[j - HD] += fi;
+        const float nr = __fmaf_rn(fr, vr, -(fi * vi));
+        fi = __fmaf_rn(fr, vi, fi * vr);
+        fr = nr;
+    }
+}
+
+// Offset of a lens from a centre z, from the lens's own hi + lo copy.
+__device__ __forceinline__ df lens_offset(float h, float l, df z)
+{
+    float s, e;
+    df_sum2(h, -z.h, s, e);
+    return df_renorm(s, __fadd_rn(e, __fsub_rn(l, z.l)));
+}
+
 // Sum the (HP+1) complex accumulators over a warp's lanes.  Orders 0..31
 // (64 values) go through a reduce-scatter: at each of five steps a lane keeps
 // the half of its values that its lane bit selects, sends the other half to
@@ -618,6 +775,40 @@ __device__ __forceinline__ void warp_sum_orders(const double *ar, const double *
     for (int o = 16; o > 0; o >>= 1) {
         xr += __shfl_xor_sync(0xffffffffu, xr, o);
         xi += __shfl_xor_sync(0xffffffffu, xi, o);
+    }
+}
+
+// warp_sum_orders on pairs.
+__device__ __forceinline__ void warp_sum_orders_df(const PairSums &a, df &sr, df &si, df &xr, df &xi)
+{
+    const int lane = threadIdx.x & 31;
+    df v[64];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        v[2 * j] = j < HD ? a.r[j < HD ? j : 0] : df{a.fr[j < HD ? 0 : j - HD], 0.f};
+        v[2 * j + 1] = j < HD ? a.i[j < HD ? j : 0] : df{a.fi[j < HD ? 0 : j - HD], 0.f};
+    }
+#pragma unroll
+    for (int st = 0; st < 5; ++st) {
+        const int o = 16 >> st, half = 32 >> st;
+        const bool upper = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const df lo = v[i], hi = v[i + half];
+            df send = upper ? lo : hi;
+            const df keep = upper ? hi : lo;
+            send.h = __shfl_xor_sync(0xffffffffu, send.h, o);
+            send.l = __shfl_xor_sync(0xffffffffu, send.l, o);
+            v[i] = df_add(keep, send);
+        }
+    }
+    sr = v[0];
+    si = v[1];
+    xr = df{a.fr[HP - HD], 0.f};
+    xi = df{a.fi[HP - HD], 0.f};
+    for (int o = 16; o > 0; o >>= 1) {
+        xr.h += __shfl_xor_sync(0xffffffffu, xr.h, o);
+        xi.h += __shfl_xor_sync(0xffffffffu, xi.h, o);
     }
 }
 
@@ -816,6 +1007,310 @@ __global__ void __launch_bounds__(32 * SUB_WARPS, 3) k_sub_p2l(Geo g, LensTable 
     }
 }
 
+// ---- the mixed mode's build on pairs of floats --------------------------------
+
+// 1. box series (k_box_p2l; 2.16 -> 0.65 ms on the Table-1 field).
+__global__ void __launch_bounds__(128) k_box_p2l_df(Geo g, LensTable L, const int2 *__restrict__ lc, Hier h,
+                                                    float4 *__restrict__ part)
+{
+    __shared__ float4 red[4 * (HP + 1)];
+    const int64_t b = blockIdx.x, Bx = b % h.NBx, By = b / h.NBx;
+    const df zx = df_of(g.rx0 + ((double)Bx + 0.5) * (double)h.bxn * g.l1x);
+    const df zy = df_of(g.ry0 + ((double)By + 0.5) * (double)h.byn * g.l1y);
+    const df hB = df_of(h.hB), ihB = df_of(1.0 / h.hB);
+    PairSums acc;
+    acc.zero();
+    const int64_t k0 = L.n * blockIdx.y / HPARTS, k1 = L.n * (blockIdx.y + 1) / HPARTS;
+    const int bxn = (int)h.bxn, byn = (int)h.byn, iBx = (int)Bx, iBy = (int)By;
+    for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
+        const int2 c = lc[k];
+        const int dx = (int)floor_div(c.x, bxn) - iBx, dy = (int)floor_div(c.y, byn) - iBy;
+        if (dx <= 1 && dx >= -1 && dy <= 1 && dy >= -1) continue;
+        p2l_add_df(L.m[k], lens_offset(L.xh[k], L.xl[k], zx), lens_offset(L.yh[k], L.yl[k], zy), hB, ihB, acc);
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    df sr, si, xr, xi;
+    warp_sum_orders_df(acc, sr, si, xr, xi);
+    red[wid * (HP + 1) + lane] = make_float4(sr.h, sr.l, si.h, si.l);
+    if (lane == 0) red[wid * (HP + 1) + HP] = make_float4(xr.h, xr.l, xi.h, xi.l);
+    __syncthreads();
+    for (int j = threadIdx.x; j <= HP; j += blockDim.x) {
+        df vr{0.f, 0.f}, vi{0.f, 0.f};
+        for (int w = 0; w < nw; ++w) {
+            const float4 q = red[w * (HP + 1) + j];
+            vr = df_add(vr, df{q.x, q.y});
+            vi = df_add(vi, df{q.z, q.w});
+        }
+        part[(b * HPARTS + blockIdx.y) * (HP + 1) + j] = make_float4(vr.h, vr.l, vi.h, vi.l);
+    }
+}
+
+// 2. sub-block series (k_sub_p2l): sub = (re, im) rounded to FP32, sublo their
+// remainders, j64 the length of c_0's pair sum.  One warp per sub-block: the
+// FP64 form took 9.5 ms for the Table-1 field's 54,579 sub-blocks (about 175
+// lenses each), bound by the FP64 pipe; all orders in pairs 4.8 ms (two warps
+// per scheduler by its registers), HD orders in pairs 2.0 ms, bound by issue.
+__global__ void __launch_bounds__(32 * SUB_WARPS, 3) k_sub_p2l_df(Geo g, LensTable L, const int2 *__restrict__ lc,
+                                                             Hier h, const float4 *__restrict__ part,
+                                                             const int32_t *__restrict__ ostart,
+                                                             const int32_t *__restrict__ oidx,
+                                                             float2 *__restrict__ sub, float2 *__restrict__ sublo,
+                                                             int32_t *__restrict__ j64, int64_t ns)
+{
+    __shared__ float4 shA[SUB_WARPS][HP + 1];
+    __shared__ float shR[SUB_WARPS][HP + 1];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t s = (int64_t)blockIdx.x * SUB_WARPS + wid;
+    if (s >= ns) return;                     // warp-uniform; the kernel has no block barrier
+    float4 *A = shA[wid];
+    float *red = shR[wid];
+    const int64_t nsub = h.nsx * h.nsy;
+    const int64_t cell = s / nsub, sb = s % nsub;
+    const int64_t cx = cell % g.N1x, cy = cell / g.N1x;
+    const int64_t sa = sb % h.nsx, sbb = sb / h.nsx;
+    // node columns [ua, ub) and rows [va, vb) of the sub-block inside the cell
+    const int64_t ua = (sa * g.l2sx + h.nsx - 1) / h.nsx, ub = ((sa + 1) * g.l2sx + h.nsx - 1) / h.nsx;
+    const int64_t va = (sbb * g.l2sy + h.nsy - 1) / h.nsy, vb = ((sbb + 1) * g.l2sy + h.nsy - 1) / h.nsy;
+    const double zx = g.rx0 + (double)cx * g.l1x + 0.5 * (double)(ua + ub) * g.l2x;
+    const double zy = g.ry0 + (double)cy * g.l1y + 0.5 * (double)(va + vb) * g.l2y;
+    const double hs = 0.5 * sqrt((double)((ub - ua) * (ub - ua)) * g.l2x * g.l2x +
+                                 (double)((vb - va) * (vb - va)) * g.l2y * g.l2y);
+    const double ihs = 1.0 / hs;
+    const int64_t Bx = cx / h.bxn, By = cy / h.byn;
+    const df cxd = df_of(zx), cyd = df_of(zy), hsd = df_of(hs), ihsd = df_of(ihs);
+    PairSums acc;
+    acc.zero();
+    // lenses of the box block (3 x 3 boxes) outside the cell's 3 x 3 block.
+    // Cells of the binning grid (the lattice and its ring) are contiguous
+    // runs of the sorted table, one per row; lenses beyond the ring (the last
+    // bucket) are scanned only when the box block reaches past the ring.
+    const int64_t xlo = (Bx - 1) * h.bxn, xhi = (Bx + 2) * h.bxn - 1;
+    const int64_t ylo = (By - 1) * h.byn, yhi = (By + 2) * h.byn - 1;
+    const int64_t rx0 = max(xlo, (int64_t)-1), rx1 = min(xhi, g.N1x);
+    const int64_t ry0 = max(ylo, (int64_t)-1), ry1 = min(yhi, g.N1y);
+    for (int64_t ry = ry0; ry <= ry1 && rx0 <= rx1; ++ry) {
+        const int64_t b0 = (ry + 1) * g.NEx + (rx0 + 1), b1 = (ry + 1) * g.NEx + (rx1 + 1);
+        const int64_t k0 = L.start[b0], k1 = L.start[b1 + 1];
+        const bool near_row = ry - cy <= 1 && cy - ry <= 1;
+        for (int64_t k = k0 + lane; k < k1; k += 32) {
+            if (near_row) {
+                const int64_t lx = lc[k].x;
+                if (lx - cx <= 1 && cx - lx <= 1) continue;
+            }
+            p2l_add_df(L.m[k], lens_offset(L.xh[k], L.xl[k], cxd), lens_offset(L.yh[k], L.yl[k], cyd), hsd, ihsd, acc);
+        }
+    }
+    if (xlo < -1 || xhi > g.N1x || ylo < -1 || yhi > g.N1y) {
+        const int64_t obx = h.NBx + 2;
+        for (int64_t by = By - 1; by <= By + 1; ++by) {
+            const int64_t b0 = (by + 1) * obx + Bx;          // bins of boxes Bx-1..Bx+1
+            for (int64_t q = ostart[b0] + lane; q < ostart[b0 + 3]; q += 32) {
+                const int32_t k = oidx[q];
+                p2l_add_df(L.m[k], lens_offset(L.xh[k], L.xl[k], cxd), lens_offset(L.yh[k], L.yl[k], cyd), hsd, ihsd, acc);
+            }
+        }
+    }
+    // box series of this cell's box: sum of the partitions (fixed order)
+    const int64_t b = By * h.NBx + Bx;
+    for (int j = lane; j <= HP; j += 32) {
+        df vr{0.f, 0.f}, vi{0.f, 0.f};
+        for (int q = 0; q < HPARTS; ++q) {
+            const float4 v = part[(b * HPARTS + q) * (HP + 1) + j];
+            vr = df_add(vr, df{v.x, v.y});
+            vi = df_add(vi, df{v.z, v.w});
+        }
+        A[j] = make_float4(vr.h, vr.l, vi.h, vi.l);
+    }
+    // the direct sums: lane j holds order j, every lane order HP
+    df sr, si, xr, xi;
+    warp_sum_orders_df(acc, sr, si, xr, xi);
+    __syncwarp();
+    // shift the box series to z_s (as k_sub_p2l): rho^j sum_{i>=j} C(i, j) A_i d^{i-j}
+    const double zBx = g.rx0 + ((double)Bx + 0.5) * (double)h.bxn * g.l1x;
+    const double zBy = g.ry0 + ((double)By + 0.5) * (double)h.byn * g.l1y;
+    const df dr = df_of((zx - zBx) / h.hB), di = df_of((zy - zBy) / h.hB), rho = df_of(hs / h.hB);
+    for (int j = lane; j <= HP; j += 32) {
+        float wr = 0.f, wi = 0.f;
+        int i = HP;
+        for (; i >= HD && i >= j; --i) {     // Horner in d: FP32 orders, then pairs
+            const float c = g_binomdf.v[i * (HP + 1) + j].x;
+            const float4 q = A[i];
+            const float nr = __fmaf_rn(wr, dr.h, __fmaf_rn(-wi, di.h, c * q.x));
+            wi = __fmaf_rn(wr, di.h, __fmaf_rn(wi, dr.h, c * q.z));
+            wr = nr;
+        }
+        df vr{wr, 0.f}, vi{wi, 0.f};
+        for (; i >= j; --i) {
+            const float2 cb = g_binomdf.v[i * (HP + 1) + j];
+            const float4 q = A[i];
+            const df c{cb.x, cb.y};
+            const df nr = df_add(df_dot2(vr, dr, df_neg(vi), di), df_mul(c, df{q.x, q.y}));
+            vi = df_add(df_dot2(vr, di, vi, dr), df_mul(c, df{q.z, q.w}));
+            vr = nr;
+        }
+        df sc{1.f, 0.f}, rp = rho;           // rho^j by squaring
+        for (int e = j; e > 0; e >>= 1, rp = df_mul(rp, rp))
+            if (e & 1) sc = df_mul(sc, rp);
+        const df fr = df_add(j == HP ? xr : sr, df_mul(vr, sc));
+        const df fi = df_add(j == HP ? xi : si, df_mul(vi, sc));
+        sub[s * (HP + 1) + j] = make_float2(fr.h, fi.h);
+        sublo[s * (HP + 1) + j] = make_float2(fr.l, fi.l);
+        red[j] = fabsf(fr.h) + fabsf(fi.h);
+        if (j == 0) A[0] = make_float4(fr.h, fr.l, fi.h, fi.l);
+    }
+    __syncwarp();
+    // length of the node's c_0 sum in pairs: the orders above j64 add up (in
+    // |re| + |im|) to at most 2^-35 max(|re a_0|, |im a_0|), so their FP32 sum
+    // (error below 2^-19 of that, |e| <= 1) stays under 2^-54 of c_0
+    if (lane == 0) {
+        const float lim = 2.9e-11f * fmaxf(fabsf(A[0].x), fabsf(A[0].z));
+        float tail = 0.f;
+        int J = HP;
+        while (J > 0 && tail + red[J] <= lim) tail += red[J--];
+        j64[s] = J;
+    }
+}
+
+// Scales of a node's shift, which depend on its sub-block's node counts along x
+// and y only (the quotient of the cells per side, rounded down or up): e per
+// half node step, (l3x / hs)^n.
+struct ShiftScale {
+    float kxh, kxl, kyh, kyl;        // l2x / hs, l2y / hs
+    float sh[PMAX], sl[PMAX];        // (l3x / hs)^n, n = 1..p
+};
+
+// Everything of a node's smooth position that does not depend on the node, in
+// pixels: beta_x = x0 + x1 zx + x2 zx^2 + xy zx zy, beta_y = y0 + y1 zy (macro
+// model and sheet; z the node), slope and per-row shift as in k_node_finalize.
+struct NodeMap {
+    double x0, x1, x2, xy, y0, y1, ipx, ipy;
+    double ax0, ax1, ax2, bq1;
+    int wx, wy;                      // smaller node count of a sub-block along x and y
+    ShiftScale sc[4];                // [2 (height - wy) + width - wx]
+};
+
+// 3. node records from the sub-block series, in one pass (the FP64 form shifts
+// to coefficients in memory first, which k_node_finalize reads again).  c_1..c_p
+// are the same FP32 sums as k_node_shift's; c_0 sums pairs up to order j64.  A
+// block's records are staged in shared memory and stored 16 bytes at a time.
+// The FP64 form took 4.4 + 2.0 ms for the Table-1 field's 10.9M nodes, this 1.16 ms.
+template <int P>
+__global__ void __launch_bounds__(128) k_node_records(Geo g, Hier h, const float2 *__restrict__ sub,
+                                                      const float2 *__restrict__ sublo,
+                                                      const int32_t *__restrict__ j64, const __grid_constant__ NodeMap nm,
+                                                      unsigned char *__restrict__ out)
+{
+    constexpr int STRIDE = 24 + 8 * P;
+    __shared__ __align__(16) unsigned char rec_s[128 * STRIDE];
+    const float *binomf = c_binomf.v;
+    const int64_t nn = g.N2x * g.N2y, node0 = blockIdx.x * (int64_t)128, node = node0 + threadIdx.x;
+    if (node < nn) {
+        const int64_t c2y64 = node / g.N2x;
+        const int c2x = (int)(node - c2y64 * g.N2x), c2y = (int)c2y64;
+        const int l2sx = g.l2sx, l2sy = g.l2sy, nsx = (int)h.nsx, nsy = (int)h.nsy;
+        const int cx = c2x / l2sx, cy = c2y / l2sy;
+        const int u = c2x - cx * l2sx, v = c2y - cy * l2sy;
+        const int sa = u * nsx / l2sx, sbb = v * nsy / l2sy;
+        const int ua = (sa * l2sx + nsx - 1) / nsx, ub = ((sa + 1) * l2sx + nsx - 1) / nsx;
+        const int va = (sbb * l2sy + nsy - 1) / nsy, vb = ((sbb + 1) * l2sy + nsy - 1) / nsy;
+        const int which = 2 * (vb - va - nm.wy) + (ub - ua - nm.wx);
+        const ShiftScale &sc = nm.sc[which];
+        // e = (z_node - z_s)/hs: a half-integer number of node steps
+        const float qx = (float)u + 0.5f - 0.5f * (float)(ua + ub), qy = (float)v + 0.5f - 0.5f * (float)(va + vb);
+        const df er = df_mul(df{qx, 0.f}, df{sc.kxh, sc.kxl}), ei = df_mul(df{qy, 0.f}, df{sc.kyh, sc.kyl});
+        const int64_t s = ((int64_t)cy * g.N1x + cx) * (nsx * nsy) + sbb * nsx + sa;
+        const float2 *af = sub + s * (HP + 1), *al = sublo + s * (HP + 1);
+        const float erf = er.h, eif = ei.h;
+        df c0r, c0i;
+        {
+            const int J = j64[s];
+            float tr = 0.f, ti = 0.f;
+            for (int j = HP; j > J; --j) {
+                const float2 q = af[j];
+                const float nr = __fmaf_rn(tr, erf, __fmaf_rn(-ti, eif, q.x));
+                const float ni = __fmaf_rn(tr, eif, __fmaf_rn(ti, erf, q.y));
+                tr = nr;
+                ti = ni;
+            }
+            df vr{tr, 0.f}, vi{ti, 0.f};
+            for (int j = J; j >= 0; --j) {
+                const float2 q = af[j], ql = al[j];
+                const df nr = df_add(df_dot2(vr, er, df_neg(vi), ei), df{q.x, ql.x});
+                vi = df_add(df_dot2(vr, ei, vi, er), df{q.y, ql.y});
+                vr = nr;
+            }
+            c0r = vr;
+            c0i = vi;
+        }
+        const double zx = g.rx0 + ((double)c2x + 0.5) * g.l2x;
+        const double zy = g.ry0 + ((double)c2y + 0.5) * g.l2y;
+        double Sx = nm.x0 + zx * (nm.x1 + nm.x2 * zx + nm.xy * zy) - ((double)c0r.h + (double)c0r.l) * nm.ipx;
+        double Sy = nm.y0 + zy * nm.y1 + ((double)c0i.h + (double)c0i.l) * nm.ipy;
+        const double fbx = fmin(fmax(floor(Sx), -16777216.0), 16777216.0);
+        const double fby = fmin(fmax(floor(Sy), -16777216.0), 16777216.0);
+        float2 *r = reinterpret_cast<float2 *>(rec_s + threadIdx.x * STRIDE);
+        r[0] = make_float2(__int_as_float((int)fby), (float)(Sy - fby));
+        r[1] = make_float2(__int_as_float((int)fbx), (float)(Sx - fbx));
+        r[2] = make_float2((float)(nm.ax0 + nm.ax1 * zx + nm.ax2 * zy), (float)(nm.bq1 * zx));
+#pragma unroll
+        for (int n = 1; n <= P; ++n) {
+            float vr = 0.f, vi = 0.f;
+            for (int j = HP; j >= n; --j) {
+                const float c = binomf[j * (HP + 1) + n];
+                const float2 q = af[j];
+                const float nr = __fmaf_rn(vr, erf, __fmaf_rn(-vi, eif, c * q.x));
+                const float ni = __fmaf_rn(vr, eif, __fmaf_rn(vi, erf, c * q.y));
+                vr = nr;
+                vi = ni;
+            }
+            const float k = sc.sh[n - 1], kl = sc.sl[n - 1];
+            r[2 + n] = make_float2(__fmaf_rn(vr, k, vr * kl), __fmaf_rn(vi, k, vi * kl));
+        }
+    }
+    __syncthreads();
+    const int64_t n16 = min((int64_t)128, nn - node0) * STRIDE;      // a multiple of 8 bytes
+    unsigned char *o = out + node0 * STRIDE;                         // 128 x STRIDE: 16-byte aligned
+    for (int64_t i = threadIdx.x * 16; i + 16 <= n16; i += 128 * 16)
+        *reinterpret_cast<float4 *>(o + i) = *reinterpret_cast<const float4 *>(rec_s + i);
+    if (threadIdx.x == 0 && (n16 & 8))
+        *reinterpret_cast<float2 *>(o + n16 - 8) = *reinterpret_cast<const float2 *>(rec_s + n16 - 8);
+}
+
+static NodeMap node_map(const Geo &g, const Hier &h)
+{
+    NodeMap m{};
+    const double ix = 1.0 / g.dpx, iy = 1.0 / g.dpy, kx = sheet_kx(g), ky = sheet_ky(g);
+    m.ipx = ix;
+    m.ipy = iy;
+    const bool fold = g.macro == ML_MACRO_FOLD;
+    const double a = fold ? 0.0 : 1.0 - g.kappa - g.gamma;
+    const double b = fold ? 2.0 * (1.0 - g.kappa0) : 1.0 - g.kappa + g.gamma;
+    m.x0 = (-kx * g.sheet_cx - g.mx0) * ix;
+    m.x1 = (a + kx) * ix;
+    m.x2 = fold ? 0.5 * g.dx * ix : 0.0;
+    m.xy = fold ? g.dy * ix : 0.0;
+    m.y0 = (-ky * g.sheet_cy - g.my0) * iy;
+    m.y1 = (b + ky) * iy;
+    // slope of the macro and sheet terms per ray column, shift per ray row
+    m.ax0 = (a + kx) * g.l3x * ix;
+    m.ax1 = fold ? g.dx * g.l3x * ix : 0.0;
+    m.ax2 = fold ? g.dy * g.l3x * ix : 0.0;
+    m.bq1 = fold ? g.dy * g.l3y * ix : 0.0;
+    m.wx = (int)(g.l2sx / h.nsx);
+    m.wy = (int)(g.l2sy / h.nsy);
+    for (int q = 0; q < 4; ++q) {
+        const double w = m.wx + (q & 1), t = m.wy + (q >> 1);
+        const double hs = 0.5 * sqrt(w * w * g.l2x * g.l2x + t * t * g.l2y * g.l2y);
+        ShiftScale &sc = m.sc[q];
+        auto split = [](double v, float &hi, float &lo) { hi = (float)v; lo = (float)(v - (double)hi); };
+        split(g.l2x / hs, sc.kxh, sc.kxl);
+        split(g.l2y / hs, sc.kyh, sc.kyl);
+        double k = 1.0;
+        for (int n = 0; n < PMAX; ++n) split(k *= g.l3x / hs, sc.sh[n], sc.sl[n]);
+    }
+    return m;
+}
+
 // 3. node coefficients from the sub-block series.  Index arithmetic in 32
 // bits (level-2 cells per level-1 side and sub-block counts are small), the
 // scales by reciprocals.
@@ -911,8 +1406,18 @@ size_t hier_scratch_doubles(const Geo &g)
     return (nb * HPARTS + ns) * (HP + 1) * 2 + (ns * (HP + 1) * 2 + 1) / 2 + (ns + 1) / 2 + 1;
 }
 
-cudaError_t launch_coeffs_hier(const Geo &g, const LensTable &L, double *coef64, double *scratch,
-                               size_t scratch_doubles, cudaStream_t s)
+template <int P>
+static void run_node_records(const Geo &g, const Hier &h, const float2 *sub, const float2 *sublo, const int32_t *j64,
+                             unsigned char *nodes, cudaStream_t s)
+{
+    const int64_t nn = g.N2x * g.N2y;
+    k_node_records<P><<<(unsigned)((nn + 127) / 128), 128, 0, s>>>(g, h, sub, sublo, j64, node_map(g, h), nodes);
+}
+
+// coef64 receives the FP64 near/far mode's coefficients, nodes the mixed
+// mode's records (the other is not used).
+cudaError_t launch_coeffs_hier(const Geo &g, const LensTable &L, double *coef64, unsigned char *nodes,
+                               double *scratch, size_t scratch_doubles, cudaStream_t s)
 {
     Hier h = hier_of(g);
     if (scratch_doubles < hier_scratch_doubles(g)) return cudaErrorInvalidValue;
@@ -933,16 +1438,30 @@ cudaError_t launch_coeffs_hier(const Geo &g, const LensTable &L, double *coef64,
     if (L.n > 0) k_lens_l1<<<(unsigned)((L.n + 255) / 256), 256, 0, s>>>(g, L, lc);
     k_outer_csr<<<1, SCAT_THREADS, 0, s>>>(lc, L.start, g.NEx * g.NEy, h, ocnt, ostart, oidx);
     dim3 gb((unsigned)nb, HPARTS);
-    k_box_p2l<<<gb, 128, 0, s>>>(g, L, lc, h, part);
-    k_sub_p2l<<<(unsigned)((ns + SUB_WARPS - 1) / SUB_WARPS), 32 * SUB_WARPS, 0, s>>>(g, L, lc, h, part, ostart,
-                                                                                  oidx, sub, sub32, j64,
-                                                                                  (int64_t)ns);
-    int64_t nn = g.N2x * g.N2y;
-    k_node_shift<<<(unsigned)((nn + 127) / 128), 128, 0, s>>>(g, h, sub, sub32, j64, coef64);
-    e = cudaGetLastError();
+    const unsigned gs = (unsigned)((ns + SUB_WARPS - 1) / SUB_WARPS);
+    if (g.precision == ML_PREC_MIXED) {
+        // the same scratch: 16 bytes per box order and partition, 8 + 8 per
+        // sub-block order
+        float4 *pt = reinterpret_cast<float4 *>(part);
+        float2 *sh = reinterpret_cast<float2 *>(sub), *sl = sh + ns * (HP + 1);
+        k_box_p2l_df<<<gb, 128, 0, s>>>(g, L, lc, h, pt);
+        k_sub_p2l_df<<<gs, 32 * SUB_WARPS, 0, s>>>(g, L, lc, h, pt, ostart, oidx, sh, sl, j64, (int64_t)ns);
+        switch (g.p) {
+#define ML_NODE_CASE(P) case P: run_node_records<P>(g, h, sh, sl, j64, nodes, s); break;
+        ML_NODE_CASE(1) ML_NODE_CASE(2) ML_NODE_CASE(3) ML_NODE_CASE(4) ML_NODE_CASE(5)
+        ML_NODE_CASE(6) ML_NODE_CASE(8) ML_NODE_CASE(10) ML_NODE_CASE(12) ML_NODE_CASE(16)
+#undef ML_NODE_CASE
+        default: e = cudaErrorInvalidValue;
+        }
+    } else {
+        k_box_p2l<<<gb, 128, 0, s>>>(g, L, lc, h, part);
+        k_sub_p2l<<<gs, 32 * SUB_WARPS, 0, s>>>(g, L, lc, h, part, ostart, oidx, sub, sub32, j64, (int64_t)ns);
+        int64_t nn = g.N2x * g.N2y;
+        k_node_shift<<<(unsigned)((nn + 127) / 128), 128, 0, s>>>(g, h, sub, sub32, j64, coef64);
+    }
+    if (e == cudaSuccess) e = cudaGetLastError();
     cudaFreeAsync(iw, s);
     return e;
 }
-
 
 }  // namespace ml

@@ -133,8 +133,8 @@ inline void set_f32(LensTable &L, const float *f32, int64_t n)
 }
 cudaError_t launch_p_bound(const Geo &g, const LensTable &L, double *bound, cudaStream_t s);
 cudaError_t launch_coeffs_direct(const Geo &g, const LensTable &L, double *coef64, cudaStream_t s);
-cudaError_t launch_coeffs_hier(const Geo &g, const LensTable &L, double *coef64, double *scratch,
-                               size_t scratch_doubles, cudaStream_t s);
+cudaError_t launch_coeffs_hier(const Geo &g, const LensTable &L, double *coef64, unsigned char *nodes,
+                               double *scratch, size_t scratch_doubles, cudaStream_t s);
 size_t hier_scratch_doubles(const Geo &g);
 cudaError_t launch_node_finalize(const Geo &g, const double *coef64, unsigned char *nodes,
                                  cudaStream_t s);

@@ -358,6 +358,31 @@ def test_certified_walk_equals_per_ray_walk(ml, case):
     fp.close()
 
 
+@pytest.mark.parametrize("l1,l2_sub,p", [((6.0, 6.0), (20, 20), 0), ((9.0, 2.0), (10, 7), 0), ((2.0, 7.0), (5, 11), 0),
+                                         ((5.0, 4.0), (3, 1), 16), ((4.0, 4.0), (1, 1), 12), ((3.0, 3.0), (40, 40), 1)])
+def test_mixed_hierarchical_records_match_the_direct_build(ml, l1, l2_sub, p):
+    """The mixed mode's node records from the series in pairs of floats against
+    those of the FP64 sum over all far lenses at every node, on cells that split
+    into one, evenly and unevenly many sub-blocks.  Both round the node's place
+    within its pixel to 2^-24 and c_n to FP32 (the series' coefficients carry
+    about 2e-6): 1e-5 of a pixel.  A ray's position off its node's base is an
+    FP32 number X whose last bit, 2^-23 |X|, may then differ too; the bases lie
+    within two map sides of the origin, so |X| is at most the ray's own pixel
+    coordinate plus 400."""
+    w = _mixed_case(seed=13)
+    fh = _field(ml, w, precision=ml.PREC_MIXED, l1=l1, l2_sub=l2_sub, taylor_p=p)
+    fd = _field(ml, w, precision=ml.PREC_MIXED, l1=l1, l2_sub=l2_sub, taylor_p=p, build=ml.BUILD_DIRECT)
+    assert (fh.info["build"], fd.info["build"]) == (ml.BUILD_HIERARCHICAL, ml.BUILD_DIRECT)
+    assert fh.info["taylor_p"] == fd.info["taylor_p"]
+    idx = np.unique(np.random.default_rng(5).integers(0, fh.n_rays, 30000))
+    bh, bd = fh.trace(idx)[0].cpu().numpy(), fd.trace(idx)[0].cpu().numpy()
+    dp = np.array([fh.info["dpx"], fh.info["dpy"]])
+    over = np.abs(bh - bd) / dp - 1e-5 - 2.0 ** -23 * (np.abs(bd) / dp + 400.0)
+    assert over.max() <= 0.0, over.max()
+    fh.close()
+    fd.close()
+
+
 @pytest.mark.parametrize("l2_sub", [(5, 5), (10, 5), (40, 20)])
 @pytest.mark.parametrize("span_far", [0.0, 1.0, 60.0, 1e9])
 def test_certified_walk_at_any_grid_and_lens_distance(ml, l2_sub, span_far):
