@@ -9,8 +9,8 @@
 //    offsets; each lane evaluates the node's Taylor series as a polynomial in
 //    its x offset, subtracts the near sum, bins the ray and merges runs of
 //    rays that fall in the same pixel before one atomic add.
-//  - k_shoot_direct64 / k_shoot_nearfar64: one thread per ray, FP64, the
-//    reference-precision modes.
+//  - k_shoot_direct64 / k_shoot_nearfar64: FP64, the reference-precision
+//    modes.
 //  - k_trace_*: the same arithmetic for listed rays, returning beta.
 #include "ml_internal.cuh"
 #include "ml_task.cuh"
@@ -46,72 +46,168 @@ __device__ __forceinline__ void sheet64(const Geo &g, double tx, double ty, doub
     sy = f * uy;
 }
 
-// beta of ray (i, j) in FP64 by the direct sum over all lenses (Eq. 6).
-// Returns false for a ray that coincides with a lens.
-__device__ bool beta_direct64(const ShootArgs &a, int64_t i, int64_t j, double &bx, double &by)
+// m / r2 for r2 > 0 to about one unit in the last place: the hardware's
+// approximate reciprocal (rcp.approx.ftz.f64, which reads r2's upper word) and
+// one third-order Newton step, y (1 + e + e^2) with e = 1 - r2 y (below 2^-18, so
+// e^3 is below the rounding).  Five FP64 instructions; FP64 runs at 1/64 of
+// FP32's rate here, and a division takes about ten.  Outside the exponents
+// where that holds (zero among them) the quotient is taken by division.
+template <bool UNIT>
+__device__ __forceinline__ double over_r2(double m, double r2)
 {
-    const Geo &g = a.g;
-    double tx = g.rx0 + ((double)i + 0.5) * g.l3x;
-    double ty = g.ry0 + ((double)j + 0.5) * g.l3y;
-    double ax = 0.0, ay = 0.0;
-    bool hit = false;
-    for (int64_t k = 0; k < a.L.n; ++k) {
-        double dx = tx - a.L.x[k], dy = ty - a.L.y[k];
-        double r2 = dx * dx + dy * dy;
-        hit |= (r2 == 0.0);
-        double s = a.L.m[k] / r2;
-        ax += dx * s;
-        ay += dy * s;
-    }
-    double sx, sy;
-    sheet64(g, tx, ty, sx, sy);
-    double mx, my;
-    macro64(g, tx, ty, mx, my);
-    bx = mx - ax - sx;
-    by = my - ay - sy;
-    return !hit;
+    if ((unsigned)(__double2hiint(r2) - 0x00200000) >= 0x7fb00000u) return m / r2;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+    const double e = __fma_rn(-r2, y, 1.0), t = __fma_rn(e, e, e);
+    const double my = UNIT ? y : __dmul_rn(m, y);      // UNIT: m is 1
+    return __fma_rn(my, t, my);
 }
 
-// beta of ray (i, j) in FP64 by the near/far scheme (Eq. 9): near lenses of
-// the 3 x 3 level-1 block summed directly, far field from the node series.
-__device__ bool beta_nearfar64(const ShootArgs &a, int64_t i, int64_t j, double &bx, double &by)
+// Adds lens (x, y, m) to the deflection of R rays of one row at tx[], ty.
+// Returns (per ray, in hit) whether the ray coincides with the lens.
+template <int R, bool UNIT>
+__device__ __forceinline__ void add_lens64_of(double x, double y, double m, const double (&tx)[R], double ty,
+                                           double (&ax)[R], double (&ay)[R], bool (&hit)[R])
+{
+    const double dy = __dadd_rn(ty, -y), dy2 = __dmul_rn(dy, dy);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const double dx = __dadd_rn(tx[r], -x);
+        const double r2 = __fma_rn(dx, dx, dy2);
+        hit[r] |= __double_as_longlong(r2) == 0;
+        const double s = over_r2<UNIT>(m, r2);
+        ax[r] = __fma_rn(dx, s, ax[r]);
+        ay[r] = __fma_rn(dy, s, ay[r]);
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void add_lens64(double x, double y, double m, const double (&tx)[R], double ty,
+                                           double (&ax)[R], double (&ay)[R], bool (&hit)[R])
+{
+    // (an integer comparison: FP64 ones take the FP64 pipe)
+    if (__double_as_longlong(m) == 0x3ff0000000000000ll) add_lens64_of<R, true>(x, y, m, tx, ty, ax, ay, hit);
+    else add_lens64_of<R, false>(x, y, m, tx, ty, ax, ay, hit);
+}
+
+__device__ __forceinline__ double ray_x64(const Geo &g, int64_t i) { return __fma_rn((double)i + 0.5, g.l3x, g.rx0); }
+__device__ __forceinline__ double ray_y64(const Geo &g, int64_t j) { return __fma_rn((double)j + 0.5, g.l3y, g.ry0); }
+
+// beta of R rays of one row in FP64 by the direct sum over all lenses (Eq. 6).
+template <int R>
+__device__ __forceinline__ void beta_direct64(const ShootArgs &a, const double (&tx)[R], double ty, double (&bx)[R],
+                                              double (&by)[R], bool (&hit)[R])
 {
     const Geo &g = a.g;
-    double tx = g.rx0 + ((double)i + 0.5) * g.l3x;
-    double ty = g.ry0 + ((double)j + 0.5) * g.l3y;
-    int64_t c1x = i / g.n1x, c1y = j / g.n1y;
-    int64_t c2x = i / g.n2x, c2y = j / g.n2y;
-    double ax = 0.0, ay = 0.0;
-    bool hit = false;
-    for (int64_t ey = c1y; ey <= c1y + 2; ++ey) {
-        int64_t b0 = ey * g.NEx + c1x;
-        for (int32_t k = a.L.start[b0]; k < a.L.start[b0 + 3]; ++k) {
-            double dx = tx - a.L.x[k], dy = ty - a.L.y[k];
-            double r2 = dx * dx + dy * dy;
-            hit |= (r2 == 0.0);
-            double s = a.L.m[k] / r2;
-            ax += dx * s;
-            ay += dy * s;
+    double ax[R], ay[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        ax[r] = ay[r] = 0.0;
+        hit[r] = false;
+    }
+    const double *x = a.L.x, *y = a.L.y, *m = a.L.m;
+    for (int64_t k = 0; k < a.L.n; ++k) add_lens64<R>(__ldg(x + k), __ldg(y + k), __ldg(m + k), tx, ty, ax, ay, hit);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        double sx, sy, mx, my;
+        sheet64(g, tx[r], ty, sx, sy);
+        macro64(g, tx[r], ty, mx, my);
+        bx[r] = mx - ax[r] - sx;
+        by[r] = my - ay[r] - sy;
+    }
+}
+
+// The FP64 near/far scheme (Eq. 9) for one row within one level-2 column: the
+// node series re-expanded in the rays' x offset dr from the node, as two real
+// polynomials (p FMAs each per ray instead of 2p), the near lenses' runs of the
+// sorted table, and the row's own part of beta.
+struct RowFar64 {
+    double br[PMAX + 1], bi[PMAX + 1];
+    double zx, ty, by0;
+    int32_t s[3], e[3];
+};
+
+__device__ __forceinline__ void row_far64(const ShootArgs &a, int64_t c2x, int64_t j, RowFar64 &f)
+{
+    const Geo &g = a.g;
+    const int64_t c2y = j / g.n2y, c1x = c2x / g.l2sx, c1y = j / g.n1y;
+    f.ty = ray_y64(g, j);
+    f.zx = __fma_rn((double)c2x + 0.5, g.l2x, g.rx0);
+    const double di = __dadd_rn(f.ty, -__fma_rn((double)c2y + 0.5, g.l2y, g.ry0));
+    const double2 *c = reinterpret_cast<const double2 *>(a.coef64) + (c2y * g.N2x + c2x) * (int64_t)(g.p + 1);
+    for (int n = 0; n <= g.p; ++n) {
+        const double2 v = __ldg(c + n);
+        f.br[n] = v.x;
+        f.bi[n] = v.y;
+    }
+    // b_n += (i di) b_{n+1} (repeated synthetic division)
+    for (int k = 0; k < g.p; ++k)
+        for (int n = g.p - 1; n >= k; --n) {
+            f.br[n] = __fma_rn(-di, f.bi[n + 1], f.br[n]);
+            f.bi[n] = __fma_rn(di, f.br[n + 1], f.bi[n]);
+        }
+    for (int q = 0; q < 3; ++q) {
+        const int64_t b0 = (c1y + q) * g.NEx + c1x;
+        f.s[q] = a.L.start[b0];
+        f.e[q] = a.L.start[b0 + 3];
+    }
+    const double my = g.macro == ML_MACRO_FOLD ? 2.0 * (1.0 - g.kappa0) : 1.0 - g.kappa + g.gamma;
+    f.by0 = __fma_rn(my, f.ty, __dmul_rn(sheet_ky(g), __dadd_rn(f.ty, -g.sheet_cy)));
+}
+
+// beta of R rays of that row at tx[] (all rays lie inside the sheet).
+template <int R>
+__device__ __forceinline__ void beta_nearfar64(const ShootArgs &a, const RowFar64 &f, const double (&tx)[R],
+                                               double (&bx)[R], double (&by)[R], bool (&hit)[R])
+{
+    const Geo &g = a.g;
+    double ax[R], ay[R], dr[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        dr[r] = __dadd_rn(tx[r], -f.zx);
+        bx[r] = f.br[g.p];
+        by[r] = f.bi[g.p];
+        ax[r] = ay[r] = 0.0;
+        hit[r] = false;
+    }
+    for (int n = g.p - 1; n >= 0; --n) {
+        const double cr = f.br[n], ci = f.bi[n];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            bx[r] = __fma_rn(bx[r], dr[r], cr);
+            by[r] = __fma_rn(by[r], dr[r], ci);
         }
     }
-    double zx = g.rx0 + ((double)c2x + 0.5) * g.l2x;
-    double zy = g.ry0 + ((double)c2y + 0.5) * g.l2y;
-    double dr = tx - zx, di = ty - zy;
-    const double *c = a.coef64 + (c2y * g.N2x + c2x) * (int64_t)(g.p + 1) * 2;
-    double Fr = 0.0, Fi = 0.0;
-    for (int n = g.p; n >= 0; --n) {      // Horner: F = F d + c_n
-        double nr = Fr * dr - Fi * di + c[2 * n];
-        double ni = Fr * di + Fi * dr + c[2 * n + 1];
-        Fr = nr;
-        Fi = ni;
+    for (int q = 0; q < 3; ++q)
+        for (int32_t k = f.s[q]; k < f.e[q]; ++k)
+            add_lens64<R>(__ldg(a.L.x + k), __ldg(a.L.y + k), __ldg(a.L.m + k), tx, f.ty, ax, ay, hit);
+    const double kx = sheet_kx(g);
+    const bool fold = g.macro == ML_MACRO_FOLD;
+    const double a1 = fold ? g.dy * f.ty : 1.0 - g.kappa - g.gamma, a2 = fold ? 0.5 * g.dx : 0.0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        // alpha_far = conj(F), F = (bx, by) so far
+        const double mx = fold ? __dmul_rn(tx[r], __fma_rn(a2, tx[r], a1)) : __dmul_rn(a1, tx[r]);
+        bx[r] = __dadd_rn(__dadd_rn(mx, -ax[r]), __fma_rn(kx, __dadd_rn(tx[r], -g.sheet_cx), -bx[r]));
+        by[r] = __dadd_rn(__dadd_rn(f.by0, -ay[r]), by[r]);
     }
-    double sx, sy;
-    sheet64(g, tx, ty, sx, sy);
-    double mx, my;
-    macro64(g, tx, ty, mx, my);
-    bx = mx - ax - Fr - sx;   // alpha_far = conj(F)
-    by = my - ay + Fi - sy;
-    return !hit;
+}
+
+// Pixel floor((b - m0) / dp) of Eq. 12 by a product with 1/dp; where that lies
+// within 1e-6 of a pixel edge, or far out, by the division itself, so that no
+// pixel depends on the product's rounding.  False outside [0, n).
+__device__ __forceinline__ bool bin64(double b, double m0, double dp, double idp, int n, int &pix)
+{
+    const double q = __dmul_rn(__dadd_rn(b, -m0), idp), f = floor(q);
+    const float fr = (float)(q - f);
+    pix = __double2int_rn(f);
+    if (!(fr > 1e-6f && fr < 0.999999f) || abs(pix) > 1000000) {
+        const double d = floor((b - m0) / dp);
+        if (!(d >= 0.0 && d < (double)n)) return false;
+        pix = (int)d;
+        return true;
+    }
+    return (unsigned)pix < (unsigned)n;
 }
 
 __device__ __forceinline__ void deposit_one(const ShootArgs &a, bool ok, double bx, double by,
@@ -179,21 +275,102 @@ struct SpanCount {
     unsigned long long evals = 0, spans = 0;
 };
 
-// One thread per ray over [ray_begin, ray_end), FP64 (direct or near/far).
-template <bool NEARFAR>
-__global__ void __launch_bounds__(256) k_shoot_fp64(ShootArgs a)
+// NGP count of one ray in the FP64 modes (CIC: deposit_one).
+__device__ __forceinline__ void deposit64(const ShootArgs &a, bool hit, double bx, double by, double ipx, double ipy,
+                                          unsigned long long &in, unsigned long long &out, unsigned long long &drop,
+                                          unsigned &ovf)
 {
-    unsigned long long in = 0, out = 0, drop = 0, pairs = 0;
-    unsigned ovf = 0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t r = a.ray_begin + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < a.ray_end;
-         r += stride) {
-        int64_t i = r % a.g.n3x, j = r / a.g.n3x;
-        double bx, by;
-        bool ok = NEARFAR ? beta_nearfar64(a, i, j, bx, by) : beta_direct64(a, i, j, bx, by);
-        deposit_one(a, ok, bx, by, in, out, drop, ovf);
+    const Geo &g = a.g;
+    if (g.deposit != ML_DEPOSIT_NGP) {
+        deposit_one(a, !hit, bx, by, in, out, drop, ovf);
+        return;
     }
-    flush_stats(a, in, out, drop, pairs, 0, ovf);
+    if (hit) { ++drop; return; }
+    int ix, iy;
+    if (bin64(bx, g.mx0, g.dpx, ipx, g.mnx, ix) && bin64(by, g.my0, g.dpy, ipy, g.mny, iy)) {
+        const unsigned old = atomicAdd(a.map_u32 + (size_t)iy * (unsigned)g.mnx + (unsigned)ix, 1u);
+        ovf |= (old == 0xFFFFFFFFu);
+        ++in;
+    } else {
+        ++out;
+    }
+}
+
+// Direct mode: a warp takes 32 R consecutive rays of one lattice row, lane l
+// the rays l, l + 32, ... (R of them share the lens's row offset, and their
+// chains hide the FP64 latency).  Bound by the FP64 pipe: 8 instructions per
+// ray and lens (7 for a unit mass) and 2/R shared, against about 16 with one
+// ray a thread, a division and an FP64 compare: 4e8 pairs took 10.9 ms, now
+// 5.8 ms at 90 % of the pipe.
+template <int R>
+__global__ void __launch_bounds__(256) k_shoot_direct64(ShootArgs a)
+{
+    const Geo &g = a.g;
+    unsigned long long in = 0, out = 0, drop = 0;
+    unsigned ovf = 0;
+    const int lane = threadIdx.x & 31;
+    const int64_t nseg = (g.n3x + 32 * R - 1) / (32 * R);
+    const int64_t jb = a.ray_begin / g.n3x, je = (a.ray_end - 1) / g.n3x, items = (je - jb + 1) * nseg;
+    const double ipx = 1.0 / g.dpx, ipy = 1.0 / g.dpy;
+    for (int64_t it = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
+        const int64_t j = jb + it / nseg, i0 = (it % nseg) * (32 * R) + lane;
+        bool have[R], any = false, hit[R];
+        double tx[R], bx[R], by[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int64_t i = i0 + 32 * r, ray = j * g.n3x + i;
+            have[r] = i < g.n3x && ray >= a.ray_begin && ray < a.ray_end;
+            any |= have[r];
+            tx[r] = ray_x64(g, i);
+        }
+        if (!__any_sync(0xffffffffu, any)) continue;
+        beta_direct64<R>(a, tx, ray_y64(g, j), bx, by, hit);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (have[r]) deposit64(a, hit[r], bx[r], by[r], ipx, ipy, in, out, drop, ovf);
+    }
+    flush_stats(a, in, out, drop, 0, 0, ovf);
+}
+
+// Near/far mode: lane = lattice row, a warp takes 32 rows and a chunk of up to
+// NF_CHUNK rays of one level-2 column; four rays at a time.  Bound by the FP64
+// pipe: 2p + 8 per near lens + about 20 per ray instead of 4p + 16 per near lens
+// + about 40 and five 64-bit divisions: 1.2e7 rays at p = 10 took 2.84 ms, now
+// 1.30 ms at 90 % of the pipe.
+constexpr int NF_CHUNK = 64;
+
+__global__ void __launch_bounds__(256) k_shoot_nearfar64(ShootArgs a)
+{
+    constexpr int R = 4;
+    const Geo &g = a.g;
+    unsigned long long in = 0, out = 0, drop = 0;
+    unsigned ovf = 0;
+    const int lane = threadIdx.x & 31;
+    const int64_t cpc = (g.n2x + NF_CHUNK - 1) / NF_CHUNK, ncol = g.N2x * cpc;
+    const int64_t jb = a.ray_begin / g.n3x, je = (a.ray_end - 1) / g.n3x, items = ((je - jb) / 32 + 1) * ncol;
+    const double ipx = 1.0 / g.dpx, ipy = 1.0 / g.dpy;
+    for (int64_t it = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
+        const int64_t j = jb + 32 * (it / ncol) + lane, cc = it % ncol, c2x = cc / cpc;
+        if (j > je) continue;
+        int64_t i0 = c2x * g.n2x + (cc % cpc) * NF_CHUNK;
+        int64_t i1 = min(min(i0 + NF_CHUNK, (c2x + 1) * g.n2x), g.n3x);
+        i0 = max(i0, a.ray_begin - j * g.n3x);
+        i1 = min(i1, a.ray_end - j * g.n3x);
+        if (i0 >= i1) continue;
+        RowFar64 f;
+        row_far64(a, c2x, j, f);
+        for (int64_t i = i0; i < i1; i += R) {
+            double tx[R], bx[R], by[R];
+            bool hit[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) tx[r] = ray_x64(g, i + r);
+            beta_nearfar64<R>(a, f, tx, bx, by, hit);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (i + r < i1) deposit64(a, hit[r], bx[r], by[r], ipx, ipy, in, out, drop, ovf);
+        }
+    }
+    flush_stats(a, in, out, drop, 0, 0, ovf);
 }
 
 // ---- mixed precision: per-task staging and the walk --------------------------
@@ -1242,9 +1419,19 @@ __global__ void k_trace_fp64(ShootArgs a, const int64_t *__restrict__ idx, int64
         pix[2 * q] = pix[2 * q + 1] = -3;
         return;
     }
-    int64_t i = r % g.n3x, j = r / g.n3x;
-    double bx, by;
-    bool ok = NEARFAR ? beta_nearfar64(a, i, j, bx, by) : beta_direct64(a, i, j, bx, by);
+    const int64_t i = r % g.n3x, j = r / g.n3x;
+    const double tx[1] = {ray_x64(g, i)};
+    double vx[1], vy[1];
+    bool hit[1];
+    if constexpr (NEARFAR) {
+        RowFar64 f;
+        row_far64(a, i / g.n2x, j, f);
+        beta_nearfar64<1>(a, f, tx, vx, vy, hit);
+    } else {
+        beta_direct64<1>(a, tx, ray_y64(g, j), vx, vy, hit);
+    }
+    const double bx = vx[0], by = vy[0];
+    const bool ok = !hit[0];
     beta[2 * q] = bx;
     beta[2 * q + 1] = by;
     if (!ok) { pix[2 * q] = -2; pix[2 * q + 1] = -2; return; }
@@ -1311,14 +1498,22 @@ cudaError_t launch_shoot(const ShootArgs &a, int num_sms, cudaStream_t s)
         default: return cudaErrorInvalidValue;
         }
     }
-    int64_t n = a.ray_end - a.ray_begin;
-    int64_t blocks = (n + 255) / 256;
-    int64_t cap = (int64_t)num_sms * 8;
-    if (blocks > cap) blocks = cap;
-    if (a.g.precision == ML_PREC_NEARFAR64)
-        k_shoot_fp64<true><<<(unsigned)blocks, 256, 0, s>>>(a);
-    else
-        k_shoot_fp64<false><<<(unsigned)blocks, 256, 0, s>>>(a);
+    const int64_t rows = (a.ray_end - 1) / a.g.n3x - a.ray_begin / a.g.n3x + 1;
+    auto blocks_of = [&](int64_t items) {
+        return (unsigned)std::min<int64_t>((items + 7) / 8, (int64_t)num_sms * 4096);
+    };
+    if (a.g.precision == ML_PREC_NEARFAR64) {
+        const int64_t ncol = a.g.N2x * ((a.g.n2x + NF_CHUNK - 1) / NF_CHUNK);
+        k_shoot_nearfar64<<<blocks_of((rows + 31) / 32 * ncol), 256, 0, s>>>(a);
+        return cudaGetLastError();
+    }
+    // rays per thread: as many as leave no more of the row's last segment empty
+    // than fewer would, to 3 %
+    auto segs = [&](int r) { return (a.g.n3x + 32 * r - 1) / (32 * r); };
+    const double full = 1.03 * (double)segs(1);
+    if ((double)(4 * segs(4)) <= full) k_shoot_direct64<4><<<blocks_of(rows * segs(4)), 256, 0, s>>>(a);
+    else if ((double)(2 * segs(2)) <= full) k_shoot_direct64<2><<<blocks_of(rows * segs(2)), 256, 0, s>>>(a);
+    else k_shoot_direct64<1><<<blocks_of(rows * segs(1)), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

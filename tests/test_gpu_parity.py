@@ -358,6 +358,34 @@ def test_certified_walk_equals_per_ray_walk(ml, case):
     fp.close()
 
 
+@pytest.mark.parametrize("precision", ["direct64", "nearfar64"])
+@pytest.mark.parametrize("n3x,n3y,mass", [(1, 70, "unit"), (33, 5, "lognormal"), (65, 40, "unit"), (128, 33, "lognormal"),
+                                          (301, 64, "lognormal")])
+def test_fp64_modes_over_lattice_widths_and_ranges(ml, precision, n3x, n3y, mass):
+    """Lattices around the FP64 kernels' segments (32 to 128 rays of a row) and
+    chunks (64 rays of a level-2 column, 32 rows), whole and in ragged ranges: the
+    counts are the histogram of the traced pixels, and the traced positions those
+    of the oracle's direct sum to FP64 rounding (the near/far mode at order 16:
+    to its truncation bound)."""
+    w = _mixed_case(seed=3)
+    w.lenses = inputs.lens_disc(w.lenses.n, w.lenses.radius, 3, mass)
+    g0 = oracle.derive_geometry(w.kappa, w.gamma, w.kappa_star, [], [], (0, 0, 1), w.map_box, w.map_n, n_av=60)
+    w.ray_box, w.ray_n = (g0.rx0, g0.ry0, g0.rx1, g0.ry1), (n3x, n3y)
+    near = precision == "nearfar64"
+    f = _field(ml, w, precision=ml.PREC_NEARFAR64 if near else ml.PREC_DIRECT64, taylor_p=16 if near else 0,
+               l1=(8.0, 4.0), l2_sub=(1, 1))
+    n = n3x * n3y
+    for r0, r1 in ((0, n), (n // 3 + 1, n - n // 5), (n // 2, n // 2 + 1)):
+        _shot_equals_traced(ml, f, r0, r1)
+    beta = f.trace(np.arange(n))[0].cpu().numpy()
+    g = _geometry(w, f)
+    ref, flag = oracle.beta_direct(g, w.lenses.x, w.lenses.y, w.lenses.m, np.arange(n))
+    assert not np.any(flag)
+    tol = 1e-11 * (1.0 + np.abs(ref)) + (f.info["far_bound"] if near else 0.0)
+    assert np.all(np.abs(beta - ref) <= tol)
+    f.close()
+
+
 @pytest.mark.parametrize("l1,l2_sub,p", [((6.0, 6.0), (20, 20), 0), ((9.0, 2.0), (10, 7), 0), ((2.0, 7.0), (5, 11), 0),
                                          ((5.0, 4.0), (3, 1), 16), ((4.0, 4.0), (1, 1), 12), ((3.0, 3.0), (40, 40), 1)])
 def test_mixed_hierarchical_records_match_the_direct_build(ml, l1, l2_sub, p):
