@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, (P <= 4 ? ML_ADJ_LOWP_BLOC
         const bool head = active && (lane == 0 || j == c2y * g.n2y);
         for (int64_t c2x = ts.c2a; c2x < ts.c2b; ++c2x) {
             const double xnode = g.rx0 + ((double)c2x + 0.5) * g.l2x;
-            stage_near_x<false>(a, nn, xnode, near, nlo, lane);
+            stage_near_x<false>(a, nn, c2x, near, nlo, lane);
             const int64_t i0 = c2x * g.n2x;
             const int kend = (int)(min(i0 + g.n2x, g.n3x) - i0);
             RowPoly<P> rp;

@@ -94,6 +94,7 @@ struct ShootArgs {
     float q2_f;                     // beta_x curvature in u (fold: d_x l3x^2 / (2 dpx)), else 0
     float rc2;                      // close-pass radius^2 of near_sum_f32 (theta_E^2)
     float rc2u;                     // the same in lattice units (near_sum_lat)
+    float piece_max;                // rays per piece of run_nodes: 0.15 level-1 cell widths
     float l3yx_f;                   // l3y / l3x: a ray row in lattice units
     float yx_f;                     // dpx / dpy: y deflection per x deflection unit (pixels)
     double rho_y;                   // (d(macro_y)/d(theta_y) + kappa_*) * l3y / dpy

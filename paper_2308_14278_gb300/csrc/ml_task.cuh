@@ -73,11 +73,15 @@ __device__ __forceinline__ int stage_near_y(const ShootArgs &a, const NearRuns &
     return nn;
 }
 
+// c2x: the level-2 column (its node's x, in FP64, only where there are lenses:
+// an FP64 instruction takes 16 cycles of the SM a warp here)
 template <bool LAT>
-__device__ __forceinline__ void stage_near_x(const ShootArgs &a, int nn, double xnode,
+__device__ __forceinline__ void stage_near_x(const ShootArgs &a, int nn, int64_t c2x,
                                              float4 *near, float2 *nlo, int lane)
 {
     __syncwarp();
+    if (nn == 0) return;
+    const double xnode = a.g.rx0 + ((double)c2x + 0.5) * a.g.l2x;
     for (int k = lane; k < nn; k += 32) {
         double dx = a.L.x[__float_as_int(near[k].w)] - xnode;
         if (LAT) dx *= a.il3x;

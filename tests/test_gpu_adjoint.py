@@ -294,6 +294,34 @@ def test_map_light_curves_match_oracle(ml):
     assert np.allclose(out.cpu().numpy(), ref, rtol=1e-5, atol=1e-6)
 
 
+@pytest.mark.parametrize("l2", [(10, 10), (3, 2), (1, 1)])
+@pytest.mark.parametrize("px", [(64, 48), (301, 7), (5, 4)])
+def test_cic_runs_by_quadrature_match_the_rays_one_by_one(ml, l2, px):
+    """Columns without near lenses sum a quad's rays by quadrature; the per-ray
+    walk evaluates each.  Long columns on short quads, quads longer than a column
+    and a few rays wide, on a sparse field: the same rays in and out of the map,
+    and every pixel within the FP32 sums' rounding, 2^-24 of the pixel's sum per
+    quad added (some hundred), and weights of 2e-7 a ray."""
+    w = _case()
+    w.map_n = px
+    n_rays = w.ray_n[0] * w.ray_n[1]
+    kw = dict(l1=(2.0, 1.5), l2_sub=l2)
+    fq, fr = _field(ml, w, **kw), _field(ml, w, walk=ml.WALK_PER_RAY, **kw)
+    for r0, r1 in ((0, n_rays), (n_rays // 3 + 5, n_rays // 2 + 1)):
+        out = []
+        for f in (fq, fr):
+            f.clear()
+            f.shoot(r0, r1)
+            out.append((f.mu().cpu().numpy().astype(np.float64), f.stats()))
+        (a, sa), (b, sb) = out
+        for k in ("rays_in", "rays_out", "rays_dropped", "near_pairs"):
+            assert sa[k] == sb[k], k
+        assert np.abs(a - b).max() <= 2e-5 * b.max(), np.abs(a - b).max() / b.max()
+        assert abs(a.sum() - b.sum()) <= 1e-6 * b.sum()
+    fq.close()
+    fr.close()
+
+
 def _corner_sums(mu, tracks, ns, sigma):
     """Light curves corner by corner and tap by tap in FP64 with float taps, as
     the library documents them: corners outside the map or of weight zero and
