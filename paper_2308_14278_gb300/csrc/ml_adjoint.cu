@@ -454,26 +454,62 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, (P <= 4 ? ML_ADJ_LOWP_BLOC
                     gdy2 = __fmul_rn(gdy, gdy);
                 }
                 float nax = 0.f, nay = 0.f, nam = 0.f;
-                unsigned cqx = 0xFFFFFFFFu, cqy = 0xFFFFFFFFu;
-                auto load_quad = [&](unsigned ix, unsigned iy) {
-                    cqx = ix;
-                    cqy = iy;
-                    return quad_g(g, d.G, ix, iy);
-                };
+                // row polynomial, quad floors, dL/dbeta and t-power sums run on
+                // (x, y) pairs with two-lane instructions, each lane rounded as
+                // the scalar one: per ray 40 issue slots instead of 61 (1.27 ->
+                // 1.13 ms for the differentiable field's 4e8 rays)
+                f32x2 C[P + 1], T2[P + 1];
+#pragma unroll
+                for (int m = 0; m <= P; ++m) {
+                    C[m] = pack2(rp.X[m], rp.Y[m]);
+                    T2[m] = pack2(T[2 * m], T[2 * m + 1]);
+                }
+                f32x2 sg = pack2(sgx, sgy);
+                const f32x2 ONE = pack2(1.f, 1.f), NEG1 = pack2(-1.f, -1.f), NHALF = pack2(-0.5f, -0.5f);
+                const f32x2 MAGIC = pack2(12582912.0f, 12582912.0f), NMAGIC = pack2(-12582912.0f, -12582912.0f);
+                const f32x2 IP = pack2(d.ipx, d.ipy), L3 = pack2(a.l3x_f, a.l3x_f), HI = pack2(d.hinv, d.hinv);
+                // the quad of a pixel position in raw floor form (bits of the
+                // floor + 1.5 2^23), compared in that form
+                const unsigned offx = (unsigned)rp.bx - 0x4B400000u, offy = (unsigned)rp.by - 0x4B400000u;
                 // the cache starts as a real quad (the one whose only pixel
                 // in the map is (0, 0)), with its own values
-                QuadG cq = load_quad(cqx, cqy);
-                auto add_ray = [&](float gbx, float gby, float tt) {
-                    sgx += gbx;
-                    sgy += gby;
-                    stx = __fmaf_rn(gbx, tt, stx);
-                    const float th = __fmul_rn(tt, d.hinv);
-                    float pw = 1.f;
+                unsigned rqx = 0xFFFFFFFFu - offx, rqy = 0xFFFFFFFFu - offy;
+                f32x2 QA, QB;                          // (e10, e20), (e32, e31)
+                auto load_quad = [&](unsigned rx, unsigned ry) {
+                    rqx = rx;
+                    rqy = ry;
+                    const QuadG q = quad_g(g, d.G, rx + offx, ry + offy);
+                    QA = pack2(q.e10, q.e20);
+                    QB = pack2(q.e32, q.e31);
+                };
+                load_quad(rqx, rqy);
+                // quad (raw) and weights of a ray, swapped to (wy, wx)
+                auto quad_of = [&](float X, float Y, unsigned &rx, unsigned &ry) {
+                    const f32x2 f = add2(pack2(X, Y), NHALF), fl = add2_rd(f, MAGIC);
+                    float x, y;
+                    unpack2(fl, x, y);
+                    rx = (unsigned)__float_as_int(x);
+                    ry = (unsigned)__float_as_int(y);
+                    unpack2(fma2(add2(fl, NMAGIC), NEG1, f), x, y);
+                    return pack2(y, x);
+                };
+                // quad_dbeta's operations on the pair
+                auto dbeta = [&](f32x2 w) {
+                    return mul2(IP, fma2(QB, w, mul2(QA, fma2(w, NEG1, ONE))));
+                };
+                auto add_ray = [&](f32x2 gb, f32x2 tt) {
+                    float gx, gy, t, th;
+                    unpack2(gb, gx, gy);
+                    unpack2(tt, t, th);
+                    sg = add2(sg, gb);
+                    stx = __fmaf_rn(gx, t, stx);
+                    const f32x2 h = mul2(tt, HI);
+                    f32x2 pw = h;
+                    T2[0] = add2(T2[0], gb);
 #pragma unroll
-                    for (int n = 0; n <= P; ++n) {
-                        T[2 * n] = __fmaf_rn(gbx, pw, T[2 * n]);
-                        T[2 * n + 1] = __fmaf_rn(gby, pw, T[2 * n + 1]);
-                        pw = __fmul_rn(pw, th);
+                    for (int n = 1; n <= P; ++n) {
+                        T2[n] = fma2(gb, pw, T2[n]);
+                        pw = mul2(pw, h);
                     }
                 };
                 auto near_fwd = [&](float tt, float &X, float &Y, float &r2) {
@@ -499,10 +535,18 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, (P <= 4 ? ML_ADJ_LOWP_BLOC
                 for (int k = 0; k < kend; k += 2, u += 2.f) {
                     const bool on1 = active && k + 1 < kend;
                     const float u1 = __fadd_rn(u, 1.f);
-                    const float t0 = __fmul_rn(u, a.l3x_f), t1 = __fmul_rn(u1, a.l3x_f);
-                    float X0, Y0, X1, Y1;
-                    row_eval<P>(rp, u, X0, Y0);
-                    row_eval<P>(rp, u1, X1, Y1);
+                    const f32x2 U0 = pack2(u, u), U1 = pack2(u1, u1), tt0 = mul2(U0, L3), tt1 = mul2(U1, L3);
+                    f32x2 p0 = C[P], p1 = C[P];
+#pragma unroll
+                    for (int m = P - 1; m >= 0; --m) {
+                        p0 = fma2(p0, U0, C[m]);
+                        p1 = fma2(p1, U1, C[m]);
+                    }
+                    float X0, Y0, X1, Y1, t0, t1, th;
+                    unpack2(p0, X0, Y0);
+                    unpack2(p1, X1, Y1);
+                    unpack2(tt0, t0, th);
+                    unpack2(tt1, t1, th);
                     bool ok0 = active, ok1 = on1;
                     if (NN == 1) {
                         const float Xp0 = X0, Yp0 = Y0, Xp1 = X1, Yp1 = Y1;
@@ -525,31 +569,32 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, (P <= 4 ? ML_ADJ_LOWP_BLOC
                             }
                         }
                     }
-                    unsigned ix0, iy0, ix1, iy1;
-                    float wx0, wy0, wx1, wy1;
-                    cic_quad(rp.bx, rp.by, X0, Y0, ix0, iy0, wx0, wy0);
-                    cic_quad(rp.bx, rp.by, X1, Y1, ix1, iy1, wx1, wy1);
+                    unsigned rx0, ry0, rx1, ry1;
+                    const f32x2 w0 = quad_of(X0, Y0, rx0, ry0), w1 = quad_of(X1, Y1, rx1, ry1);
                     // ray 1 compares with the quad after ray 0 (unchanged
                     // when ray 0 is dropped)
-                    const bool ch0 = ok0 && (ix0 != cqx || iy0 != cqy);
-                    const bool ch1 = ok1 && (ix1 != (ok0 ? ix0 : cqx) || iy1 != (ok0 ? iy0 : cqy));
+                    const bool ch0 = ok0 && (rx0 != rqx || ry0 != rqy);
+                    const bool ch1 = ok1 && (rx1 != (ok0 ? rx0 : rqx) || ry1 != (ok0 ? ry0 : rqy));
                     const bool any = __ballot_sync(0xffffffffu, ch0 || ch1) != 0u;
                     float gx0, gy0, gx1, gy1;
-                    if (any && ch0) cq = load_quad(ix0, iy0);
-                    quad_dbeta(cq, wx0, wy0, d.ipx, d.ipy, gx0, gy0);
-                    if (any && ch1) cq = load_quad(ix1, iy1);
-                    quad_dbeta(cq, wx1, wy1, d.ipx, d.ipy, gx1, gy1);
+                    if (any && ch0) load_quad(rx0, ry0);
+                    unpack2(dbeta(w0), gx0, gy0);
+                    if (any && ch1) load_quad(rx1, ry1);
+                    unpack2(dbeta(w1), gx1, gy1);
                     gx0 = ok0 ? gx0 : 0.f;
                     gy0 = ok0 ? gy0 : 0.f;
                     gx1 = ok1 ? gx1 : 0.f;
                     gy1 = ok1 ? gy1 : 0.f;
-                    add_ray(gx0, gy0, t0);
-                    add_ray(gx1, gy1, t1);
+                    add_ray(pack2(gx0, gy0), tt0);
+                    add_ray(pack2(gx1, gy1), tt1);
                     if (NN == 1) {
                         near_grad(ok0, t0, gx0, gy0);
                         near_grad(ok1, t1, gx1, gy1);
                     }
                 }
+                unpack2(sg, sgx, sgy);
+#pragma unroll
+                for (int m = 0; m <= P; ++m) unpack2(T2[m], T[2 * m], T[2 * m + 1]);
                 if (NN == 1) {
                     for (int off = 16; off > 0; off >>= 1) {
                         nax += __shfl_down_sync(0xffffffffu, nax, off);
