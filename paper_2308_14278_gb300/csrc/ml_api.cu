@@ -831,41 +831,26 @@ ml_status create_plan(const ml_field_desc *d_in, cudaStream_t s, ml_field *f)
                          f->d_sy, f->d_sm, f->d_scell, f->d_perm, f->d_f32, s));
     if (!nearfar) return ML_OK;
 
-    // largest near list: the 3 x 3 block of each level-1 cell
-    std::vector<int32_t> start(NE + 2);
-    ML_CK(cudaMemcpyAsync(start.data(), f->d_start, (NE + 2) * sizeof(int32_t),
-                          cudaMemcpyDeviceToHost, s));
-    ML_CK(cudaStreamSynchronize(s));
-    int32_t mx = 0;
-    for (int64_t cy = 0; cy < g.N1y; ++cy)
-        for (int64_t cx = 0; cx < g.N1x; ++cx) {
-            int32_t t = 0;
-            for (int64_t ey = cy; ey <= cy + 2; ++ey) {
-                int64_t b = ey * g.NEx + cx;
-                t += start[b + 3] - start[b];
-            }
-            mx = std::max(mx, t);
-        }
-    f->max_near = mx;
-    if (d->precision == ML_PREC_MIXED && (int64_t)mx * WARPS_PER_CTA * 24 > 200 * 1024)
-        return fail(ML_ERR_UNSUPPORTED, "a level-1 cell has " + std::to_string(mx) +
-                                            " near lenses; use a finer level-1 grid (l1_x, l1_y)");
-
-    // truncation bound of every Taylor order, worst level-1 cell
-    std::vector<double> bound((size_t)(g.N1x * g.N1y) * PMAX);
-    double *d_bound = nullptr;
-    ML_CK(ml_malloc_async((void **)&d_bound, bound.size() * sizeof(double), s));
+    // truncation bound of every Taylor order at each level-1 cell; their worst
+    // cell and the longest near list come to the host in one small read
+    const size_t nb = (size_t)(g.N1x * g.N1y) * PMAX;
+    char *scratch = nullptr;
+    ML_CK(ml_malloc_async((void **)&scratch, nb * sizeof(double) + (PMAX + 1) * sizeof(unsigned long long), s));
+    double *d_bound = reinterpret_cast<double *>(scratch);
+    unsigned long long *d_max = reinterpret_cast<unsigned long long *>(d_bound + nb), worst[PMAX + 1] = {};
     g.p = 1;
     cudaError_t e = launch_p_bound(g, f->table(), d_bound, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(bound.data(), d_bound, bound.size() * sizeof(double),
-                            cudaMemcpyDeviceToHost, s);
-    cudaFreeAsync(d_bound, s);
+    if (e == cudaSuccess) e = launch_plan_max(g, f->d_start, d_bound, d_max, f->num_sms, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(worst, d_max, sizeof(worst), cudaMemcpyDeviceToHost, s);
+    cudaFreeAsync(scratch, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "truncation bound");
-    ML_CK(cudaStreamSynchronize(s));
+    f->max_near = (int32_t)worst[0];
+    if (d->precision == ML_PREC_MIXED && (int64_t)f->max_near * WARPS_PER_CTA * 24 > 200 * 1024)
+        return fail(ML_ERR_UNSUPPORTED, "a level-1 cell has " + std::to_string(f->max_near) +
+                                            " near lenses; use a finer level-1 grid (l1_x, l1_y)");
     f->worst.assign(PMAX, 0.0);
-    for (size_t c = 0; c < bound.size() / PMAX; ++c)
-        for (int q = 0; q < PMAX; ++q) f->worst[q] = std::max(f->worst[q], bound[c * PMAX + q]);
+    for (int q = 0; q < PMAX; ++q) memcpy(&f->worst[q], &worst[q + 1], sizeof(double));
     return ML_OK;
 }
 

@@ -358,6 +358,46 @@ cudaError_t launch_p_bound(const Geo &g, const LensTable &L, double *bound, cuda
     return cudaGetLastError();
 }
 
+// Largest near list (3 x 3 block of extended cells) and largest bound of each
+// order over the level-1 cells, for the host's choice of the order: out[0] the
+// near lenses, out[q] the bits of order q's bound (not negative, NaN left out,
+// as in the comparison v > m).  The host used to read every cell's values: 7 MB
+// and 0.4 million comparisons for the Table-1 field.
+__global__ void __launch_bounds__(256) k_plan_max(Geo g, const int32_t *__restrict__ start,
+                                                  const double *__restrict__ bound, unsigned long long *out)
+{
+    static_assert(PMAX == 16, "one thread per order");
+    const int q = threadIdx.x % PMAX;
+    const int64_t ncell = g.N1x * g.N1y, step = (int64_t)gridDim.x * (blockDim.x / PMAX);
+    double m = 0.0;
+    int near = 0;
+    for (int64_t c = blockIdx.x * (int64_t)(blockDim.x / PMAX) + threadIdx.x / PMAX; c < ncell; c += step) {
+        const double v = bound[c * PMAX + q];
+        if (v > m) m = v;
+        if (q < 1) {
+            const int64_t cy = c / g.N1x, b = cy * g.NEx + (c - cy * g.N1x);
+            int t = 0;
+            for (int r = 0; r < 3; ++r) t += start[b + r * g.NEx + 3] - start[b + r * g.NEx];
+            near = max(near, t);
+        }
+    }
+    const double o = __shfl_xor_sync(0xffffffffu, m, PMAX);
+    if (o > m) m = o;
+    near = __reduce_max_sync(0xffffffffu, near);
+    if ((threadIdx.x & 31) < PMAX && m > 0.0) atomicMax(out + 1 + q, (unsigned long long)__double_as_longlong(m));
+    if ((threadIdx.x & 31) == 0 && near > 0) atomicMax(out, (unsigned long long)near);
+}
+
+cudaError_t launch_plan_max(const Geo &g, const int32_t *start, const double *bound, unsigned long long *out,
+                            int num_sms, cudaStream_t s)
+{
+    cudaError_t e = cudaMemsetAsync(out, 0, (PMAX + 1) * sizeof(unsigned long long), s);
+    if (e != cudaSuccess) return e;
+    const int64_t want = (g.N1x * g.N1y + 15) / 16;
+    k_plan_max<<<(unsigned)(want < 4 * num_sms ? want : 4 * num_sms), 256, 0, s>>>(g, start, bound, out);
+    return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------------------
 // Far-field Taylor coefficients at the level-2 nodes, by direct summation:
 // c_n = - sum_{k far} m_k / (z_k - z_node)^{n+1},  n = 0..p.

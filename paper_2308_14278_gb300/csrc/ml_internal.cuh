@@ -133,6 +133,8 @@ inline void set_f32(LensTable &L, const float *f32, int64_t n)
     L.xh = f32; L.xl = f32 + n; L.yh = f32 + 2 * n; L.yl = f32 + 3 * n; L.mf = f32 + 4 * n;
 }
 cudaError_t launch_p_bound(const Geo &g, const LensTable &L, double *bound, cudaStream_t s);
+cudaError_t launch_plan_max(const Geo &g, const int32_t *start, const double *bound, unsigned long long *out,
+                            int num_sms, cudaStream_t s);
 cudaError_t launch_coeffs_direct(const Geo &g, const LensTable &L, double *coef64, cudaStream_t s);
 cudaError_t launch_coeffs_hier(const Geo &g, const LensTable &L, double *coef64, unsigned char *nodes,
                                double *scratch, size_t scratch_doubles, cudaStream_t s);
