@@ -90,12 +90,15 @@ template <class Key, class Emit>
 __device__ void cta_stable_scatter(const Key &key, int64_t n, int64_t nb, const int32_t *start,
                                    int32_t *ostart, int32_t *cnt, const Emit &emit)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+    // W counting warps: their rows of buckets are cleared and turned into slots,
+    // W x nb counters, so many buckets take fewer warps (eight beyond 16,384
+    // buckets: Table-1 field, 56,000 buckets, 0.45 -> SCAT_NOTE ms)
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = nb > 16384 ? 8 : blockDim.x >> 5;
     const int64_t chunk = (n + W - 1) / W;
-    const int64_t kb = min(n, w * chunk), ke = min(n, kb + chunk);
+    const int64_t kb = w < W ? min(n, w * chunk) : n, ke = min(n, kb + chunk);
     int32_t *my = cnt + w * nb;
-    for (int64_t b = lane; b < nb; b += 32) my[b] = 0;
-    __syncwarp();
+    for (int64_t b = threadIdx.x; b < W * nb; b += blockDim.x) cnt[b] = 0;
+    __syncthreads();
     for (int64_t base = kb; base < ke; base += 32) {
         const int64_t k = base + lane;
         const int32_t c = k < ke ? key(k) : -1;
