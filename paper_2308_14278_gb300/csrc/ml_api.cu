@@ -641,8 +641,8 @@ GridChoice best_single(const std::vector<TuneCand> &cands)
 }
 
 ml_status measure_grid(const ml_field_desc &d, const std::vector<double> &hx, const std::vector<double> &hy,
-                       const std::vector<double> &hm, const TuneCand &c, cudaStream_t s, double &est_ms,
-                       float &span_far, bool &use_span);
+                       const std::vector<double> &hm, const TuneCand &c, cudaStream_t s, int &option,
+                       double &est_ms, float &span_far, bool &use_span);
 
 std::unordered_map<uint64_t, GridChoice> g_measured;   // guarded by g_tune_mu
 
@@ -685,6 +685,7 @@ ml_status tune_grid(const ml_field_desc &d, const std::vector<double> &hx, const
     });
     double best_est = 0.0;
     bool found = false;
+    int option = -1;                 // the last candidate's best walk option
     for (size_t i = 0; i < std::min<size_t>(3, order.size()); ++i) {
         const TuneCand &c = cands[order[i]];
         double est = 0.0;
@@ -692,7 +693,7 @@ ml_status tune_grid(const ml_field_desc &d, const std::vector<double> &hx, const
         bool span = true;
         // a candidate that cannot be built (near lists too long for the
         // mixed kernel's shared memory, memory) is passed over
-        if (measure_grid(d, hx, hy, hm, c, s, est, far, span) != ML_OK) {
+        if (measure_grid(d, hx, hy, hm, c, s, option, est, far, span) != ML_OK) {
             cudaGetLastError();
             continue;
         }
@@ -932,8 +933,8 @@ ml_status create_impl(const ml_field_desc *d, cudaStream_t s, ml_field *f)
 // whole lattice.  The lenses come from the tuner's host copies (the
 // descriptor being built has handed its own pointers over already).
 ml_status measure_grid(const ml_field_desc &d, const std::vector<double> &hx, const std::vector<double> &hy,
-                       const std::vector<double> &hm, const TuneCand &c, cudaStream_t s, double &est_ms,
-                       float &span_far, bool &use_span)
+                       const std::vector<double> &hm, const TuneCand &c, cudaStream_t s, int &option,
+                       double &est_ms, float &span_far, bool &use_span)
 {
     ml_field_desc dc = d;
     dc.lens_x = hx.data();
@@ -959,47 +960,71 @@ ml_status measure_grid(const ml_field_desc &d, const std::vector<double> &hx, co
     const double create_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     if (st == ML_OK) {
         // the time per ray is the slope between slices of n and 2n rays, which
-        // cancels a launch's fixed start and tail
+        // cancels a launch's fixed start and tail (long enough that these, some
+        // tens of microseconds, stay a few per cent of it)
         const Geo &g = f->g;
         const uint64_t total = (uint64_t)g.n3x * (uint64_t)g.n3y;
-        // (long enough that a launch's start and tail, some tens of microseconds,
-        // stay a few per cent of it)
         const uint64_t n = std::min<uint64_t>(total / 2, std::max<uint64_t>({500000000ull, total / 100,
                                                                              std::min<uint64_t>(total / 32, 4000000000ull)}));
         const uint64_t r0 = (total - 2 * n) / 2;
         const uint64_t warm = std::min<uint64_t>(n, 64ull * (uint64_t)g.n3x);
-        // the certified walk is timed with lens columns spanned beyond five
-        // distances about a factor 1.6 apart around the library's rule (where
-        // spanning pays differs between fields), and without spans (the per-ray
-        // kernel); the fastest counts
-        const bool certified = f->desc.walk == ML_WALK_CERTIFIED && f->g.deposit == ML_DEPOSIT_NGP;
-        constexpr int NV = 6;
-        const float rule = (float)span_far_of(mean_abs_mass(hm), g.l3x, g.dpx);
-        const float fars[NV] = {rule, 2.5f * rule, 1.6f * rule, 0.6f * rule, 0.4f * rule, rule};
-        double best_ray = -1.0;
-        for (int v = 0; v < (certified ? NV : 1) && st == ML_OK; ++v) {
-            f->span_far = fars[v];
-            f->use_span = v < NV - 1;
+        // milliseconds per ray over slices of m and 2m rays, each at `parts`
+        // places spread over the lattice
+        auto slope = [&](uint64_t m, int parts, double &per_ray) {
             float ms[2] = {0.f, 0.f};
-            st = ml_shoot_rays(f, r0, r0 + warm, s);
-            for (int q = 0; q < 2 && st == ML_OK && n > 0; ++q) {
+            for (int q = 0; q < 2 && st == ML_OK && m > 0; ++q) {
+                const uint64_t len = (q + 1) * m;
                 ce = cudaEventRecord(e1, s);
-                if (ce == cudaSuccess) st = ml_shoot_rays(f, r0, r0 + (q + 1) * n, s);
+                for (int k = 0; k < parts && st == ML_OK; ++k) {
+                    const uint64_t mid = (uint64_t)((double)total * (k + 0.5) / parts);
+                    const uint64_t at = std::min(total - len, mid > len / 2 ? mid - len / 2 : 0);
+                    if (ce == cudaSuccess) st = ml_shoot_rays(f, at, at + len, s);
+                }
                 if (st == ML_OK && ce == cudaSuccess) ce = cudaEventRecord(e2, s);
                 if (st == ML_OK && ce == cudaSuccess) ce = cudaEventSynchronize(e2);
                 if (st == ML_OK && ce == cudaSuccess) ce = cudaEventElapsedTime(&ms[q], e1, e2);
                 if (st == ML_OK && ce != cudaSuccess) st = cuda_fail(ce, "grid autotuner");
             }
-            const double per_ray = n > 0 ? std::max(0.0, (double)(ms[1] - ms[0])) / (double)n : 0.0;
+            per_ray = m > 0 ? std::max(0.0, (double)(ms[1] - ms[0])) / ((double)m * parts) : 0.0;
+        };
+        // the certified walk is timed with lens columns spanned beyond five
+        // distances about a factor 1.6 apart around the library's rule (where
+        // spanning pays differs between fields), and without spans (the per-ray
+        // kernel); the fastest counts.  Later candidates try the neighbours of
+        // the last one's best.
+        const bool certified = f->desc.walk == ML_WALK_CERTIFIED && f->g.deposit == ML_DEPOSIT_NGP;
+        constexpr int NV = 6;
+        const float rule = (float)span_far_of(mean_abs_mass(hm), g.l3x, g.dpx);
+        const float fars[NV] = {0.4f * rule, 0.6f * rule, rule, 1.6f * rule, 2.5f * rule, rule};
+        double best_ray = -1.0;
+        int best_v = 0;
+        st = ml_shoot_rays(f, r0, r0 + warm, s);
+        for (int v = 0; v < (certified ? NV : 1) && st == ML_OK; ++v) {
+            if (certified && option >= 0 && abs(v - option) > 1) continue;
+            f->span_far = fars[v];
+            f->use_span = v < NV - 1;
+            double per_ray = 0.0;
+            slope(n, 1, per_ray);
             if (st == ML_OK && (best_ray < 0.0 || per_ray < best_ray)) {
                 best_ray = per_ray;
-                span_far = fars[v];
-                use_span = v < NV - 1;
+                best_v = v;
             }
             if (st == ML_OK && getenv("ML_TUNE_LOG"))
-                fprintf(stderr, "ml tune:   create %.2f ms, %.3g and %.3g of %.3g rays in %.3f and %.3f ms (%s %g)\n",
-                        create_ms, (double)n, (double)(2 * n), (double)total, ms[0], ms[1],
+                fprintf(stderr, "ml tune:   create %.2f ms, %.4f ps a ray over %.3g of %.3g (%s %g)\n", create_ms,
+                        per_ray * 1e9, (double)n, (double)total,
                         certified && v < NV - 1 ? "lens columns spanned beyond" : "no spans", fars[v]);
+        }
+        // the candidates are compared at two heights of the lattice: level-1
+        // cells are a tenth of it high, and their lenses differ (Table-1 field,
+        // 1e11 rays: by one slice at the centre level-2 cells of 40 x 20 came
+        // first, whose whole lattice takes 19.6 ms; by two heights 20 x 5 in a
+        // narrower level 1, 14.7-15.0 ms)
+        if (st == ML_OK) {
+            f->span_far = span_far = fars[best_v];
+            f->use_span = use_span = !certified || best_v < NV - 1;
+            option = certified ? best_v : -1;
+            const uint64_t m = std::min<uint64_t>(total / 4, n);
+            slope(m, 2, best_ray);
         }
         if (st == ML_OK) est_ms = create_ms + best_ray * (double)total;
     }
