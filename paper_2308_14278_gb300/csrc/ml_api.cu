@@ -428,16 +428,18 @@ double mean_abs_mass(const std::vector<double> &hm)
 }
 
 // Shooting time per ray of the certified walk, picoseconds: a least-squares
-// fit to 210 grids of the paper-scale field, the Table-1 field and four of
-// the batched maps (level-1 cells of 1 to 1/(2 sqrt 2) times Eq. 10's, level-2
-// cells of 11 to 2806 rays along a row, p = 3 to 16), each at its best lens
-// distance; 12 % rms.  The constant is the fields' mean (0.05 to 0.28, by
-// their runs' lengths).  A column's set-up and its first and last window carry
-// the cost, so long level-2 cells with a high order pay.
+// fit to whole maps of seven of the batched fields over 199 grids (level-1
+// cells of 1 to 1/(2 sqrt 2) times Eq. 10's, level-2 cells of 21 to 928 rays
+// along a row, p = 4 to 16), each at its best lens distance; 8 % rms.  The
+// constant is the fields' mean (it differs by their runs' lengths).  A column's
+// set-up and its first and last window carry the cost, so long level-2 cells
+// with a high order pay.  The seven maps take 12.9 ms on the grids that it
+// chooses and 12.3 on the best of all; an earlier fit to centred slices, with
+// near lenses and orders cheaper per ray and dearer per column, chose grids
+// that take 14.9.
 double span_cost_ps(int P, double near_per_ray, double n2x)
 {
-    return 0.187 + 0.0335 * near_per_ray + 0.0072 * P +
-           (16.8 + 0.79 * P + 1.87 * near_per_ray) / std::max(1.0, n2x);
+    return 0.15 + 0.09 * near_per_ray + 0.016 * P + 21.5 / std::max(1.0, n2x);
 }
 
 // The share of columns that the certified walk spans: no near lens within
