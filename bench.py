@@ -41,13 +41,17 @@ SMS, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 HBM_GBS_FALLBACK = 6790.0
 # DRAM bytes per ray of the certified counting kernel, from one ncu capture
 # per workload (dram__bytes_read.sum + dram__bytes_write.sum of one launch
-# over a centred slice of the lattice at the autotuned grid: 2e10 rays of the
-# paper-scale map, 2e9 of the Table-1 fold field, whose 84 MB map stays in
-# L2), valid for the kernel sources whose code (comments and blank space left
-# out, code_hash) has these sha1 prefixes only.
+# over a centred slice of the lattice: 2e10 rays of the paper-scale map, level-2
+# (20, 10), and 2e9 of the Table-1 fold field, level-2 (20, 10), whose 84 MB map
+# stays in L2).  They were taken on the walk before its bound was taken once per
+# column; on the present sources the same launches move 209.2 + 252.6 MB (5 %
+# less) and 23.8 + 0 MB, so the figures are upper ends.  They hold for the kernel
+# sources whose code (comments and blank space left out, code_hash) has these
+# sha1 prefixes only.
 TRAFFIC_BYTES_PER_RAY = {"paper": (216.402944e6 + 269.967104e6) / 2.0e10,
                          "fold": (23.782144e6 + 512.0) / 2.0e9}
-TRAFFIC_SOURCES = {"ml_shoot.cu": "48c686ae", "ml_internal.cuh": "4806c1e0", "ml_task.cuh": "3d1d5136"}
+TRAFFIC_SOURCES = {"ml_shoot.cu": "4e7a0a4c", "ml_internal.cuh": "600f1be7", "ml_task.cuh": "891fab5e",
+                   "ml_walk.cuh": "b83910bc"}
 
 
 def code_hash(text: str) -> str:
@@ -61,10 +65,10 @@ def code_hash(text: str) -> str:
 
 
 # The library's kernels in one field build: k_lens_cells, k_scan, k_scatter,
-# k_p_bound, k_lens_l1, k_outer_csr, k_box_p2l, k_sub_p2l, k_node_shift,
-# k_node_finalize.  A step adds the shooting launches, mu and the light curves
-# (the fold step: the two peak kernels; the differentiable step: the CIC
-# forward, mu, and k_adj_rays, k_adj_far, k_adj_unsort).
+# k_p_bound, k_plan_max, k_lens_l1, k_outer_csr, k_box_p2l_df, k_sub_p2l_df,
+# k_node_records.  A step adds the shooting launches, mu and the light curves
+# (the fold step: k_peaks, k_peak_bins and k_peak_stats; the differentiable
+# step: the CIC forward, mu, and k_adj_rays, k_adj_far, k_adj_unsort).
 BUILD_KERNELS = 10
 # distance bins of the fold step's peak statistics: beta_x from 0.02 to 63 theta_E,
 # four per decade (the fold map spans beta_x in [0, 40])
@@ -507,7 +511,7 @@ def run_ours(args, rank, world, local):
                        "conserved": n_local == expected_local},
         "gpu_launches": int(args.steps * (BUILD_KERNELS + stats["launches"] + 1
                                           + (2 if consumer else 0)
-                                          + (4 if args.workload == "fold" and consumer else 0))),
+                                          + (3 if args.workload == "fold" and consumer else 0))),
     }
     clk_sum = clk.summary()
     if clk_sum:
