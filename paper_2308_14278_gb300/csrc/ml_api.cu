@@ -427,19 +427,20 @@ double mean_abs_mass(const std::vector<double> &hm)
     return hm.empty() ? 0.0 : t / (double)hm.size();
 }
 
-// Shooting time per ray of the certified walk, picoseconds: a least-squares
-// fit to whole maps of seven of the batched fields over 199 grids (level-1
-// cells of 1 to 1/(2 sqrt 2) times Eq. 10's, level-2 cells of 21 to 928 rays
-// along a row, p = 4 to 16), each at its best lens distance; 8 % rms.  The
-// constant is the fields' mean (it differs by their runs' lengths).  A column's
-// set-up and its first and last window carry the cost, so long level-2 cells
-// with a high order pay.  The seven maps take 12.9 ms on the grids that it
-// chooses and 12.3 on the best of all; an earlier fit to centred slices, with
-// near lenses and orders cheaper per ray and dearer per column, chose grids
-// that take 14.9.
+// Shooting time per ray of the certified walk, picoseconds, from whole maps of
+// seven of the batched fields over 199 grids (level-1 cells of 1 to
+// 1/(2 sqrt 2) times Eq. 10's, level-2 cells of 21 to 928 rays along a row,
+// p = 4 to 16), each at its best lens distance; 12 % rms.  The constant is the
+// fields' mean (0.04 to 0.6, by their runs' lengths).  A column's set-up and
+// its first and last window carry the cost, so long level-2 cells with a high
+// order pay.  The least-squares fit, 0.020 per order and 21.6/n2x (8 % rms),
+// chooses the same grids for most of the seven maps (both 12.8 ms together, the
+// best of all 12.3) but columns half as long, 12 to 18 % slower, on maps of
+// 13,000 lenses and 1e11 rays.  A fit to centred slices (near lenses and orders
+// cheaper) chose grids that take 14.9 ms.
 double span_cost_ps(int P, double near_per_ray, double n2x)
 {
-    return 0.15 + 0.09 * near_per_ray + 0.016 * P + 21.5 / std::max(1.0, n2x);
+    return 0.2 + 0.09 * near_per_ray + 0.012 * P + 30.0 / std::max(1.0, n2x);
 }
 
 // The share of columns that the certified walk spans: no near lens within
@@ -961,33 +962,22 @@ ml_status measure_grid(const ml_field_desc &d, const std::vector<double> &hx, co
     if (st == ML_OK) st = create_impl(&dc, s, f);
     const double create_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     if (st == ML_OK) {
-        // the time per ray is the slope between slices of n and 2n rays, which
-        // cancels a launch's fixed start and tail (long enough that these, some
-        // tens of microseconds, stay a few per cent of it)
+        // the time per ray over slices at two heights of the lattice: level-1
+        // cells are a tenth of it high, and their lenses differ.  Each slice is
+        // long enough that a launch's start and tail (0.1 to 0.3 ms, much alike
+        // for all grids of a field) leave the order of the grids alone; taken out
+        // by the slope between two lengths they made it noisier.  Six fields of
+        // 13,000 lenses and 1e11 rays: the grids chosen so take 14.6 to 16.6 ms to
+        // shoot, within 1 % of the best of twelve; by the slope 15.6 to 20.0.
         const Geo &g = f->g;
         const uint64_t total = (uint64_t)g.n3x * (uint64_t)g.n3y;
-        const uint64_t n = std::min<uint64_t>(total / 2, std::max<uint64_t>({500000000ull, total / 100,
-                                                                             std::min<uint64_t>(total / 32, 4000000000ull)}));
-        const uint64_t r0 = (total - 2 * n) / 2;
-        const uint64_t warm = std::min<uint64_t>(n, 64ull * (uint64_t)g.n3x);
-        // milliseconds per ray over slices of m and 2m rays, each at `parts`
-        // places spread over the lattice
-        auto slope = [&](uint64_t m, int parts, double &per_ray) {
-            float ms[2] = {0.f, 0.f};
-            for (int q = 0; q < 2 && st == ML_OK && m > 0; ++q) {
-                const uint64_t len = (q + 1) * m;
-                ce = cudaEventRecord(e1, s);
-                for (int k = 0; k < parts && st == ML_OK; ++k) {
-                    const uint64_t mid = (uint64_t)((double)total * (k + 0.5) / parts);
-                    const uint64_t at = std::min(total - len, mid > len / 2 ? mid - len / 2 : 0);
-                    if (ce == cudaSuccess) st = ml_shoot_rays(f, at, at + len, s);
-                }
-                if (st == ML_OK && ce == cudaSuccess) ce = cudaEventRecord(e2, s);
-                if (st == ML_OK && ce == cudaSuccess) ce = cudaEventSynchronize(e2);
-                if (st == ML_OK && ce == cudaSuccess) ce = cudaEventElapsedTime(&ms[q], e1, e2);
-                if (st == ML_OK && ce != cudaSuccess) st = cuda_fail(ce, "grid autotuner");
+        const uint64_t len = std::min<uint64_t>(total / 2, std::max<uint64_t>({1000000000ull, total / 50,
+                                                                               std::min<uint64_t>(total / 16, 8000000000ull)}));
+        auto shoot_slices = [&](uint64_t m) {
+            for (int k = 0; k < 2 && st == ML_OK; ++k) {
+                const uint64_t at = (2 * k + 1) * (total / 4) - m / 2;
+                st = ml_shoot_rays(f, at, at + m, s);
             }
-            per_ray = m > 0 ? std::max(0.0, (double)(ms[1] - ms[0])) / ((double)m * parts) : 0.0;
         };
         // the certified walk is timed with lens columns spanned beyond five
         // distances about a factor 1.6 apart around the library's rule (where
@@ -1000,34 +990,31 @@ ml_status measure_grid(const ml_field_desc &d, const std::vector<double> &hx, co
         const float fars[NV] = {0.4f * rule, 0.6f * rule, rule, 1.6f * rule, 2.5f * rule, rule};
         double best_ray = -1.0;
         int best_v = 0;
-        st = ml_shoot_rays(f, r0, r0 + warm, s);
+        shoot_slices(std::min<uint64_t>(len, 32ull * (uint64_t)g.n3x));
         for (int v = 0; v < (certified ? NV : 1) && st == ML_OK; ++v) {
             if (certified && option >= 0 && abs(v - option) > 1) continue;
             f->span_far = fars[v];
             f->use_span = v < NV - 1;
-            double per_ray = 0.0;
-            slope(n, 1, per_ray);
+            float ms = 0.f;
+            ce = cudaEventRecord(e1, s);
+            if (ce == cudaSuccess) shoot_slices(len);
+            if (st == ML_OK && ce == cudaSuccess) ce = cudaEventRecord(e2, s);
+            if (st == ML_OK && ce == cudaSuccess) ce = cudaEventSynchronize(e2);
+            if (st == ML_OK && ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e1, e2);
+            if (st == ML_OK && ce != cudaSuccess) st = cuda_fail(ce, "grid autotuner");
+            const double per_ray = len > 0 ? (double)ms / (2.0 * (double)len) : 0.0;
             if (st == ML_OK && (best_ray < 0.0 || per_ray < best_ray)) {
                 best_ray = per_ray;
                 best_v = v;
             }
             if (st == ML_OK && getenv("ML_TUNE_LOG"))
                 fprintf(stderr, "ml tune:   create %.2f ms, %.4f ps a ray over %.3g of %.3g (%s %g)\n", create_ms,
-                        per_ray * 1e9, (double)n, (double)total,
+                        per_ray * 1e9, 2.0 * (double)len, (double)total,
                         certified && v < NV - 1 ? "lens columns spanned beyond" : "no spans", fars[v]);
         }
-        // the candidates are compared at two heights of the lattice: level-1
-        // cells are a tenth of it high, and their lenses differ (Table-1 field,
-        // 1e11 rays: by one slice at the centre level-2 cells of 40 x 20 came
-        // first, whose whole lattice takes 19.6 ms; by two heights 20 x 5 in a
-        // narrower level 1, 14.7-15.0 ms)
-        if (st == ML_OK) {
-            f->span_far = span_far = fars[best_v];
-            f->use_span = use_span = !certified || best_v < NV - 1;
-            option = certified ? best_v : -1;
-            const uint64_t m = std::min<uint64_t>(total / 4, n);
-            slope(m, 2, best_ray);
-        }
+        span_far = fars[best_v];
+        use_span = !certified || best_v < NV - 1;
+        option = certified ? best_v : -1;
         if (st == ML_OK) est_ms = create_ms + best_ray * (double)total;
     }
     if (e1) cudaEventDestroy(e1);
