@@ -334,11 +334,11 @@ bool rays_inside_sheet(const Geo &g)
 // the long side of the level-1 cells shrinks the expansion radius, so a lower
 // Taylor order meets the same truncation bound, at the price of more nodes to
 // build; smaller level-1 cells shorten the near lists, at the price of more
-// cells and nodes.  The tuner evaluates level-1 scales (1, 1/sqrt 2, 1/2 of
-// Eq. 10's size, unless the caller fixed L1) times (l2_sub_x, l2_sub_y)
+// cells and nodes.  The tuner evaluates level-1 scales (1, 1/sqrt 2, 1/2 and
+// 1/(2 sqrt 2) of Eq. 10's size, unless the caller fixed L1) times (l2_sub_x, l2_sub_y)
 // candidates with their rigorous bound (one p_bound launch each) and their
 // mean near-list length, and ranks them by a cost model of GB300 measurements:
-//   time = rays * ray_cost(P, near) + nodes * (P + 1) * node_cost,
+//   time = rays * ray_cost(P, near) + nodes * (P + 1) * node_cost + cells * cell_cost,
 // the field's build plus one shot of all its rays.
 
 // Shooting time per ray of the mixed kernel on the whole GB300, in
@@ -968,7 +968,7 @@ ml_status measure_grid(const ml_field_desc &d, const std::vector<double> &hx, co
         // for all grids of a field) leave the order of the grids alone; taken out
         // by the slope between two lengths they made it noisier.  Six fields of
         // 13,000 lenses and 1e11 rays: the grids chosen so take 14.6 to 16.6 ms to
-        // shoot, within 1 % of the best of twelve; by the slope 15.6 to 20.0.
+        // shoot, within 3 % of the best of twelve; by the slope 15.6 to 20.0.
         const Geo &g = f->g;
         const uint64_t total = (uint64_t)g.n3x * (uint64_t)g.n3y;
         const uint64_t len = std::min<uint64_t>(total / 2, std::max<uint64_t>({1000000000ull, total / 50,
