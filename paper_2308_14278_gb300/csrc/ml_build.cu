@@ -576,6 +576,7 @@ struct Hier {
     int64_t NBx, NBy;                // boxes across the level-1 grid
     int64_t nsx, nsy;                // sub-blocks per level-1 cell side
     double hB;                       // box scale (half-diagonal)
+    int32_t parts;                   // lens partitions per box of the pair build (at most HPARTS)
 };
 
 // Box size: the box series costs (boxes) x (lenses) terms and the sub-block
@@ -598,6 +599,12 @@ __host__ __device__ inline Hier hier_of(const Geo &g)
     h.NBx = (g.N1x + h.bxn - 1) / h.bxn;
     h.NBy = (g.N1y + h.byn - 1) / h.byn;
     h.hB = 0.5 * sqrt((double)(h.bxn * h.bxn) * g.l1x * g.l1x + (double)(h.byn * h.byn) * g.l1y * g.l1y);
+    // a partition ends in a reduction of all orders over its block, so no more
+    // of them than give the GPU 912 blocks, two for each of its 456 slots
+    // (always 16: the Table-1 field's build 6.11 ms, now 5.82; 13,000 lenses on
+    // 1.23 theta_E cells 1.37 -> 1.33; at 456 blocks the latter takes 1.46)
+    h.parts = HPARTS;
+    while (h.parts > 1 && h.NBx * h.NBy * (h.parts / 2) >= 912) h.parts /= 2;
     return h;
 }
 
@@ -1052,7 +1059,8 @@ __global__ void __launch_bounds__(32 * SUB_WARPS, 3) k_sub_p2l(Geo g, LensTable 
 
 // ---- the mixed mode's build on pairs of floats --------------------------------
 
-// 1. box series (k_box_p2l; 2.16 -> 0.65 ms on the Table-1 field).
+// 1. box series (k_box_p2l; 2.16 -> 0.48 ms on the Table-1 field), the lenses in
+// h.parts partitions.
 __global__ void __launch_bounds__(128) k_box_p2l_df(Geo g, LensTable L, const int2 *__restrict__ lc, Hier h,
                                                     float4 *__restrict__ part)
 {
@@ -1063,7 +1071,7 @@ __global__ void __launch_bounds__(128) k_box_p2l_df(Geo g, LensTable L, const in
     const df hB = df_of(h.hB), ihB = df_of(1.0 / h.hB);
     PairSums acc;
     acc.zero();
-    const int64_t k0 = L.n * blockIdx.y / HPARTS, k1 = L.n * (blockIdx.y + 1) / HPARTS;
+    const int64_t k0 = L.n * blockIdx.y / h.parts, k1 = L.n * (blockIdx.y + 1) / h.parts;
     const int bxn = (int)h.bxn, byn = (int)h.byn, iBx = (int)Bx, iBy = (int)By;
     for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
         const int2 c = lc[k];
@@ -1157,7 +1165,7 @@ __global__ void __launch_bounds__(32 * SUB_WARPS, 3) k_sub_p2l_df(Geo g, LensTab
     const int64_t b = By * h.NBx + Bx;
     for (int j = lane; j <= HP; j += 32) {
         df vr{0.f, 0.f}, vi{0.f, 0.f};
-        for (int q = 0; q < HPARTS; ++q) {
+        for (int q = 0; q < h.parts; ++q) {
             const float4 v = part[(b * HPARTS + q) * (HP + 1) + j];
             vr = df_add(vr, df{v.x, v.y});
             vi = df_add(vi, df{v.z, v.w});
@@ -1487,7 +1495,7 @@ cudaError_t launch_coeffs_hier(const Geo &g, const LensTable &L, double *coef64,
         // sub-block order
         float4 *pt = reinterpret_cast<float4 *>(part);
         float2 *sh = reinterpret_cast<float2 *>(sub), *sl = sh + ns * (HP + 1);
-        k_box_p2l_df<<<gb, 128, 0, s>>>(g, L, lc, h, pt);
+        k_box_p2l_df<<<dim3((unsigned)nb, (unsigned)h.parts), 128, 0, s>>>(g, L, lc, h, pt);
         k_sub_p2l_df<<<gs, 32 * SUB_WARPS, 0, s>>>(g, L, lc, h, pt, ostart, oidx, sh, sl, j64, (int64_t)ns);
         switch (g.p) {
 #define ML_NODE_CASE(P) case P: run_node_records<P>(g, h, sh, sl, j64, nodes, s); break;

@@ -387,11 +387,13 @@ def test_fp64_modes_over_lattice_widths_and_ranges(ml, precision, n3x, n3y, mass
 
 
 @pytest.mark.parametrize("l1,l2_sub,p", [((6.0, 6.0), (20, 20), 0), ((9.0, 2.0), (10, 7), 0), ((2.0, 7.0), (5, 11), 0),
-                                         ((5.0, 4.0), (3, 1), 16), ((4.0, 4.0), (1, 1), 12), ((3.0, 3.0), (40, 40), 1)])
+                                         ((5.0, 4.0), (3, 1), 16), ((4.0, 4.0), (1, 1), 12), ((3.0, 3.0), (40, 40), 1),
+                                         ((0.15, 0.15), (2, 2), 0), ((0.06, 0.06), (2, 2), 0), ((0.02, 0.02), (1, 1), 0)])
 def test_mixed_hierarchical_records_match_the_direct_build(ml, l1, l2_sub, p):
     """The mixed mode's node records from the series in pairs of floats against
     those of the FP64 sum over all far lenses at every node, on cells that split
-    into one, evenly and unevenly many sub-blocks.  Both round the node's place
+    into one, evenly and unevenly many sub-blocks, and on cells so many that the
+    box series' lenses come in fewer partitions.  Both round the node's place
     within its pixel to 2^-24 and c_n to FP32 (the series' coefficients carry
     about 2e-6): 1e-5 of a pixel.  A ray's position off its node's base is an
     FP32 number X whose last bit, 2^-23 |X|, may then differ too; the bases lie
