@@ -1100,7 +1100,7 @@ __global__ void __launch_bounds__(128) k_box_p2l_df(Geo g, LensTable L, const in
 // remainders, j64 the length of c_0's pair sum.  One warp per sub-block: the
 // FP64 form took 9.5 ms for the Table-1 field's 54,579 sub-blocks (about 175
 // lenses each), bound by the FP64 pipe; all orders in pairs 4.8 ms (two warps
-// per scheduler by its registers), HD orders in pairs 2.0 ms, bound by issue.
+// per scheduler by its registers), HD orders in pairs 1.9 ms, bound by issue.
 __global__ void __launch_bounds__(32 * SUB_WARPS, 3) k_sub_p2l_df(Geo g, LensTable L, const int2 *__restrict__ lc,
                                                              Hier h, const float4 *__restrict__ part,
                                                              const int32_t *__restrict__ ostart,
