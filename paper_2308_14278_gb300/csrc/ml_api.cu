@@ -386,6 +386,9 @@ double ray_cost_ps(int P, double near_per_ray)
 // field's kernels (10.9M nodes of order 4 in 1.16 ms; 54,579 cells in 5.5 ms).
 constexpr double kNodeCostNs = 0.022;
 constexpr double kCellCostNs = 100.0;
+// The same for the maps of a batch (see cand_cost).
+constexpr double kBatchNodeCostNs = 0.12;
+constexpr double kBatchCellCostNs = 400.0;
 
 struct GridChoice {
     int sx = 20, sy = 20, p = 0;
@@ -451,11 +454,20 @@ double span_share(double near_per_ray, double far, double l1x, double l1y)
     return exp(-near_per_ray * 3.14159265358979 * far * far / (9.0 * l1x * l1y));
 }
 
-double cand_cost(const TuneCand &c, int P)
+// `batch`: a map of a batch, whose grid is not measured afterwards.  Its build
+// weighs as it did when those grids were set: they fix which rays lie within a
+// rounding of a pixel edge, and so the batch's counts.  Cheaper builds and the
+// certified walk's cost would favour columns four times as long (1e9 to 1e10
+// rays on 4096 x 4096 pixels: 300 to 550 rays at p = 8 to 12 instead of 42 to
+// 129 at p = 4 to 6), whose FP32 positions, larger numbers of pixels from the
+// node, lie 27 % further off the FP64 ones (median of 16 maps 9.3e-8 against
+// 7.3e-8 pixels).
+double cand_cost(const TuneCand &c, int P, bool batch = false)
 {
     const double f = c.walk == ML_WALK_CERTIFIED ? c.span_frac : 0.0;
     const double ps = f * span_cost_ps(P, c.near_per_ray, c.n2x) + (1.0 - f) * ray_cost_ps(P, c.near_per_ray);
-    return c.rays * ps * 1e-3 + c.nodes * (P + 1) * kNodeCostNs + c.cells * kCellCostNs;   // ns
+    const double node = batch ? kBatchNodeCostNs : kNodeCostNs, cell = batch ? kBatchCellCostNs : kCellCostNs;
+    return c.rays * ps * 1e-3 + c.nodes * (P + 1) * node + c.cells * cell;   // ns
 }
 
 uint64_t mix64(uint64_t h, uint64_t v)
@@ -628,12 +640,12 @@ ml_status tune_candidates(uint64_t key, const ml_field_desc &d, const std::vecto
 }
 
 // Cheapest candidate of a single field (its own order).
-GridChoice best_single(const std::vector<TuneCand> &cands)
+GridChoice best_single(const std::vector<TuneCand> &cands, bool batch)
 {
     GridChoice best;
     bool found = false;
     for (const TuneCand &c : cands) {
-        double cost = cand_cost(c, c.P);
+        double cost = cand_cost(c, c.P, batch);
         if (!found || cost < best.cost) {
             best.sx = c.sx; best.sy = c.sy; best.p = c.P; best.cost = cost;
             best.l1x = c.l1x; best.l1y = c.l1y;
@@ -663,7 +675,7 @@ ml_status tune_grid(const ml_field_desc &d, const std::vector<double> &hx, const
     const uint64_t key = tune_key(d, hx, hy, hm);
     ml_status st = tune_candidates(key, d, hx, hy, hm, dx, dy, dm, s, cands);
     if (st != ML_OK) return st;
-    best = cands.empty() ? GridChoice() : best_single(cands);
+    best = cands.empty() ? GridChoice() : best_single(cands, !measure);
     if (!measure || cands.size() < 2) return ML_OK;
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
@@ -1255,8 +1267,11 @@ ml_status batch_create_impl(const ml_field_desc *descs, int32_t n, int32_t tpm, 
         }
         GridChoice best;
         // the batch's grids come from the cost model alone (timing every map
-        // would cost more than it saves)
-        if (e == cudaSuccess) st = tune_grid(plan[i], hx, hy, hm, dx, dy, dm, s, false, best);
+        // would cost more than it saves), as the per-ray walk's costs rank
+        // them (see cand_cost)
+        ml_field_desc model = plan[i];
+        model.walk = ML_WALK_PER_RAY;
+        if (e == cudaSuccess) st = tune_grid(model, hx, hy, hm, dx, dy, dm, s, false, best);
         cudaFreeAsync(dx, s);
         cudaFreeAsync(dy, s);
         cudaFreeAsync(dm, s);

@@ -67,6 +67,18 @@ def test_tuned_batch_groups_orders_and_matches_single_maps(ml):
     b.close()
 
 
+def test_batch_grids_stay_as_they_were(ml):
+    """The grid and order of a batch's tuned maps fix its counts (rays within a
+    rounding of a pixel edge fall to either side): subdivisions, order and
+    rays per level-2 column of four maps, as they have always been chosen."""
+    ws = inputs.batched_maps(16, 5, 4096, (1e9, 1e10), 10)
+    want = {0: (20, 10, 6, 67), 6: (60, 10, 4, 46), 9: (40, 20, 4, 69), 15: (60, 10, 5, 129)}
+    b = ml.Batch([ml.make_desc(ws[i], tune=True) for i in want])
+    got = [tuple(b.info(q)[k] for k in ("l2_sub_x", "l2_sub_y", "taylor_p", "n2x")) for q in range(len(want))]
+    assert got == list(want.values())
+    b.close()
+
+
 def test_batch_graph_replay_and_direct_launch_agree(ml):
     ws, descs, tracks = _small_batch(ml, n_maps=4)
     b = ml.Batch(descs, tracks=tracks, n_samples=64, sigma_px=0.5)
