@@ -1323,7 +1323,9 @@ ml_status batch_create_impl(const ml_field_desc *descs, int32_t n, int32_t tpm, 
     size_t mu_total = 0;
     for (int32_t i = 0; i < n; ++i) {
         b->mu_off.push_back(mu_total);
-        mu_total += (size_t)b->fields[i]->g.mnx * b->fields[i]->g.mny;
+        // every map starts on a 16-byte boundary (launch_mu stores four pixels
+        // at a time), also after one of an odd number of pixels
+        mu_total += ((size_t)b->fields[i]->g.mnx * b->fields[i]->g.mny + 3) / 4 * 4;
     }
     for (int32_t i = 0; i < n; ++i) {
         const int P = b->fields[i]->g.p;

@@ -79,6 +79,24 @@ def test_batch_grids_stay_as_they_were(ml):
     b.close()
 
 
+@pytest.mark.parametrize("px", [(33, 21), (1, 1), (50, 31), (63, 65)])
+def test_batch_maps_of_odd_sizes(ml, px):
+    """Maps whose pixel counts are 1, 2 and 3 beyond a multiple of four: every
+    map's mu starts on a 16-byte boundary and is the single map's."""
+    ws = inputs.batched_maps(n_maps=4, seed=3, map_px=64, ray_range=(1e5, 1e6), tracks_per_map=2)
+    for w in ws[:3]:
+        w.map_n, w.n_av = px, 2e5 / (px[0] * px[1])
+    b = ml.Batch([ml.make_desc(w, precision=ml.PREC_MIXED) for w in ws])
+    b.run()
+    for i, w in enumerate(ws):
+        f = ml.Field(w, precision=ml.PREC_MIXED)
+        f.shoot()
+        assert np.array_equal(b.counts(i).cpu().numpy(), f.counts().cpu().numpy()), i
+        assert np.array_equal(b.mu(i).cpu().numpy(), f.mu().cpu().numpy()), i
+        f.close()
+    b.close()
+
+
 def test_batch_graph_replay_and_direct_launch_agree(ml):
     ws, descs, tracks = _small_batch(ml, n_maps=4)
     b = ml.Batch(descs, tracks=tracks, n_samples=64, sigma_px=0.5)
