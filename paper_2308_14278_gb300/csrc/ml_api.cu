@@ -1082,15 +1082,33 @@ ShootArgs make_args(const ml_field *f)
     return a;
 }
 
-// Task decomposition of rays [b, e) for the mixed kernel.  A task's level-2
-// columns (about 2048 rays along a row, within one level-1 cell) share the
-// staging of its near lenses.  Small launches take fewer columns per task,
-// down to one, so that about eight tasks come on each of the GPU's 24 resident
-// warps per SM: a launch of a few hundred tasks otherwise leaves most warps
-// idle, and a task next to a lens takes several times one without (the
-// differentiable step of 4e8 rays at 2, 4, 8 and 16 tasks a warp: 3.21, 3.10,
-// 2.84 and 2.84 ms).
-void set_tasks(ShootArgs &a, const Geo &g, int64_t b, int64_t e, int num_sms)
+// Microseconds a warp takes for one ray of a level-2 column next to a lens,
+// where each ray is evaluated, before its near lenses' share: counts, cloud in
+// cell, adjoint.
+constexpr double kRayUsNgp = 0.25, kRayUsCic = 0.4, kRayUsAdj = 0.8;
+
+// Level-2 columns (of 32 rows) that rays [b, e) touch.
+int64_t launch_columns(const Geo &g, int64_t b, int64_t e)
+{
+    const int64_t gpb = (g.n1y + 31) / 32, jb = b / g.n3x, je = (e - 1) / g.n3x;
+    auto rg = [&](int64_t j) { return (j / g.n1y) * gpb + (j % g.n1y) / 32; };
+    return (rg(je) - rg(jb) + 1) * g.N2x;
+}
+
+// Task decomposition of rays [b, e) for the mixed kernels.  A task's level-2
+// columns (at most about 2048 rays along a row, within one level-1 cell) share
+// the staging of its near lenses.  `cols` columns of one launch in tasks of c:
+// every task costs the launch 6.8 ns (one counter for all warps, and the abort
+// flag in host memory), and its end waits for the last task, c columns next to
+// a lens: cols / c 6.8 ns + c t is least at c = sqrt(cols 6.8 ns / t), t = 2 us
+// and `ray_us` a ray, a quarter more per near lens.  By measurement over 70
+// lattices of 1e5 to 5e9 rays that c lies within 15 % of the fastest of 1, 2, 3,
+// 5, 10, 20 and 40 for most.  One
+// column a task up to eight tasks a resident warp (54,000 columns of 14 rays 392
+// us, 91 at ten; 212,000 of 4 rays 1446 us, 206 at ten) and always the most (112
+// columns of one ray 31 us instead of 14; the adjoint of 24,000 of 113 rays 1150
+// instead of 576) were each up to five times slower.
+void set_tasks(ShootArgs &a, const Geo &g, int64_t b, int64_t e, double ray_us, int64_t cols)
 {
     a.ray_begin = b;
     a.ray_end = e;
@@ -1100,8 +1118,12 @@ void set_tasks(ShootArgs &a, const Geo &g, int64_t b, int64_t e, int num_sms)
     a.groups_per_band = gpb;
     a.rg_first = rg(jb);
     a.n_rg = rg(je) - a.rg_first + 1;
-    const int64_t most = a.n_rg * g.N2x / (8 * 24 * (int64_t)num_sms);
-    const int64_t l2_per_cc = std::max<int64_t>(1, std::min({(int64_t)g.l2sx, (2048 + g.n2x - 1) / g.n2x, most}));
+    const double c = sqrt((double)cols * 6.8e-3 / (2.0 + ray_us * (1.0 + 0.25 * a.near_cap) * (double)g.n2x));
+    const int64_t most = std::min<int64_t>(g.l2sx, (2048 + g.n2x - 1) / g.n2x);
+    // (a level-1 cell's columns in up to three runs about equally long)
+    const int64_t runs = (int64_t)((double)g.l2sx / std::max(c, 1.0) + 0.5);
+    const int64_t want = runs <= 3 ? (g.l2sx + std::max<int64_t>(runs, 1) - 1) / std::max<int64_t>(runs, 1) : (int64_t)(c + 0.5);
+    const int64_t l2_per_cc = std::max<int64_t>(1, std::min(want, most));
     const int64_t cc_per_l1 = (g.l2sx + l2_per_cc - 1) / l2_per_cc;
     a.l2_per_cc = l2_per_cc;
     a.cc_per_l1 = cc_per_l1;
@@ -1342,10 +1364,15 @@ ml_status batch_create_impl(const ml_field_desc *descs, int32_t n, int32_t tpm, 
         const size_t m = gr.maps.size();
         std::vector<ShootArgs> args(m);
         std::vector<int64_t> base(m + 1, 0);
+        int64_t cols = 0;
+        for (int i : gr.maps) {
+            const Geo &g = b->fields[i]->g;
+            cols += launch_columns(g, 0, g.n3x * g.n3y);
+        }
         for (size_t q = 0; q < m; ++q) {
             ml_field *f = b->fields[gr.maps[q]];
             args[q] = make_args(f);
-            set_tasks(args[q], f->g, 0, f->g.n3x * f->g.n3y, f->num_sms);
+            set_tasks(args[q], f->g, 0, f->g.n3x * f->g.n3y, kRayUsNgp, cols);
             gr.near_cap = std::max(gr.near_cap, args[q].near_cap);
             base[q + 1] = base[q] + args[q].n_tasks;
         }
@@ -1587,7 +1614,8 @@ ml_status ml_shoot_rays(ml_field *f, uint64_t ray_begin, uint64_t ray_end, void 
         a.ray_begin = (int64_t)b;
         a.ray_end = (int64_t)e;
         if (g.precision == ML_PREC_MIXED) {
-            set_tasks(a, g, (int64_t)b, (int64_t)e, f->num_sms);
+            set_tasks(a, g, (int64_t)b, (int64_t)e, g.deposit == ML_DEPOSIT_NGP ? kRayUsNgp : kRayUsCic,
+                      launch_columns(g, (int64_t)b, (int64_t)e));
             ML_CK(cudaMemsetAsync(f->d_work, 0, sizeof(unsigned long long), s));
         }
         ML_CK(launch_shoot(a, f->num_sms, s));
@@ -1795,7 +1823,7 @@ ml_status ml_cic_backward_ex(ml_field *f, const float *dL_dM, double *grad_lens,
                                         grad_params, scale, f->num_sms, s));
         return ML_OK;
     }
-    set_tasks(a, g, 0, g.n3x * g.n3y, f->num_sms);
+    set_tasks(a, g, 0, g.n3x * g.n3y, kRayUsAdj, launch_columns(g, 0, g.n3x * g.n3y));
     const size_t n_mom = (size_t)(g.N2x * g.N2y) * (size_t)(g.p + 1);
     double *gs = nullptr;
     double2 *mom = nullptr;

@@ -440,6 +440,26 @@ def test_certified_walk_at_any_grid_and_lens_distance(ml, l2_sub, span_far):
     fp.close()
 
 
+@pytest.mark.parametrize("px,n_av,l1,l2_sub,most", [((1024, 1024), 20.0, 1.5, 10, 10000), ((1024, 1024), 4.0, 6.0, 40, 5000),
+                                                    ((64, 64), 2.0, 6.0, 10, 1000)])
+def test_launches_on_many_short_columns_take_few_tasks(ml, px, n_av, l1, l2_sub, most):
+    """Sparse lattices of tens of thousands of level-2 columns a few rays long: a
+    task takes several of them (each task costs the launch several nanoseconds),
+    and the counts do not depend on the cut: ranges of rays, whose launches cut
+    their tasks differently, add up to the whole."""
+    w = inputs.differentiable_field(3, 1000, n_av * px[0] * px[1], px[0])
+    f = _field(ml, w, precision=ml.PREC_MIXED, l1=(l1, l1), l2_sub=(l2_sub, l2_sub))
+    f.shoot()
+    whole = f.counts().cpu().numpy()
+    assert f.stats()["tasks"] <= most, f.stats()["tasks"]
+    f.clear()
+    cuts = [0, f.n_rays // 50, f.n_rays // 3 + 7, f.n_rays]
+    for r0, r1 in zip(cuts, cuts[1:]):
+        f.shoot(r0, r1)
+    assert np.array_equal(f.counts().cpu().numpy(), whole)
+    f.close()
+
+
 def test_mixed_map_matches_oracle_and_split_invariance(ml):
     w = _mixed_case(6)
     f = _field(ml, w, precision=ml.PREC_MIXED)
