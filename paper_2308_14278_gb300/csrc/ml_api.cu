@@ -489,6 +489,8 @@ uint64_t tune_key(const ml_field_desc &d, const std::vector<double> &hx, const s
     h = mix64(h, (uint64_t)d.map_nx); h = mix64(h, (uint64_t)d.map_ny);
     h = mix64(h, (uint64_t)d.taylor_p); h = mix64(h, (uint64_t)hx.size());
     h = mix64(h, (uint64_t)d.walk); h = mix64(h, (uint64_t)d.macro_mode);
+    // what picks the candidate list and what is built and timed
+    h = mix64(h, (uint64_t)d.deposit); h = mix64(h, (uint64_t)d.build);
     h = mix64(h, (uint64_t)d.sheet_shape); mixd(d.kappa0); mixd(d.d_x); mixd(d.d_y);
     // the lens arrays in four independent lanes (no serial dependency per word),
     // then the lanes into the parameter hash

@@ -157,3 +157,23 @@ def test_tuned_field_meets_bound_and_matches_oracle(ml):
         (info["l2_sub_x"], info["l2_sub_y"], info["n1x"], info["n1y"])
     f.close()
     f2.close()
+
+
+@pytest.mark.parametrize("first", ["counts", "cic"])
+def test_tuner_keeps_deposits_and_builds_apart(ml, first):
+    """Counted and cloud-in-cell fields of one workload are tuned from different
+    lists of level-2 subdivisions (the certified walk gains by long columns), and
+    the build is part of what is timed: a field's grid comes from its own mode's
+    list, whichever was created first."""
+    w = inputs.paper_map(7 if first == "cic" else 8, n_rays=4e8, map_px=512)
+    lists = {ml.DEPOSIT_NGP: ((5, 10, 20, 40), (5, 10, 20)), ml.DEPOSIT_CIC: ((20, 40, 60, 80, 120, 160), (10, 20))}
+    order = [ml.DEPOSIT_NGP, ml.DEPOSIT_CIC]
+    for dep in (order if first == "counts" else order[::-1]):
+        for build in (ml.BUILD_HIERARCHICAL, ml.BUILD_DIRECT):
+            f = ml.Field(w, deposit=dep, build=build, tune=True)
+            sub = sorted((f.info["l2_sub_x"], f.info["l2_sub_y"]))
+            assert f.info["build"] == build
+            assert sub[1] in lists[dep][0] and sub[0] in lists[dep][1], (dep, build, sub)
+            if dep == ml.DEPOSIT_NGP:
+                assert sub not in ([10, 20], [20, 20], [10, 40], [20, 40]), sub   # else the lists are not told apart
+            f.close()
