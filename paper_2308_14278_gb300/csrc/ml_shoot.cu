@@ -651,8 +651,9 @@ __device__ __forceinline__ void count_spans(const RowPoly<P> &rp, const SpanBoun
     CountSink sink{a.map_u32, (unsigned)a.g.mnx, (unsigned)a.g.mny, (unsigned)rp.bx - 0x4B400000u,
                    (unsigned)rp.by - 0x4B400000u, &rs.in};
     // the run's first ray, as if all its rays lay in this column (an exact
-    // float: counts this long are flushed first)
-    if (rs.cnt > 1048576u) {
+    // float); carries that are long, or that could make a run of the 2^23 rays
+    // that count_of no longer holds, are flushed first
+    if (rs.cnt > 1048576u || (float)rs.cnt + (uhi - ulo) >= 8388607.f) {
         run_flush(rs, a.map_u32, a.g.mnx, a.g.mny);
         rs.cnt = 0;
     }

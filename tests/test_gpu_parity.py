@@ -460,6 +460,24 @@ def test_launches_on_many_short_columns_take_few_tasks(ml, px, n_av, l1, l2_sub,
     f.close()
 
 
+def test_runs_carried_into_the_longest_columns_are_counted_whole(ml):
+    """A lane's run goes on from a row's short last column (1e6 rays) into the
+    next task's whole one (8.2e6, close to the longest that create takes, 2^23 -
+    1), all in the map's only pixel: its length stays below the 2^23 that a
+    float's integer bits hold.  The pixel wraps 2^32 (flagged); rays_in is exact."""
+    nx, ny = 9200000, 32 * 4000
+    w = inputs.Workload("wide", inputs.LensField(np.zeros(0), np.zeros(0), np.zeros(0)), 0.25, 0.25, 0.0,
+                        (0.0, 0.0, 1e6), (-1.0, -1.0, 1.0, 1.0), (1, 1), ray_box=(-1.0, -0.5, 1.0, 0.5), ray_n=(nx, ny))
+    f = _field(ml, w, precision=ml.PREC_MIXED, l1=(2.0 * 8.2 / 9.2, 1.0), l2_sub=(1, 1),
+               max_launch_rays=1 << 62)
+    assert (f.info["n2x"], f.info["N2x"]) == (8200000, 2)
+    f.shoot()
+    s = f.stats(check=False)
+    assert (s["rays_in"], s["rays_out"], s["rays_dropped"]) == (nx * ny, 0, 0)
+    assert int(f.counts().cpu().numpy().astype(np.uint32)[0, 0]) == nx * ny % 2 ** 32
+    f.close()
+
+
 def test_mixed_map_matches_oracle_and_split_invariance(ml):
     w = _mixed_case(6)
     f = _field(ml, w, precision=ml.PREC_MIXED)
