@@ -47,48 +47,60 @@ __device__ __forceinline__ void sheet64(const Geo &g, double tx, double ty, doub
     sy = f * uy;
 }
 
-// m / r2 for r2 > 0 to about one unit in the last place: the hardware's
-// approximate reciprocal (rcp.approx.ftz.f64, which reads r2's upper word) and
-// one third-order Newton step, y (1 + e + e^2) with e = 1 - r2 y (below 2^-18, so
-// e^3 is below the rounding).  Five FP64 instructions; FP64 runs at 1/64 of
-// FP32's rate here, and a division takes about ten.  Outside the exponents
-// where that holds (zero among them) the quotient is taken by division.
-template <bool UNIT>
-__device__ __forceinline__ double over_r2(double m, double r2)
-{
-    if ((unsigned)(__double2hiint(r2) - 0x00200000) >= 0x7fb00000u) return m / r2;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
-    const double e = __fma_rn(-r2, y, 1.0), t = __fma_rn(e, e, e);
-    const double my = UNIT ? y : __dmul_rn(m, y);      // UNIT: m is 1
-    return __fma_rn(my, t, my);
-}
-
-// Adds lens (x, y, m) to the deflection of R rays of one row at tx[], ty.
-// Returns (per ray, in hit) whether the ray coincides with the lens.
-template <int R, bool UNIT>
-__device__ __forceinline__ void add_lens64_of(double x, double y, double m, const double (&tx)[R], double ty,
-                                           double (&ax)[R], double (&ay)[R], bool (&hit)[R])
-{
-    const double dy = __dadd_rn(ty, -y), dy2 = __dmul_rn(dy, dy);
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const double dx = __dadd_rn(tx[r], -x);
-        const double r2 = __fma_rn(dx, dx, dy2);
-        hit[r] |= __double_as_longlong(r2) == 0;
-        const double s = over_r2<UNIT>(m, r2);
-        ax[r] = __fma_rn(dx, s, ax[r]);
-        ay[r] = __fma_rn(dy, s, ay[r]);
-    }
-}
+// Adds lens (x, y, m) to the deflection of R rays of one row at tx[], ty:
+// m (dx, dy) / r2.  Returns (per ray, in hit) whether the ray coincides with the
+// lens.  The quotients come from the hardware's approximate reciprocal v
+// (rcp.approx.ftz.f64, which reads r2's upper word) and Newton's method, with
+// e = 1 - r2 v below 2^-18: for unit masses v (1 + e + e^2) in one rounding, e^3
+// below it; else with w = v (1 + e) the product m w, corrected by its remainder,
+// m w + (m - m w r2) w, as a division rounds it.  (The product of m with
+// v (1 + e + e^2) is one operation less but rounds twice: lognormal masses came
+// out 0.5 % further off the sums in 80 bits than with divisions.)  FP64 runs at
+// 1/64 of FP32's rate here, and a division takes about ten instructions.  This
+// holds for r2 and |m| within 2^-500 and 2^500, where nothing over- or
+// underflows; elsewhere (zero among them) the quotients are taken by division.
+constexpr unsigned FP64_LOW = 0x20b00000u, FP64_SPAN = 0x3e800000u;   // upper words of 2^-500, 2^500 less it
 
 template <int R>
 __device__ __forceinline__ void add_lens64(double x, double y, double m, const double (&tx)[R], double ty,
                                            double (&ax)[R], double (&ay)[R], bool (&hit)[R])
 {
-    // (an integer comparison: FP64 ones take the FP64 pipe)
-    if (__double_as_longlong(m) == 0x3ff0000000000000ll) add_lens64_of<R, true>(x, y, m, tx, ty, ax, ay, hit);
-    else add_lens64_of<R, false>(x, y, m, tx, ty, ax, ay, hit);
+    const double dy = __dadd_rn(ty, -y), dy2 = __dmul_rn(dy, dy);
+    double dx[R], r2[R], s[R];
+    // (integer comparisons: FP64 ones take the FP64 pipe)
+    bool fast = ((unsigned)__double2hiint(m) & 0x7fffffffu) - FP64_LOW < FP64_SPAN;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        dx[r] = __dadd_rn(tx[r], -x);
+        r2[r] = __fma_rn(dx[r], dx[r], dy2);
+        hit[r] |= __double_as_longlong(r2[r]) == 0;
+        fast = fast && (unsigned)__double2hiint(r2[r]) - FP64_LOW < FP64_SPAN;
+    }
+    double v[R], e[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(v[r]) : "d"(r2[r]));
+        e[r] = __fma_rn(-r2[r], v[r], 1.0);
+    }
+    if (__double_as_longlong(m) == 0x3ff0000000000000ll) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) s[r] = __fma_rn(v[r], __fma_rn(e[r], e[r], e[r]), v[r]);
+    } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const double w = __fma_rn(v[r], e[r], v[r]), q = __dmul_rn(m, w);
+            s[r] = __fma_rn(__fma_rn(-q, r2[r], m), w, q);
+        }
+    }
+    if (!fast) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) s[r] = m / r2[r];
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        ax[r] = __fma_rn(dx[r], s[r], ax[r]);
+        ay[r] = __fma_rn(dy, s[r], ay[r]);
+    }
 }
 
 __device__ __forceinline__ double ray_x64(const Geo &g, int64_t i) { return __fma_rn((double)i + 0.5, g.l3x, g.rx0); }

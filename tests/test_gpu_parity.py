@@ -386,6 +386,28 @@ def test_fp64_modes_over_lattice_widths_and_ranges(ml, precision, n3x, n3y, mass
     f.close()
 
 
+@pytest.mark.parametrize("mass", [1.0, 0.37, 3.0, -0.2, 1e-9, 2.0 ** 501, 5e-324, 0.0])
+def test_fp64_deflection_quotients_are_rounded_once(ml, mass):
+    """One lens at a distance of exactly 1 along x from a column of rays, a macro
+    map and a sheet that give nothing: beta_x is minus m / (1 + dy^2), which a
+    division rounds.  The kernel's quotient must be that number for any mass (unit
+    masses: within one unit of the last place, nearly always that number)."""
+    n, ly = 4096, 0.7390851332151607
+    w = inputs.Workload("one lens", inputs.LensField(np.zeros(1), np.array([ly]), np.array([mass])), 1.0, 0.0, 0.0,
+                        (0.0, 0.0, 100.0), (-1.0, -1.0, 1.0, 1.0), (4, 4), ray_box=(0.0, -4.0, 2.0, 4.0), ray_n=(1, n))
+    f = _field(ml, w, precision=ml.PREC_DIRECT64)
+    beta = f.trace(np.arange(n))[0].cpu().numpy()
+    dy = (np.arange(n) + 0.5) * 2.0 ** -9 - 4.0 - ly          # the rows' positions are exact
+    want = mass / (1.0 + dy * dy)
+    bx = -beta[:, 0]
+    if mass == 1.0:
+        assert np.all(np.abs(bx - want) <= np.spacing(want)) and (bx == want).mean() > 0.95
+    else:
+        assert np.array_equal(bx, want), (bx - want)[bx != want][:5]
+    assert np.all(np.isfinite(beta))
+    f.close()
+
+
 @pytest.mark.parametrize("l1,l2_sub,p", [((6.0, 6.0), (20, 20), 0), ((9.0, 2.0), (10, 7), 0), ((2.0, 7.0), (5, 11), 0),
                                          ((5.0, 4.0), (3, 1), 16), ((4.0, 4.0), (1, 1), 12), ((3.0, 3.0), (40, 40), 1),
                                          ((0.15, 0.15), (2, 2), 0), ((0.06, 0.06), (2, 2), 0), ((0.02, 0.02), (1, 1), 0)])
