@@ -302,32 +302,46 @@ __device__ __forceinline__ void deposit64(const ShootArgs &a, bool hit, double b
     }
 }
 
+// (one warp per FP64 pipe of an SM, so that few of them spread over all SMs)
+constexpr int FP64_THREADS = 128;
+
 // Direct mode: a warp takes 32 R consecutive rays of one lattice row, lane l
 // the rays l, l + 32, ... (R of them share the lens's row offset, and their
-// chains hide the FP64 latency).  Bound by the FP64 pipe: 8 instructions per
-// ray and lens (7 for a unit mass) and 2/R shared, against about 16 with one
-// ray a thread, a division and an FP64 compare: 4e8 pairs took 10.9 ms, now
-// 5.8 ms at 90 % of the pipe.
+// chains hide the FP64 latency); with R = 1 any 32 consecutive rays.  Bound by
+// the FP64 pipe: 9 instructions per ray and lens (7 for a unit mass) and 2/R
+// shared, against about 16 with one ray a thread, a division and an FP64 compare:
+// 4e8 pairs took 10.9 ms, now 5.7 ms at 90 % of the pipe.
 template <int R>
-__global__ void __launch_bounds__(256) k_shoot_direct64(ShootArgs a)
+__global__ void __launch_bounds__(FP64_THREADS) k_shoot_direct64(ShootArgs a)
 {
     const Geo &g = a.g;
     unsigned long long in = 0, out = 0, drop = 0;
     unsigned ovf = 0;
     const int lane = threadIdx.x & 31;
     const int64_t nseg = (g.n3x + 32 * R - 1) / (32 * R);
-    const int64_t jb = a.ray_begin / g.n3x, je = (a.ray_end - 1) / g.n3x, items = (je - jb + 1) * nseg;
+    const int64_t jb = a.ray_begin / g.n3x, je = (a.ray_end - 1) / g.n3x;
+    const int64_t items = R == 1 ? (a.ray_end - a.ray_begin + 31) / 32 : (je - jb + 1) * nseg;
     const double ipx = 1.0 / g.dpx, ipy = 1.0 / g.dpy;
-    for (int64_t it = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
-        const int64_t j = jb + it / nseg, i0 = (it % nseg) * (32 * R) + lane;
+    constexpr int W = FP64_THREADS / 32;
+    for (int64_t it = blockIdx.x * (int64_t)W + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * W) {
         bool have[R], any = false, hit[R];
         double tx[R], bx[R], by[R];
+        int64_t j;
+        if constexpr (R == 1) {
+            const int64_t ray = a.ray_begin + it * 32 + lane;
+            have[0] = any = ray < a.ray_end;
+            j = ray / g.n3x;
+            tx[0] = ray_x64(g, ray - j * g.n3x);
+        } else {
+            const int64_t i0 = (it % nseg) * (32 * R) + lane;
+            j = jb + it / nseg;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int64_t i = i0 + 32 * r, ray = j * g.n3x + i;
-            have[r] = i < g.n3x && ray >= a.ray_begin && ray < a.ray_end;
-            any |= have[r];
-            tx[r] = ray_x64(g, i);
+            for (int r = 0; r < R; ++r) {
+                const int64_t i = i0 + 32 * r, ray = j * g.n3x + i;
+                have[r] = i < g.n3x && ray >= a.ray_begin && ray < a.ray_end;
+                any |= have[r];
+                tx[r] = ray_x64(g, i);
+            }
         }
         if (!__any_sync(0xffffffffu, any)) continue;
         beta_direct64<R>(a, tx, ray_y64(g, j), bx, by, hit);
@@ -340,12 +354,12 @@ __global__ void __launch_bounds__(256) k_shoot_direct64(ShootArgs a)
 
 // Near/far mode: lane = lattice row, a warp takes 32 rows and a chunk of up to
 // NF_CHUNK rays of one level-2 column; four rays at a time.  Bound by the FP64
-// pipe: 2p + 8 per near lens + about 20 per ray instead of 4p + 16 per near lens
+// pipe: 2p + 10 per near lens + about 20 per ray instead of 4p + 16 per near lens
 // + about 40 and five 64-bit divisions: 1.2e7 rays at p = 10 took 2.84 ms, now
-// 1.30 ms at 90 % of the pipe.
+// 1.15 ms.
 constexpr int NF_CHUNK = 64;
 
-__global__ void __launch_bounds__(256) k_shoot_nearfar64(ShootArgs a)
+__global__ void __launch_bounds__(FP64_THREADS) k_shoot_nearfar64(ShootArgs a)
 {
     constexpr int R = 4;
     const Geo &g = a.g;
@@ -355,7 +369,8 @@ __global__ void __launch_bounds__(256) k_shoot_nearfar64(ShootArgs a)
     const int64_t cpc = (g.n2x + NF_CHUNK - 1) / NF_CHUNK, ncol = g.N2x * cpc;
     const int64_t jb = a.ray_begin / g.n3x, je = (a.ray_end - 1) / g.n3x, items = ((je - jb) / 32 + 1) * ncol;
     const double ipx = 1.0 / g.dpx, ipy = 1.0 / g.dpy;
-    for (int64_t it = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
+    constexpr int W = FP64_THREADS / 32;
+    for (int64_t it = blockIdx.x * (int64_t)W + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * W) {
         const int64_t j = jb + 32 * (it / ncol) + lane, cc = it % ncol, c2x = cc / cpc;
         if (j > je) continue;
         int64_t i0 = c2x * g.n2x + (cc % cpc) * NF_CHUNK;
@@ -375,6 +390,49 @@ __global__ void __launch_bounds__(256) k_shoot_nearfar64(ShootArgs a)
             for (int r = 0; r < R; ++r)
                 if (i + r < i1) deposit64(a, hit[r], bx[r], by[r], ipx, ipy, in, out, drop, ovf);
         }
+    }
+    flush_stats(a, in, out, drop, 0, 0, ovf);
+}
+
+// The same with one ray a thread and Horner's rule in complex numbers, for level-2
+// columns too short to repay the row's re-expansion and lattices too small to fill
+// the FP64 pipes with chunks of them (106 x 15 rays with 30 near lenses: 38 us
+// instead of 55; 725 x 104 rays in columns of 15 at p = 16: 23 instead of 75).
+__global__ void __launch_bounds__(FP64_THREADS) k_shoot_nearfar64_rays(ShootArgs a)
+{
+    const Geo &g = a.g;
+    unsigned long long in = 0, out = 0, drop = 0;
+    unsigned ovf = 0;
+    const double ipx = 1.0 / g.dpx, ipy = 1.0 / g.dpy;
+    const double kx = sheet_kx(g), ky = sheet_ky(g);
+    for (int64_t ray = a.ray_begin + blockIdx.x * (int64_t)FP64_THREADS + threadIdx.x; ray < a.ray_end;
+         ray += (int64_t)gridDim.x * FP64_THREADS) {
+        const int64_t j = ray / g.n3x, i = ray - j * g.n3x, c2x = i / g.n2x, c2y = j / g.n2y;
+        const double tx[1] = {ray_x64(g, i)}, ty = ray_y64(g, j);
+        const double dr = __dadd_rn(tx[0], -__fma_rn((double)c2x + 0.5, g.l2x, g.rx0));
+        const double di = __dadd_rn(ty, -__fma_rn((double)c2y + 0.5, g.l2y, g.ry0));
+        const double2 *c = reinterpret_cast<const double2 *>(a.coef64) + (c2y * g.N2x + c2x) * (int64_t)(g.p + 1);
+        double2 F = __ldg(c + g.p);
+        for (int n = g.p - 1; n >= 0; --n) {
+            const double2 v = __ldg(c + n);
+            const double re = __fma_rn(F.x, dr, __fma_rn(-F.y, di, v.x));
+            F.y = __fma_rn(F.x, di, __fma_rn(F.y, dr, v.y));
+            F.x = re;
+        }
+        double ax[1] = {0.0}, ay[1] = {0.0};
+        bool hit[1] = {false};
+        const int64_t b0 = j / g.n1y * g.NEx + i / g.n1x;
+        for (int q = 0; q < 3; ++q) {
+            const int32_t *st = a.L.start + b0 + q * g.NEx;
+            for (int32_t k = st[0]; k < st[3]; ++k)
+                add_lens64<1>(__ldg(a.L.x + k), __ldg(a.L.y + k), __ldg(a.L.m + k), tx, ty, ax, ay, hit);
+        }
+        double mx, my;
+        macro64(g, tx[0], ty, mx, my);
+        // alpha_far = conj(F)
+        const double bx = __dadd_rn(__dadd_rn(mx, -ax[0]), __fma_rn(kx, __dadd_rn(tx[0], -g.sheet_cx), -F.x));
+        const double by = __dadd_rn(__dadd_rn(__fma_rn(ky, __dadd_rn(ty, -g.sheet_cy), my), -ay[0]), F.y);
+        deposit64(a, hit[0], bx, by, ipx, ipy, in, out, drop, ovf);
     }
     flush_stats(a, in, out, drop, 0, 0, ovf);
 }
@@ -1280,22 +1338,39 @@ cudaError_t launch_shoot(const ShootArgs &a, int num_sms, cudaStream_t s)
         default: return cudaErrorInvalidValue;
         }
     }
-    const int64_t rows = (a.ray_end - 1) / a.g.n3x - a.ray_begin / a.g.n3x + 1;
-    auto blocks_of = [&](int64_t items) {
-        return (unsigned)std::min<int64_t>((items + 7) / 8, (int64_t)num_sms * 4096);
+    // FP64: a launch's time in operations of one of the GPU's FP64 pipes (four an
+    // SM), the warps on the busiest pipe times a warp's operations.  Chosen so, 60
+    // near/far and direct lattices from 32 x 32 to 10,000 x 1,500 rays take the
+    // faster kernel or lie within 7 % of it.  (Direct mode by the row's last segment
+    // alone: 128 x 128 rays and 1000 lenses 2373 us with four rays a thread, now
+    // 640; 3 x 20,000 rays 5.6 times as long as one ray a thread.)
+    const int64_t rows = (a.ray_end - 1) / a.g.n3x - a.ray_begin / a.g.n3x + 1, n = a.ray_end - a.ray_begin;
+    const int64_t pipes = 4 * (int64_t)num_sms;
+    auto cost = [&](int64_t warps, double ops) { return (double)((warps + pipes - 1) / pipes) * ops; };
+    auto blocks_of = [&](int64_t warps) {
+        return (unsigned)std::min<int64_t>((warps + FP64_THREADS / 32 - 1) / (FP64_THREADS / 32), (int64_t)num_sms * 8192);
     };
+    const int64_t by_ray = (n + 31) / 32;
     if (a.g.precision == ML_PREC_NEARFAR64) {
-        const int64_t ncol = a.g.N2x * ((a.g.n2x + NF_CHUNK - 1) / NF_CHUNK);
-        k_shoot_nearfar64<<<blocks_of((rows + 31) / 32 * ncol), 256, 0, s>>>(a);
+        const int64_t chunk = std::min<int64_t>(a.g.n2x, NF_CHUNK), per = (chunk + 3) / 4 * 4, p = a.g.p;
+        const int64_t items = (rows + 31) / 32 * a.g.N2x * ((a.g.n2x + NF_CHUNK - 1) / NF_CHUNK);
+        const double near = 0.5 * (double)a.near_cap;
+        // a ray by itself, and a chunk of a row's rays with its re-expansion
+        if (cost(by_ray, 4.0 * p + 10.0 * near + 40.0) <
+            cost(items, 60.0 + p * (p + 1) + per * (2.0 * p + 8.5 * near + 20.0)))
+            k_shoot_nearfar64_rays<<<blocks_of(by_ray), FP64_THREADS, 0, s>>>(a);
+        else
+            k_shoot_nearfar64<<<blocks_of(items), FP64_THREADS, 0, s>>>(a);
         return cudaGetLastError();
     }
-    // rays per thread: as many as leave no more of the row's last segment empty
-    // than fewer would, to 3 %
-    auto segs = [&](int r) { return (a.g.n3x + 32 * r - 1) / (32 * r); };
-    const double full = 1.03 * (double)segs(1);
-    if ((double)(4 * segs(4)) <= full) k_shoot_direct64<4><<<blocks_of(rows * segs(4)), 256, 0, s>>>(a);
-    else if ((double)(2 * segs(2)) <= full) k_shoot_direct64<2><<<blocks_of(rows * segs(2)), 256, 0, s>>>(a);
-    else k_shoot_direct64<1><<<blocks_of(rows * segs(1)), 256, 0, s>>>(a);
+    // rays per thread: one warp's time per lens by measurement, relative, and what a
+    // pipe's only warp waits for besides
+    auto segs = [&](int r) { return rows * ((a.g.n3x + 32 * r - 1) / (32 * r)); };
+    const double c1 = cost(by_ray, 17.0), c2 = cost(segs(2), 10.5) + 1.0, c4 = cost(segs(4), 20.8) + 5.0;
+    const int R = c4 <= c1 && c4 <= c2 ? 4 : c2 <= c1 ? 2 : 1;
+    if (R == 4) k_shoot_direct64<4><<<blocks_of(segs(4)), FP64_THREADS, 0, s>>>(a);
+    else if (R == 2) k_shoot_direct64<2><<<blocks_of(segs(2)), FP64_THREADS, 0, s>>>(a);
+    else k_shoot_direct64<1><<<blocks_of(by_ray), FP64_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -386,6 +386,24 @@ def test_fp64_modes_over_lattice_widths_and_ranges(ml, precision, n3x, n3y, mass
     f.close()
 
 
+@pytest.mark.parametrize("precision,n3,l2", [("direct64", (3, 3001), 20), ("direct64", (40, 701), 20), ("direct64", (2016, 1003), 20),
+                                             ("nearfar64", (106, 15), 20), ("nearfar64", (530, 77), 20),
+                                             ("nearfar64", (1501, 402), 20), ("nearfar64", (1501, 402), 3)])
+def test_fp64_launch_forms(ml, precision, n3, l2):
+    """Lattices that take each form of the FP64 kernels (any rays, two or four of a
+    row per thread; one ray a thread or a row's chunk of a column), whole and in
+    ragged ranges: the counts are the histogram of the traced pixels."""
+    w = _mixed_case(seed=5)
+    w.lenses = inputs.lens_disc(40, w.lenses.radius, 5, "lognormal")
+    g0 = oracle.derive_geometry(w.kappa, w.gamma, w.kappa_star, [], [], (0, 0, 1), w.map_box, w.map_n, n_av=60)
+    w.ray_box, w.ray_n = (g0.rx0, g0.ry0, g0.rx1, g0.ry1), n3
+    f = _field(ml, w, precision=ml.PREC_NEARFAR64 if precision == "nearfar64" else ml.PREC_DIRECT64, l2_sub=(l2, l2))
+    n = f.n_rays
+    for r0, r1 in ((0, n), (n // 3 + 1, n - n // 5), (n // 2, n // 2 + 1)):
+        _shot_equals_traced(ml, f, r0, r1)
+    f.close()
+
+
 @pytest.mark.parametrize("mass", [1.0, 0.37, 3.0, -0.2, 1e-9, 2.0 ** 501, 5e-324, 0.0])
 def test_fp64_deflection_quotients_are_rounded_once(ml, mass):
     """One lens at a distance of exactly 1 along x from a column of rays, a macro
