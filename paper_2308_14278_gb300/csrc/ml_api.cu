@@ -1068,7 +1068,8 @@ ShootArgs make_args(const ml_field *f)
         a.rc2u = (float)((rc / g.l3x) * (rc / g.l3x));
         a.span_far2 = std::min(3.0e38f, std::max(f->span_far * f->span_far, 1.02f * a.rc2u + 1e-30f));
     }
-    a.piece_max = (float)std::max(4.0, floor(std::min(1e6, 0.15 * std::min(g.l1x, g.l1y) / g.l3x)));
+    // (three rays and fewer are the rule's own nodes)
+    a.piece_max = (float)std::max(3.0, floor(std::min(1e6, 0.15 * std::min(g.l1x, g.l1y) / g.l3x)));
     a.ipx_f = (float)(1.0 / g.dpx);
     a.ipy_f = (float)(1.0 / g.dpy);
     a.l3yx = g.l3y / g.l3x;

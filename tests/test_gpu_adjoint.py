@@ -322,6 +322,27 @@ def test_cic_runs_by_quadrature_match_the_rays_one_by_one(ml, l2, px):
     fr.close()
 
 
+@pytest.mark.parametrize("cells", [4, 5, 6, 7])
+def test_cic_quadrature_on_level1_cells_a_few_rays_wide(ml, cells):
+    """Cells a few rays wide, where far lenses come as near as that: a piece of four
+    rays there would carry up to 9e-6 of the map's largest value from the
+    quadrature; pieces of three are the rays themselves.  Against the rays one by
+    one: a pixel sums some 200 rays of weights rounded to 2^-24 of the sum at most,
+    16 x 2^-24 being several times their rms."""
+    w = _case()
+    w.map_n, w.ray_n = (30, 22), (400, 300)
+    lx, ly = (w.ray_box[2] - w.ray_box[0]) / 400, (w.ray_box[3] - w.ray_box[1]) / 300
+    kw = dict(l1=(cells * lx, 20 * ly), l2_sub=(1, 1), taylor_p=16)
+    out = []
+    for walk in (ml.WALK_CERTIFIED, ml.WALK_PER_RAY):
+        f = _field(ml, w, walk=walk, **kw)
+        assert f.info["n1x"] == cells
+        f.shoot()
+        out.append(f.mu().cpu().numpy().astype(np.float64))
+        f.close()
+    assert np.abs(out[0] - out[1]).max() <= 16 * 2.0 ** -24 * out[1].max(), np.abs(out[0] - out[1]).max() / out[1].max()
+
+
 def _corner_sums(mu, tracks, ns, sigma):
     """Light curves corner by corner and tap by tap in FP64 with float taps, as
     the library documents them: corners outside the map or of weight zero and
