@@ -343,6 +343,24 @@ def test_cic_quadrature_on_level1_cells_a_few_rays_wide(ml, cells):
     assert np.abs(out[0] - out[1]).max() <= 16 * 2.0 ** -24 * out[1].max(), np.abs(out[0] - out[1]).max() / out[1].max()
 
 
+@pytest.mark.parametrize("px,same", [((400, 300), True), ((42, 31), True), ((20, 15), False)])
+def test_sparse_cic_lattices_go_ray_by_ray(ml, px, same):
+    """Lattices of fewer than four rays a quad take the rays one by one (the runs'
+    quadrature would cost more than they do): with one lane adding to a pixel at
+    most, the map is the per-ray walk's; longer runs are summed, and differ in the
+    last bits."""
+    w = _case()
+    w.map_n, w.ray_n = px, (500, 1)
+    w.lenses, w.kappa_star = inputs.LensField(np.zeros(0), np.zeros(0), np.zeros(0)), 0.0
+    out = []
+    for walk in (ml.WALK_CERTIFIED, ml.WALK_PER_RAY):
+        f = _field(ml, w, walk=walk, l1=(20.0, 1.0), l2_sub=(2, 2))
+        f.shoot()
+        out.append(f.mu().cpu().numpy())
+        f.close()
+    assert np.array_equal(out[0], out[1]) == same
+
+
 def _corner_sums(mu, tracks, ns, sigma):
     """Light curves corner by corner and tap by tap in FP64 with float taps, as
     the library documents them: corners outside the map or of weight zero and
