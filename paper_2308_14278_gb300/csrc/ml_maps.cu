@@ -153,11 +153,12 @@ __device__ __forceinline__ void lc_point(const double *T, int k, int n_samples, 
     v = T[1] + t * (T[3] - T[1]) - 0.5;
 }
 
-// A sample corner by corner in FP64 (samples whose weighted sum is not an
-// ordinary number: infinities and NaN in the map, sums near the FP32 range's
-// ends).
+// Lane l's share of a sample corner by corner in FP64, every LANES-th row of each
+// corner's window, for samples whose sum in floats is not to be relied on:
+// infinities and NaN in the map, and sums near the ends of the FP32 range.
+template <int LANES>
 __device__ __noinline__ double lc_sample64(const uint32_t *cu, const float *cf, int mnx, int mny, double u,
-                                           double v, int h, const float *taps)
+                                           double v, int h, const float *taps, int lane)
 {
     double fu = floor(u), fv = floor(v);
     double wx = u - fu, wy = v - fv;
@@ -168,7 +169,7 @@ __device__ __noinline__ double lc_sample64(const uint32_t *cu, const float *cf, 
         double wc = ((c & 1) ? wx : 1.0 - wx) * ((c >> 1) ? wy : 1.0 - wy);
         if (pi < 0 || pi >= mnx || pj < 0 || pj >= mny || wc == 0.0) continue;
         double conv = 0.0;
-        for (int dy = -h; dy <= h; ++dy) {
+        for (int dy = lane - h; dy <= h; dy += LANES) {
             int yy = pj + dy;
             if (yy < 0 || yy >= mny) continue;
             double row = 0.0;
@@ -284,18 +285,25 @@ __global__ void __launch_bounds__(LC_THREADS) k_light_curves(int mnx, int mny, c
         C = __fadd_rn(C, __fadd_rn(c2, e));
         any |= __shfl_down_sync(0xffffffffu, any, o, LC_LANES);
     }
-    if (lane != 0 || !have) return;
     double tot = (double)S + (double)C;
-    if (!(fabs(tot) >= 1e-20 && fabs(tot) <= 1e37) && (any != 0 || !(tot == 0.0))) {
-        const uint32_t *cu = nullptr;
-        const float *cf = nullptr;
-        if constexpr (std::is_integral<T>::value) cu = map; else cf = map;
-        const int tr = (int)(q / n_samples);
-        double u, v;
-        lc_point(tracks + 4 * tr, (int)(q - (int64_t)tr * n_samples), n_samples, u, v);
-        tot = lc_sample64(cu, cf, mnx, mny, u, v, h, taps);
+    bool far = have && !(fabs(tot) >= 1e-20 && fabs(tot) <= 1e37) && (any != 0 || !(tot == 0.0));
+    far = __shfl_sync(0xffffffffu, (int)far, 0, LC_LANES) != 0;
+    if (__any_sync(0xffffffffu, far)) {
+        double part = 0.0;
+        if (far) {
+            const uint32_t *cu = nullptr;
+            const float *cf = nullptr;
+            if constexpr (std::is_integral<T>::value) cu = map; else cf = map;
+            const int tr = (int)(q / n_samples);
+            double u, v;
+            lc_point(tracks + 4 * tr, (int)(q - (int64_t)tr * n_samples), n_samples, u, v);
+            part = lc_sample64<LC_LANES>(cu, cf, mnx, mny, u, v, h, taps, lane);
+        }
+#pragma unroll
+        for (int o = LC_LANES / 2; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o, LC_LANES);
+        if (far) tot = part;
     }
-    out[q] = (float)(tot * scale);
+    if (lane == 0 && have) out[q] = (float)(tot * scale);
 }
 
 static cudaError_t run_light_curves(int mnx, int mny, const uint32_t *cu, const float *cf, double scale,
