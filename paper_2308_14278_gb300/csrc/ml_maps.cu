@@ -155,7 +155,8 @@ __device__ __forceinline__ void lc_point(const double *T, int k, int n_samples, 
 
 // Lane l's share of a sample corner by corner in FP64, every LANES-th row of each
 // corner's window, for samples whose sum in floats is not to be relied on:
-// infinities and NaN in the map, and sums near the ends of the FP32 range.
+// infinities and NaN in the map, sums near the ends of the FP32 range, and sums
+// that cancel to below 2^-12 of the window's largest value.
 template <int LANES>
 __device__ __noinline__ double lc_sample64(const uint32_t *cu, const float *cf, int mnx, int mny, double u,
                                            double v, int h, const float *taps, int lane)
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(LC_THREADS) k_light_curves(int mnx, int mny, c
                         dot_add(s, c, W.x, W.y, (float)(val & 0xFFu));
                     }
                 } else {
-                    any |= __float_as_uint(val) & 0x7FFFFFFFu;
+                    any |= __float_as_uint(val);
                     dot_add(s, c, W.x, W.y, val);
                 }
             }
@@ -286,7 +287,11 @@ __global__ void __launch_bounds__(LC_THREADS) k_light_curves(int mnx, int mny, c
         any |= __shfl_down_sync(0xffffffffu, any, o, LC_LANES);
     }
     double tot = (double)S + (double)C;
-    bool far = have && !(fabs(tot) >= 1e-20 && fabs(tot) <= 1e37) && (any != 0 || !(tot == 0.0));
+    // `any`, the values' bits or'ed: their largest magnitude up to a factor of two
+    // and, in a float map, whether one is negative
+    const float top = __uint_as_float(any & 0x7FFFFFFFu);
+    const bool cancels = !std::is_integral<T>::value && (any & 0x80000000u) != 0 && !(fabs(tot) >= 0x1p-12 * (double)top);
+    bool far = have && (cancels || (!(fabs(tot) >= 1e-20 && fabs(tot) <= 1e37) && (any != 0 || !(tot == 0.0))));
     far = __shfl_sync(0xffffffffu, (int)far, 0, LC_LANES) != 0;
     if (__any_sync(0xffffffffu, far)) {
         double part = 0.0;

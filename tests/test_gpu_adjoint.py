@@ -419,6 +419,39 @@ def test_light_curves_and_transpose_over_sources_and_spacings(ml, sigma, ns):
         assert abs(g.cpu().numpy()[at] - (col * w).sum()) <= 2.0 ** -24 * (w.size + 3) * (col * np.abs(w)).sum() + 1e-45
 
 
+@pytest.mark.parametrize("sigma,left", [(0.5, 1e-6), (4.0, 1e-6), (4.0, 1e-9)])
+def test_light_curves_of_maps_that_cancel(ml, sigma, left):
+    """Maps of both signs whose curves are far smaller than their values: 60 windows
+    of random pixels of 1000, each with one pixel set so that the sum in 64 bits
+    comes to about `left`.  The sums are those in FP64: within the rounding of the
+    float they are returned in and 2^-49 of the pixels (weights add up to one, and
+    FP64 sums of a thousand terms round to a few times 2^-53 of them)."""
+    import torch
+    rng = np.random.default_rng(4)
+    h, cell, nx, ny = int(4 * sigma), 40, 10, 6
+    mu = (rng.choice([-1000.0, 1000.0], (ny * cell, nx * cell))).astype(np.float32)
+    at = np.array([(cell * i + 20 + rng.uniform(-1, 1), cell * j + 20 + rng.uniform(-1, 1))
+                   for j in range(ny) for i in range(nx)])
+    tracks = np.concatenate([at, at], 1)
+    wide = mu.astype(np.float64)
+    for k, (x, y) in enumerate(at):
+        i, j = int(x - 0.5), int(y - 0.5)
+        for px in ((i, j), (i + 1, j), (i - h, j)):
+            one = np.zeros_like(wide)
+            one[px[1], px[0]] = 1.0
+            w = _corner_sums(one, tracks[k:k + 1], 1, sigma)[0, 0]
+            wide[px[1], px[0]] = 0.0
+            rest = _corner_sums(wide, tracks[k:k + 1], 1, sigma)[0, 0]
+            wide[px[1], px[0]] = np.float32((left - rest) / w)
+    mu = wide.astype(np.float32)
+    ref = _corner_sums(wide, tracks, 1, sigma)
+    assert np.abs(ref).max() < 2 * left
+    out = torch.empty((len(at), 1), dtype=torch.float32, device="cuda")
+    ml.ml_map_light_curves(torch.as_tensor(mu).cuda(), tracks, 1, sigma, out)
+    err = np.abs(out.cpu().numpy() - ref)
+    assert np.all(err <= 2.0 ** -24 * np.abs(ref) + 2.0 ** -49 * 1000.0), err.max()
+
+
 def test_light_curves_of_large_counts_and_unusual_maps(ml):
     """Counts up to 2^32 - 1 (beyond 2^24 a float drops bits), and infinities,
     NaN and values near the FP32 range's ends in a float map: as the corner
