@@ -200,24 +200,24 @@ __device__ __forceinline__ void dot_add(float &s, float &c, float wh, float wl, 
     c = __fadd_rn(c, __fadd_rn(f, e));
 }
 
-constexpr int LC_LANES = 8;                         // lanes per sample
 constexpr int LC_THREADS = 128;
-constexpr int LC_SAMPLES = LC_THREADS / LC_LANES;   // samples per block
 
-// Eight lanes per sample: a lane takes every eighth column of the window (a
+// LC_LANES lanes per sample, one for windows of up to six pixels, four up to 22,
+// eight beyond: a lane takes every LC_LANES-th column of the window (with eight a
 // 32-byte sector per row and group) and sums it over the rows, with weights and
 // sums as hi + lo floats.  FP64 runs at 1/64 of FP32's rate here: one thread
 // per sample, corner by corner in FP64 (4 x 33 x 33 products for a source of 4
-// pixels), took 7.9 ms for 80 curves of 4096 samples; this takes 0.34 ms and lies closer
-// to the sums in 64 bits.  Bound by FP32 issue: 18 instructions per pixel and
-// sample, 3.8e8 of them.
-template <class T>
+// pixels), took 7.9 ms for 80 curves of 4096 samples; this takes 0.32 ms and lies
+// closer to the sums in 64 bits.  Bound by FP32 issue: 18 instructions per pixel
+// and sample, 3.8e8 of them.
+template <class T, int LC_LANES>
 __global__ void __launch_bounds__(LC_THREADS) k_light_curves(int mnx, int mny, const T *__restrict__ map,
                                                              double scale, const double *__restrict__ tracks,
                                                              int n_tracks, int n_samples, int h,
                                                              const float *__restrict__ taps_g,
                                                              float *__restrict__ out)
 {
+    constexpr int LC_SAMPLES = LC_THREADS / LC_LANES;   // samples per block
     __shared__ float taps[129];
     extern __shared__ float2 lc_wy[];               // LC_SAMPLES x N
     const int N = 2 * h + 2;
@@ -317,14 +317,25 @@ static cudaError_t run_light_curves(int mnx, int mny, const uint32_t *cu, const 
 {
     const int64_t n = (int64_t)n_tracks * n_samples;
     if (n == 0) return cudaSuccess;
-    const unsigned blocks = (unsigned)((n + LC_SAMPLES - 1) / LC_SAMPLES);
-    const size_t smem = sizeof(float2) * LC_SAMPLES * (size_t)(2 * h + 2);   // at most 16.6 KB
-    if (cu)
-        k_light_curves<uint32_t><<<blocks, LC_THREADS, smem, s>>>(mnx, mny, cu, scale, d_tracks, n_tracks, n_samples,
-                                                                  h, d_taps, out);
-    else
-        k_light_curves<float><<<blocks, LC_THREADS, smem, s>>>(mnx, mny, cf, scale, d_tracks, n_tracks, n_samples, h,
-                                                               d_taps, out);
+    const int N = 2 * h + 2;
+    // lanes by the window's width: 80 curves of 4096 samples with 1, 4 and 8 lanes
+    // take 45, 66 and 118 us at N = 2 to 4, 51, 70 and 119 at 6, 113, 73 and 118 at
+    // 8, 228, 97 and 133 at 14, 539, 160 and 172 at 22, 1162, 324 and 319 at 34
+    const int lanes = N <= 6 ? 1 : N <= 22 ? 4 : 8, per = LC_THREADS / lanes;
+    const unsigned blocks = (unsigned)((n + per - 1) / per);
+    const size_t smem = sizeof(float2) * per * (size_t)N;   // at most 16.6 KB
+    auto run = [&](auto kern, auto *map) {
+        kern<<<blocks, LC_THREADS, smem, s>>>(mnx, mny, map, scale, d_tracks, n_tracks, n_samples, h, d_taps, out);
+    };
+    if (cu) {
+        if (lanes == 1) run(k_light_curves<uint32_t, 1>, cu);
+        else if (lanes == 4) run(k_light_curves<uint32_t, 4>, cu);
+        else run(k_light_curves<uint32_t, 8>, cu);
+    } else {
+        if (lanes == 1) run(k_light_curves<float, 1>, cf);
+        else if (lanes == 4) run(k_light_curves<float, 4>, cf);
+        else run(k_light_curves<float, 8>, cf);
+    }
     return cudaGetLastError();
 }
 

@@ -419,6 +419,12 @@ def test_light_curves_and_transpose_over_sources_and_spacings(ml, sigma, ns):
         assert abs(g.cpu().numpy()[at] - (col * w).sum()) <= 2.0 ** -24 * (w.size + 3) * (col * np.abs(w)).sum() + 1e-45
 
 
+@pytest.mark.parametrize("sigma", [0.74, 0.75, 2.74, 2.75])
+def test_light_curves_at_the_widths_where_lanes_change(ml, sigma):
+    """Windows of 6 and 8, 22 and 24 pixels: one, four and eight lanes a sample."""
+    test_light_curves_and_transpose_over_sources_and_spacings(ml, sigma, 33)
+
+
 @pytest.mark.parametrize("sigma,left", [(0.5, 1e-6), (4.0, 1e-6), (4.0, 1e-9)])
 def test_light_curves_of_maps_that_cancel(ml, sigma, left):
     """Maps of both signs whose curves are far smaller than their values: 60 windows
