@@ -751,8 +751,13 @@ cudaError_t launch_peak_stats(const uint32_t *N, int nx, int ny, int along, cons
 // register and is added once.  One thread and 4 (2h + 1)^2 atomics a sample
 // took 5.0 ms for 80 curves of 4096 samples of a 4-pixel source, bound by the
 // L2's atomics, N^2 atomics a sample 0.57 ms for 40 curves, this 0.28 ms
-// (0.11 against 0.43 ms at 0.5 pixels, 1.5 against 4.5 ms at 16; samples 0.3
-// to 8 pixels apart alike), bound by issue.
+// (1.5 against 4.5 ms at 16 pixels), bound by issue.  Where samples share few
+// pixels, narrow windows and samples far apart, the block adds N^2 products a
+// sample with atomics (400 x 16 samples 500 pixels apart at 0.5 pixels 202 -> 57
+// us, with the map's clearing).  The choice weighs warp steps: gathering 2.5 a row of the box and, for each of a
+// sample's rows, one per 96 columns of the samples that share it; scattering 3 per
+// 32 products.  By measurement over 250 spacings, widths and directions the lines
+// cross within 15 % of where the times do.
 constexpr int LCA_THREADS = 256;
 constexpr int LCA_CHUNK = 16;
 constexpr int LCA_COLS = 3;
@@ -766,6 +771,7 @@ __global__ void __launch_bounds__(LCA_THREADS) k_light_curves_adj(int mnx, int m
     __shared__ float taps[129];
     __shared__ int sx[LCA_CHUNK], sy[LCA_CHUNK];      // first column and row of each sample's window
     __shared__ int rows[2];
+    __shared__ bool scatter;
     __shared__ LcAxis axes[2][LCA_CHUNK];
     extern __shared__ float lca_w[];                  // per sample N x weights, N y weights (times g)
     const int N = 2 * h + 2, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -795,15 +801,33 @@ __global__ void __launch_bounds__(LCA_THREADS) k_light_curves_adj(int mnx, int m
     }
     __syncthreads();
     if (tid == 0) {
-        int c = sy[0], d = sy[0];
+        int c = sy[0], d = sy[0], l = sx[0], r = sx[0];
         for (int i = 1; i < ns; ++i) {
             c = min(c, sy[i]);
             d = max(d, sy[i]);
+            l = min(l, sx[i]);
+            r = max(r, sx[i]);
         }
         rows[0] = max(c, 0);
         rows[1] = min(d + N, mny);
+        // samples that share a row, of equally spaced ones
+        const float gaps = (float)max(1, ns - 1), live = fminf((float)ns, (float)N * gaps / fmaxf((float)(d - c), 1.f) + 1.f);
+        const float gather = 2.5f * (float)(d - c + N) +
+                             (float)(ns * N) * ceilf(((float)N + (live - 1.f) * (float)(r - l) / gaps) * (1.f / 96.f));
+        // (samples in one window: gathered, their atomics would meet)
+        scatter = d + r > c + l && gather > 3.f / 32.f * (float)(ns * N * N);
     }
     __syncthreads();
+    if (scatter) {
+        for (int q = tid; q < ns * N * N; q += blockDim.x) {
+            const int i = q / (N * N), r = q - i * N * N, ky = r / N, kx = r - ky * N;
+            const float w = lca_w[(2 * i + 1) * N + ky], v = lca_w[2 * i * N + kx];
+            const int x = sx[i] + kx, y = sy[i] + ky;
+            if (w != 0.f && v != 0.f && x >= 0 && x < mnx && y >= 0 && y < mny)
+                atomicAdd(gmap + (int64_t)y * mnx + x, __fmul_rn(w, v));
+        }
+        return;
+    }
     for (int y = rows[0] + wid; y < rows[1]; y += LCA_THREADS / 32) {
         // lane i: sample i's weight of this row (0 outside its window)
         float wy = 0.f;
@@ -840,6 +864,68 @@ __global__ void __launch_bounds__(LCA_THREADS) k_light_curves_adj(int mnx, int m
     }
 }
 
+// Windows of two and four pixels (sources below half a pixel): a thread takes
+// `per` consecutive samples of a track and keeps the products of those that share
+// a window in registers, so that a window's pixels are added once.  A million
+// samples of 0.2 pixels took 318 us in the blocks above.
+template <int N>
+__global__ void __launch_bounds__(128) k_light_curves_adj_narrow(int mnx, int mny, const double *__restrict__ tracks,
+                                                                 int n_tracks, int n_samples, int per,
+                                                                 const float *__restrict__ taps_g,
+                                                                 const float *__restrict__ dl, float *__restrict__ gmap)
+{
+    constexpr int H = (N - 2) / 2;
+    float taps[2 * H + 1];
+#pragma unroll
+    for (int t = 0; t <= 2 * H; ++t) taps[t] = __ldg(taps_g + t);
+    const int64_t runs = (n_samples + per - 1) / per, at = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (at >= runs * n_tracks) return;
+    const int tr = (int)(at / runs), k0 = (int)(at - tr * runs) * per, k1 = min(n_samples, k0 + per);
+    float acc[N][N];
+    int ci = 0, cj = 0;
+    auto clear = [&] {
+#pragma unroll
+        for (int y = 0; y < N; ++y)
+#pragma unroll
+            for (int x = 0; x < N; ++x) acc[y][x] = 0.f;
+    };
+    auto flush = [&] {
+#pragma unroll
+        for (int y = 0; y < N; ++y)
+#pragma unroll
+            for (int x = 0; x < N; ++x) {
+                const int64_t px = (int64_t)ci - H + x, py = (int64_t)cj - H + y;
+                if (acc[y][x] != 0.f && px >= 0 && px < mnx && py >= 0 && py < mny)
+                    atomicAdd(gmap + py * mnx + px, acc[y][x]);
+            }
+    };
+    clear();
+    for (int k = k0; k < k1; ++k) {
+        const float g = dl[(int64_t)tr * n_samples + k];
+        if (g == 0.f) continue;
+        double u, v;
+        lc_point(tracks + 4 * tr, k, n_samples, u, v);
+        const LcAxis ax = lc_axis(u, mnx), ay = lc_axis(v, mny);
+        if (ax.i0 != ci || ay.i0 != cj) {
+            flush();
+            clear();
+            ci = ax.i0;
+            cj = ay.i0;
+        }
+        float wx[N];
+#pragma unroll
+        for (int x = 0; x < N; ++x) wx[x] = lc_weight(ax, taps, H, x).x;
+#pragma unroll
+        for (int y = 0; y < N; ++y) {
+            const float wy = lc_weight(ay, taps, H, y).x, w = wy == 0.f ? 0.f : g * wy;
+#pragma unroll
+            for (int x = 0; x < N; ++x)
+                if (wx[x] != 0.f) acc[y][x] = fmaf(w, wx[x], acc[y][x]);
+        }
+    }
+    flush();
+}
+
 cudaError_t launch_light_curves_adj(int mnx, int mny, const double *d_tracks, int n_tracks,
                                     int n_samples, double sigma_px, const float *dl, float *gmap,
                                     cudaStream_t s)
@@ -853,10 +939,23 @@ cudaError_t launch_light_curves_adj(int mnx, int mny, const double *d_tracks, in
     e = cudaMemcpyAsync(d_taps, taps, sizeof(float) * (2 * h + 1), cudaMemcpyHostToDevice, s);
     const int64_t n = (int64_t)n_tracks * n_samples;
     if (e == cudaSuccess && n > 0) {
-        const int64_t blocks = (int64_t)n_tracks * ((n_samples + LCA_CHUNK - 1) / LCA_CHUNK);
-        if (blocks > 0x7fffffff) { cudaFreeAsync(d_taps, s); return cudaErrorInvalidConfiguration; }
-        k_light_curves_adj<<<(unsigned)blocks, LCA_THREADS, sizeof(float) * 2 * LCA_CHUNK * (size_t)(2 * h + 2), s>>>(
-            mnx, mny, d_tracks, n_samples, h, d_taps, dl, gmap);
+        // tracks per launch, within the grid's 2^31 - 1 blocks
+        const int64_t per = std::max<int64_t>(1, std::min<int64_t>(8, n / (152 * 512)));
+        const int64_t blocks1 = h <= 1 ? (((n_samples + per - 1) / per) + 127) / 128 + 1 : (n_samples + LCA_CHUNK - 1) / LCA_CHUNK;
+        const int64_t step = std::min<int64_t>(n_tracks, 0x7fffffff / blocks1);
+        for (int64_t t = 0; t < n_tracks; t += step) {
+            const int nt = (int)std::min<int64_t>(step, n_tracks - t);
+            const double *tr = d_tracks + 4 * t;
+            const float *g = dl + t * n_samples;
+            const unsigned narrow = (unsigned)(((n_samples + per - 1) / per * nt + 127) / 128);
+            if (h == 0)
+                k_light_curves_adj_narrow<2><<<narrow, 128, 0, s>>>(mnx, mny, tr, nt, n_samples, (int)per, d_taps, g, gmap);
+            else if (h == 1)
+                k_light_curves_adj_narrow<4><<<narrow, 128, 0, s>>>(mnx, mny, tr, nt, n_samples, (int)per, d_taps, g, gmap);
+            else
+                k_light_curves_adj<<<(unsigned)(nt * blocks1), LCA_THREADS, sizeof(float) * 2 * LCA_CHUNK * (size_t)(2 * h + 2),
+                                     s>>>(mnx, mny, tr, n_samples, h, d_taps, g, gmap);
+        }
         e = cudaGetLastError();
     }
     cudaFreeAsync(d_taps, s);

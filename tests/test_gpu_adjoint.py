@@ -486,6 +486,51 @@ def test_light_curves_of_large_counts_and_unusual_maps(ml):
         assert np.allclose(out.cpu().numpy(), ref, rtol=2.0 ** -22, atol=3e-45, equal_nan=True), value
 
 
+@pytest.mark.parametrize("sigma,spacing", [(0.2, 0.3), (0.5, 60.0), (1.0, 0.1), (1.0, 9.0), (4.0, 0.5), (4.0, 17.0), (4.0, 60.0)])
+@pytest.mark.parametrize("along", [(1.0, 0.001), (0.002, 1.0), (0.6, 0.8)])
+def test_light_curve_transpose_gathers_or_scatters(ml, sigma, spacing, along):
+    """Chunks of samples that share most of their pixels and chunks that share
+    none, along and across the rows, partly outside the map: the outer products of
+    each sample's weights, added up in FP64.  FP32 sums of n samples' products:
+    (n + 4) 2^-24 of the sum of their sizes."""
+    import torch
+    rng = np.random.default_rng(6)
+    ny, nx, ns, h = 700, 900, 37, int(4 * sigma)
+    a = rng.uniform(-20, 200, (3, 2))
+    tracks = np.concatenate([a, a + spacing * (ns - 1) * np.array(along)], 1)
+    w = rng.standard_normal((3, ns)).astype(np.float32)
+    t = np.exp(-0.5 * (np.arange(-h, h + 1) / sigma) ** 2)
+    taps = (t / t.sum()).astype(np.float32).astype(np.float64)
+    ref, size, hits = np.zeros((ny, nx)), np.zeros((ny, nx)), np.zeros((ny, nx))
+
+    def axis(c, n):
+        i = int(np.floor(c))
+        out = np.zeros(n + 2 * h + 4)
+        for j, f in ((i, 1.0 - (c - i)), (i + 1, c - i)):
+            if 0 <= j < n:
+                out[j: j + 2 * h + 1] += f * taps
+        return out[h: h + n]
+
+    for k in range(3):
+        for q in range(ns):
+            f = q / (ns - 1)
+            u = tracks[k, 0] + f * (tracks[k, 2] - tracks[k, 0]) - 0.5
+            v = tracks[k, 1] + f * (tracks[k, 3] - tracks[k, 1]) - 0.5
+            wy, wx = axis(v, ny), axis(u, nx)
+            y, x = np.flatnonzero(wy), np.flatnonzero(wx)
+            if len(y) and len(x):
+                at = np.ix_(y, x)
+                p = np.outer(wy[y], wx[x])
+                ref[at] += float(w[k, q]) * p
+                size[at] += abs(float(w[k, q])) * p
+                hits[at] += 1
+    g = torch.empty((ny, nx), dtype=torch.float32, device="cuda")
+    ml.ml_map_light_curves_backward(torch.as_tensor(w).cuda(), tracks, ns, sigma, g)
+    got = g.cpu().numpy()
+    assert np.all(np.abs(got - ref) <= (hits + 4) * 2.0 ** -24 * size + 1e-45)
+    assert np.all(got[hits == 0] == 0.0)
+
+
 def test_light_curve_adjoint_is_the_transpose_of_the_oracle_operator(ml):
     """Brute force: the oracle's light-curve operator J (samples x pixels),
     column by column on unit maps; the GPU backward must return J^T w."""
