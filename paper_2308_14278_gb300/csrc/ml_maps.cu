@@ -322,10 +322,15 @@ static cudaError_t run_light_curves(int mnx, int mny, const uint32_t *cu, const 
     // take 45, 66 and 118 us at N = 2 to 4, 51, 70 and 119 at 6, 113, 73 and 118 at
     // 8, 228, 97 and 133 at 14, 539, 160 and 172 at 22, 1162, 324 and 319 at 34
     const int lanes = N <= 6 ? 1 : N <= 22 ? 4 : 8, per = LC_THREADS / lanes;
-    const unsigned blocks = (unsigned)((n + per - 1) / per);
     const size_t smem = sizeof(float2) * per * (size_t)N;   // at most 16.6 KB
+    // tracks per launch, within the grid's 2^31 - 1 blocks
+    const int64_t step = std::max<int64_t>(1, 0x7fffffffll * per / n_samples);
     auto run = [&](auto kern, auto *map) {
-        kern<<<blocks, LC_THREADS, smem, s>>>(mnx, mny, map, scale, d_tracks, n_tracks, n_samples, h, d_taps, out);
+        for (int64_t t = 0; t < n_tracks; t += step) {
+            const int nt = (int)std::min<int64_t>(step, n_tracks - t);
+            kern<<<(unsigned)(((int64_t)nt * n_samples + per - 1) / per), LC_THREADS, smem, s>>>(
+                mnx, mny, map, scale, d_tracks + 4 * t, nt, n_samples, h, d_taps, out + t * n_samples);
+        }
     };
     if (cu) {
         if (lanes == 1) run(k_light_curves<uint32_t, 1>, cu);
