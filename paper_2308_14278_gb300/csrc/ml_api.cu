@@ -1903,7 +1903,8 @@ ml_status ml_find_peaks(ml_field *f, int32_t along, double nsigma, uint8_t *mask
     if (!m) e = ml_malloc_async((void **)&m, npix + 4, s);
     if (e == cudaSuccess) e = ml_malloc_async((void **)&found, sizeof(unsigned long long), s);
     if (e == cudaSuccess)
-        e = launch_peaks(f->d_map_u32, f->g.mnx, f->g.mny, along, nsigma, m, peaks, capacity, found, s);
+        e = launch_peaks(f->d_map_u32, f->g.mnx, f->g.mny, along, nsigma, m, peaks, capacity, found,
+                         f->num_sms, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h_found, found, sizeof(h_found), cudaMemcpyDeviceToHost, s);
     if (found) cudaFreeAsync(found, s);
     if (!mask && m) cudaFreeAsync(m, s);
@@ -1950,7 +1951,7 @@ ml_status ml_peak_statistics(ml_field *f, int32_t along, double nsigma, const ui
     if (e == cudaSuccess && !mask) {
         uint8_t *mm = reinterpret_cast<uint8_t *>(scratch + o_mask);
         e = launch_peaks(f->d_map_u32, nx, ny, along, nsigma, mm, nullptr, 0,
-                         reinterpret_cast<unsigned long long *>(scratch + o_found), s);
+                         reinterpret_cast<unsigned long long *>(scratch + o_found), f->num_sms, s);
         m = mm;
     }
     if (e == cudaSuccess)

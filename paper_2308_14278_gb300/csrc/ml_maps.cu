@@ -633,15 +633,18 @@ __global__ void __launch_bounds__(128) k_peaks(const uint32_t *__restrict__ N, i
 }
 
 cudaError_t launch_peaks(const uint32_t *N, int nx, int ny, int along, double nsigma, uint8_t *mask,
-                         int32_t *peaks, int64_t capacity, unsigned long long *found, cudaStream_t s)
+                         int32_t *peaks, int64_t capacity, unsigned long long *found, int num_sms, cudaStream_t s)
 {
     const int64_t n = (int64_t)nx * ny;
     cudaError_t e = cudaMemsetAsync(found, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess || n == 0) return e;
     const int64_t nseg = (nx + PK_OWN - 1) / PK_OWN;
-    // 32 rows a warp (6 to 12 % of them read twice) where that gives the GPU
-    // 16 warps per SM, else 8
-    const int rows = nseg * ((ny + 31) / 32) >= 152 * 16 ? 32 : 8;
+    // the most rows a warp, up to 32 (6 % of them read twice), that leave each SM 26
+    // warps, whose row loads follow one another: 100 x 100 pixels 3.6 us with one row
+    // (8: 8.4, 32: 28), 1000 x 1000 5.9 with two (8: 9.2), 2048 x 2048 11.4 with
+    // eight (2: 15), 4096 x 5120 48 with 32 (8: 47, 2: 65)
+    int rows = 32;
+    while (rows > 1 && nseg * ((ny + rows - 1) / rows) < 26 * (int64_t)num_sms) rows /= 2;
     const unsigned blocks = (unsigned)((nseg * ((ny + rows - 1) / rows) + 3) / 4);
     const double k2x3 = 3.0 * nsigma * nsigma;
     auto kern = nx % 4 == 0 ? (along == 0 ? k_peaks<true, 0> : k_peaks<true, 1>)

@@ -77,6 +77,26 @@ def test_peaks_at_strip_edges_match_oracle(ml, nx, ny, along):
     f.close()
 
 
+@pytest.mark.parametrize("along", ["x", "y"])
+@pytest.mark.parametrize("nx", [3, 4])
+@pytest.mark.parametrize("rows", [1, 2, 4, 8, 16, 32])
+def test_peaks_over_rows_per_warp(ml, nx, rows, along):
+    """Maps of one strip whose height gives a warp 1 to 32 rows, with five rows
+    more than fill them."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ny = 26 * sms * rows + 5
+    rng = np.random.default_rng(rows)
+    N = rng.integers(0, 3, (ny, nx)).astype(np.int64) * 40 + 300 * (rng.random((ny, nx)) < 0.3)
+    f = _blank_field(ml, nx, ny)
+    ml.ml_field_set_counts(f.h, torch.as_tensor(N.astype(np.int32)).cuda())
+    n, peaks, m = _gpu_peaks(ml, f, ml.ALONG_X if along == "x" else ml.ALONG_Y, nsigma=2.0, capacity=nx * ny)
+    ref = oracle.peaks(N, along, nsigma=2.0)
+    assert np.array_equal(m, ref) and n == int((ref & 2).astype(bool).sum()) > 0
+    assert {tuple(p) for p in peaks} == {(x, y) for y, x in zip(*np.nonzero(ref & 2))}
+    f.close()
+
+
 def test_peaks_of_a_shot_map_match_oracle(ml):
     """A fold-model map shot on the GPU: its own count map through both
     implementations (the oracle reads the GPU's counts: the check is of the
