@@ -90,10 +90,14 @@ template <class Key, class Emit>
 __device__ void cta_stable_scatter(const Key &key, int64_t n, int64_t nb, const int32_t *start,
                                    int32_t *ostart, int32_t *cnt, const Emit &emit)
 {
-    // W counting warps: their rows of buckets are cleared and turned into slots,
-    // W x nb counters, so many buckets take fewer warps (eight beyond 16,384
-    // buckets: Table-1 field, 56,000 buckets, 0.45 -> 0.27 ms)
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = nb > 16384 ? 8 : blockDim.x >> 5;
+    // W counting warps: each walks n / W items, and W x nb counters are cleared and
+    // turned into slots.  W^2 = 158 n / nb balances them (kernel times at 4, 8, 16
+    // and 32 warps: 13,000 lenses in 485 buckets 122, 69, 46 and 42 us, 8465 buckets
+    // 132, 85, 76 and 102, 53,825 buckets 187, 171, 236 and 412; 1000 lenses in 8465
+    // buckets 16, 20, 38 and 67).
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int W = 4;
+    while (W < (int)(blockDim.x >> 5) && 2 * W * W * nb < 158 * n) W *= 2;
     const int64_t chunk = (n + W - 1) / W;
     const int64_t kb = w < W ? min(n, w * chunk) : n, ke = min(n, kb + chunk);
     int32_t *my = cnt + w * nb;

@@ -404,6 +404,26 @@ def test_fp64_launch_forms(ml, precision, n3, l2):
     f.close()
 
 
+@pytest.mark.parametrize("cells,lenses", [(20, 2000), (40, 2000), (80, 2000), (110, 2000), (110, 3), (3, 2000)])
+def test_lens_sort_at_each_number_of_counting_warps(ml, cells, lenses):
+    """Lenses over level-1 cells in the ratios that give the sort 32, 16, 8 and 4
+    counting warps: near lists and far sums read every lens once and in place, so
+    the positions are the oracle's direct sums to the truncation bound."""
+    w = _mixed_case(seed=7)
+    w.lenses = inputs.lens_disc(lenses, w.lenses.radius, 7, "lognormal")
+    g0 = oracle.derive_geometry(w.kappa, w.gamma, w.kappa_star, [], [], (0, 0, 1), w.map_box, w.map_n, n_av=60)
+    w.ray_box, w.ray_n = (g0.rx0, g0.ry0, g0.rx1, g0.ry1), (4 * cells, 3 * cells)
+    l1 = ((g0.rx1 - g0.rx0) / cells, (g0.ry1 - g0.ry0) / cells)
+    f = _field(ml, w, precision=ml.PREC_NEARFAR64, taylor_p=16, l1=l1, l2_sub=(2, 2))
+    assert (f.info["N2x"] + 1) // 2 == cells
+    idx = np.unique(np.random.default_rng(2).integers(0, f.n_rays, 3000))
+    beta = f.trace(idx)[0].cpu().numpy()
+    ref, flag = oracle.beta_direct(_geometry(w, f), w.lenses.x, w.lenses.y, w.lenses.m, idx)
+    ok = ~flag
+    assert ok.any() and np.all(np.abs(beta - ref)[ok] <= 1e-9 * (1.0 + np.abs(ref[ok])) + f.info["far_bound"])
+    f.close()
+
+
 @pytest.mark.parametrize("mass", [1.0, 0.37, 3.0, -0.2, 1e-9, 2.0 ** 501, 5e-324, 0.0])
 def test_fp64_deflection_quotients_are_rounded_once(ml, mass):
     """One lens at a distance of exactly 1 along x from a column of rays, a macro
