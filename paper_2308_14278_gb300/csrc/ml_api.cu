@@ -912,7 +912,7 @@ ml_status create_finish(ml_field *f, int p, cudaStream_t s, bool sync = true)
         if (ns > 0) {
             double *scratch = nullptr;
             ML_CK(ml_malloc_async((void **)&scratch, ns * sizeof(double), s));
-            cudaError_t e = launch_coeffs_hier(g, L, f->d_coef64, f->d_nodes, scratch, ns, s);
+            cudaError_t e = launch_coeffs_hier(g, L, f->d_coef64, f->d_nodes, scratch, ns, f->num_sms, s);
             cudaFreeAsync(scratch, s);
             if (e != cudaSuccess) return cuda_fail(e, "hierarchical coefficient build");
             f->build_used = ML_BUILD_HIERARCHICAL;

@@ -603,12 +603,7 @@ __host__ __device__ inline Hier hier_of(const Geo &g)
     h.NBx = (g.N1x + h.bxn - 1) / h.bxn;
     h.NBy = (g.N1y + h.byn - 1) / h.byn;
     h.hB = 0.5 * sqrt((double)(h.bxn * h.bxn) * g.l1x * g.l1x + (double)(h.byn * h.byn) * g.l1y * g.l1y);
-    // a partition ends in a reduction of all orders over its block, so no more
-    // of them than give the GPU 912 blocks, two for each of its 456 slots
-    // (always 16: the Table-1 field's build 6.11 ms, now 5.82; 13,000 lenses on
-    // 1.23 theta_E cells 1.37 -> 1.33; at 456 blocks the latter takes 1.46)
     h.parts = HPARTS;
-    while (h.parts > 1 && h.NBx * h.NBy * (h.parts / 2) >= 912) h.parts /= 2;
     return h;
 }
 
@@ -1472,9 +1467,14 @@ static void run_node_records(const Geo &g, const Hier &h, const float2 *sub, con
 // coef64 receives the FP64 near/far mode's coefficients, nodes the mixed
 // mode's records (the other is not used).
 cudaError_t launch_coeffs_hier(const Geo &g, const LensTable &L, double *coef64, unsigned char *nodes,
-                               double *scratch, size_t scratch_doubles, cudaStream_t s)
+                               double *scratch, size_t scratch_doubles, int num_sms, cudaStream_t s)
 {
     Hier h = hier_of(g);
+    // a partition ends in a reduction of all orders over its block, so no more
+    // of them than give the GPU six blocks an SM, two for each of its three slots
+    // (always 16: the Table-1 field's build 6.11 ms, now 5.82; 13,000 lenses on
+    // 1.23 theta_E cells 1.37 -> 1.33; at three blocks an SM the latter takes 1.46)
+    while (h.parts > 1 && h.NBx * h.NBy * (h.parts / 2) >= 6 * (int64_t)num_sms) h.parts /= 2;
     if (scratch_doubles < hier_scratch_doubles(g)) return cudaErrorInvalidValue;
     size_t nb = (size_t)(h.NBx * h.NBy), ns = (size_t)(g.N1x * g.N1y * h.nsx * h.nsy);
     double *part = scratch;

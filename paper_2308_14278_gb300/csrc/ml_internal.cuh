@@ -137,7 +137,7 @@ cudaError_t launch_plan_max(const Geo &g, const int32_t *start, const double *bo
                             int num_sms, cudaStream_t s);
 cudaError_t launch_coeffs_direct(const Geo &g, const LensTable &L, double *coef64, cudaStream_t s);
 cudaError_t launch_coeffs_hier(const Geo &g, const LensTable &L, double *coef64, unsigned char *nodes,
-                               double *scratch, size_t scratch_doubles, cudaStream_t s);
+                               double *scratch, size_t scratch_doubles, int num_sms, cudaStream_t s);
 size_t hier_scratch_doubles(const Geo &g);
 cudaError_t launch_node_finalize(const Geo &g, const double *coef64, unsigned char *nodes,
                                  cudaStream_t s);
