@@ -1241,7 +1241,8 @@ struct NodeMap {
 
 // 3. node records from the sub-block series, in one pass (the FP64 form shifts
 // to coefficients in memory first, which k_node_finalize reads again).  c_1..c_p
-// are the same FP32 sums as k_node_shift's; c_0 sums pairs up to order j64.  A
+// are FP32 sums (the shifted series decays, no term cancels far below the sum); c_0
+// sums pairs up to order j64.  A
 // block's records are staged in shared memory and stored 16 bytes at a time.
 // The FP64 form took 4.4 + 2.0 ms for the Table-1 field's 10.9M nodes, this 1.16 ms.
 template <int P>
@@ -1361,7 +1362,7 @@ static NodeMap node_map(const Geo &g, const Hier &h)
     return m;
 }
 
-// 3. node coefficients from the sub-block series.  Index arithmetic in 32
+// 3. the near/far mode's node coefficients from the sub-block series.  Index arithmetic in 32
 // bits (level-2 cells per level-1 side and sub-block counts are small), the
 // scales by reciprocals.
 __global__ void __launch_bounds__(128) k_node_shift(Geo g, Hier h, const double *__restrict__ sub,
@@ -1371,7 +1372,6 @@ __global__ void __launch_bounds__(128) k_node_shift(Geo g, Hier h, const double 
 {
     // node-uniform loop indices: the binomials come from the constant cache
     const double *binom = c_binom.v;
-    const float *binomf = c_binomf.v;
     int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (node >= g.N2x * g.N2y) return;
     const int64_t c2y64 = node / g.N2x;
@@ -1392,12 +1392,8 @@ __global__ void __launch_bounds__(128) k_node_shift(Geo g, Hier h, const double 
     const double *a = sub + s * (HP + 1) * 2;
     const float *af = sub32 + s * (HP + 1) * 2;
     double *out = coef + node * (int64_t)(g.p + 1) * 2;
-    // The mixed mode keeps c_1..c_p in FP32 (node records), so they are summed
-    // in FP32 there: the shifted series decays (ratio < 0.6), no term cancels
-    // far below the sum.  c_0, the node's far deflection, is FP64 up to order
-    // j64[s] and FP32 above (the sub-block's bound); the FP64 near/far mode
-    // takes c_1..c_p in FP64.
-    const bool fp32_tail = g.precision == ML_PREC_MIXED;
+    // c_0, the node's far deflection, is FP64 up to order j64[s] and FP32 above (the
+    // sub-block's bound); c_1..c_p are FP64.
     const float erf = (float)er, eif = (float)ei;
     {
         const int J = j64[s];
@@ -1421,29 +1417,16 @@ __global__ void __launch_bounds__(128) k_node_shift(Geo g, Hier h, const double 
     double ihn = 1.0;
     for (int n = 1; n <= g.p; ++n) {
         ihn *= ihs;
-        if (fp32_tail) {
-            float vr = 0.f, vi = 0.f;
-            for (int j = HP; j >= n; --j) {
-                const float c = binomf[j * (HP + 1) + n];
-                const float nr = __fmaf_rn(vr, erf, __fmaf_rn(-vi, eif, c * af[2 * j]));
-                const float ni = __fmaf_rn(vr, eif, __fmaf_rn(vi, erf, c * af[2 * j + 1]));
-                vr = nr;
-                vi = ni;
-            }
-            out[2 * n] = (double)vr * ihn;
-            out[2 * n + 1] = (double)vi * ihn;
-        } else {
-            double vr = 0.0, vi = 0.0;
-            for (int j = HP; j >= n; --j) {
-                double c = binom[j * (HP + 1) + n];
-                double nr = vr * er - vi * ei + c * a[2 * j];
-                double ni = vr * ei + vi * er + c * a[2 * j + 1];
-                vr = nr;
-                vi = ni;
-            }
-            out[2 * n] = vr * ihn;
-            out[2 * n + 1] = vi * ihn;
+        double vr = 0.0, vi = 0.0;
+        for (int j = HP; j >= n; --j) {
+            double c = binom[j * (HP + 1) + n];
+            double nr = vr * er - vi * ei + c * a[2 * j];
+            double ni = vr * ei + vi * er + c * a[2 * j + 1];
+            vr = nr;
+            vi = ni;
         }
+        out[2 * n] = vr * ihn;
+        out[2 * n + 1] = vi * ihn;
     }
 }
 
