@@ -680,17 +680,10 @@ __device__ __forceinline__ df df_renorm(float s, float e)       // |e| <= |s| / 
     return r;
 }
 
-__device__ __forceinline__ void df_sum2(float a, float b, float &s, float &e)
-{
-    s = __fadd_rn(a, b);
-    const float t = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-
 __device__ __forceinline__ df df_add(df a, df b)
 {
     float s, e;
-    df_sum2(a.h, b.h, s, e);
+    two_sum(a.h, b.h, s, e);
     return df_renorm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
 }
 
@@ -716,7 +709,7 @@ __device__ __forceinline__ df df_dot2(df a, df b, df c, df d)
     float p, e, q, f, s, t;
     df_prod(a, b, p, e);
     df_prod(c, d, q, f);
-    df_sum2(p, q, s, t);
+    two_sum(p, q, s, t);
     return df_renorm(s, __fadd_rn(t, __fadd_rn(e, f)));
 }
 
@@ -756,10 +749,10 @@ __device__ __forceinline__ void p2l_add_df(double m, df dx, df dy, df h, df ih, 
     for (int j = 0; j < HD; ++j) {
         if (j > J) return;
         float s, e;
-        df_sum2(a.r[j].h, tr.h, s, e);
+        two_sum(a.r[j].h, tr.h, s, e);
         a.r[j].h = s;
         a.r[j].l = __fadd_rn(a.r[j].l, __fadd_rn(e, tr.l));
-        df_sum2(a.i[j].h, ti.h, s, e);
+        two_sum(a.i[j].h, ti.h, s, e);
         a.i[j].h = s;
         a.i[j].l = __fadd_rn(a.i[j].l, __fadd_rn(e, ti.l));
         const df nr = df_dot2(tr, wr, df_neg(ti), wi);
@@ -783,7 +776,7 @@ __device__ __forceinline__ void p2l_add_df(double m, df dx, df dy, df h, df ih, 
 __device__ __forceinline__ df lens_offset(float h, float l, df z)
 {
     float s, e;
-    df_sum2(h, -z.h, s, e);
+    two_sum(h, -z.h, s, e);
     return df_renorm(s, __fadd_rn(e, __fsub_rn(l, z.l)));
 }
 

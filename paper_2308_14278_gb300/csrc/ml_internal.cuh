@@ -487,6 +487,14 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
     return d;
 }
 
+// s = a + b and the rounding of that sum (Knuth's two-sum).
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
 {
     f32x2 d;

@@ -123,14 +123,6 @@ __device__ __forceinline__ LcAxis lc_axis(double t, int size)
     return a;
 }
 
-// s + c with the rounding of the sum kept (Knuth's two-sum).
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
-{
-    s = __fadd_rn(a, b);
-    const float t = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-
 // W[k] as hi + lo floats, in FP32 instructions (FP64 runs at 1/64 of their rate).
 __device__ __forceinline__ float2 lc_weight(const LcAxis &a, const float *taps, int h, int k)
 {
