@@ -655,9 +655,15 @@ __device__ __forceinline__ void p2l_add(double m, double dx, double dy, double h
 // FP32, so its series need not be carried in FP64, whose rate here is 1/64 of
 // FP32's: they run in pairs of floats (unevaluated sums h + l, about 46 bits;
 // Dekker 1971, Knuth's two-sum).  Orders HD and above are plain FP32: a lens's
-// term of order j is |w|^j < 0.6^j of its leading one, so their rounding is
-// below 2^-24 0.6^HD = 1.3e-10 of the nearest lenses' leading terms, 1e-8 of a
-// pixel at the tuned grids.  The FP64 near/far mode keeps the FP64 sums.
+// term of order j at a node is |w|^j |e|^j of its leading one, |w| the sub-block's
+// half-diagonal over the lens's distance and |e| the node's offset over that
+// half-diagonal, together below 0.6: |w| by itself where a sub-block is about
+// square, |w| |e| where the level-2 cells are so long that it is one node wide
+// (the nodes then lie on its short axis).  So their rounding is below
+// 2^-24 0.6^HD = 1.3e-10 of the nearest lenses' leading terms, 1e-8 of a pixel at
+// the tuned grids.  Against the FP64 sums at the grids of a paper-scale field, the
+// Table-1 field and 16 batched maps, 1e6 traced rays each lie as far off (rms and
+// median, two digits).  The FP64 near/far mode keeps the FP64 sums.
 constexpr int HD = 12;               // orders carried in pairs
 
 struct df {

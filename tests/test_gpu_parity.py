@@ -473,6 +473,16 @@ def test_mixed_hierarchical_records_match_the_direct_build(ml, l1, l2_sub, p):
     fd.close()
 
 
+@pytest.mark.parametrize("l1,l2_sub,p", [((9.0, 2.0), (3, 1), 16), ((9.0, 2.0), (4, 3), 16), ((2.0, 7.0), (3, 3), 16),
+                                         ((20.0, 1.0), (12, 4), 16)])
+def test_mixed_hierarchical_records_on_clipped_sub_blocks(ml, l1, l2_sub, p):
+    """Long cells of fewer level-2 columns (or rows) than their sides' ratio, as far
+    as the far series converges: a sub-block is one node wide and about as long as
+    the nearest far lens is away, so that its orders hardly decay by themselves, but
+    do at its nodes, on the short axis.  Same bounds as on other cells."""
+    test_mixed_hierarchical_records_match_the_direct_build(ml, l1, l2_sub, p)
+
+
 @pytest.mark.parametrize("l2_sub", [(5, 5), (10, 5), (40, 20)])
 @pytest.mark.parametrize("span_far", [0.0, 1.0, 60.0, 1e9])
 def test_certified_walk_at_any_grid_and_lens_distance(ml, l2_sub, span_far):
