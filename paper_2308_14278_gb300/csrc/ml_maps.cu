@@ -788,8 +788,8 @@ __global__ void __launch_bounds__(LCA_THREADS) k_light_curves_adj(int mnx, int m
         axes[1][tid] = ay;
         // (windows far outside the map, where the weights are zero, are held
         // within a range that cannot overflow)
-        sx[tid] = max(min(ax.i0, mnx + 1024), -1024) - h;
-        sy[tid] = max(min(ay.i0, mny + 1024), -1024) - h;
+        sx[tid] = max(min(ax.i0, mnx), -1024) - h;
+        sy[tid] = max(min(ay.i0, mny), -1024) - h;
     }
     __syncthreads();
     for (int q = tid; q < ns * N; q += blockDim.x) {
@@ -940,7 +940,10 @@ cudaError_t launch_light_curves_adj(int mnx, int mny, const double *d_tracks, in
     const int64_t n = (int64_t)n_tracks * n_samples;
     if (e == cudaSuccess && n > 0) {
         // tracks per launch, within the grid's 2^31 - 1 blocks
-        const int64_t per = std::max<int64_t>(1, std::min<int64_t>(8, n / (152 * 512)));
+        // samples per thread for narrow windows, more than one once 75,000 threads are
+        // busy (a million samples of 0.2 pixels on 300 x 200 pixels, where they meet:
+        // 647 us scattered one by one)
+        const int64_t per = std::max<int64_t>(1, std::min<int64_t>(8, n / 75000));
         const int64_t blocks1 = h <= 1 ? (((n_samples + per - 1) / per) + 127) / 128 + 1 : (n_samples + LCA_CHUNK - 1) / LCA_CHUNK;
         const int64_t step = std::min<int64_t>(n_tracks, 0x7fffffff / blocks1);
         for (int64_t t = 0; t < n_tracks; t += step) {
