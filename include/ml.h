@@ -48,8 +48,12 @@ typedef enum {
 #define ML_PREC_DIRECT64   0  /* FP64 direct sum over all lenses for every ray (§3.2, first formula) */
 #define ML_PREC_NEARFAR64  1  /* FP64 near/far scheme (Eq. 9), node coefficients in FP64 */
 #define ML_PREC_MIXED      2  /* near sum and Taylor evaluation in FP32 on node-relative
-                                 coordinates; node coefficients, node positions and the
-                                 integer pixel base in FP64 */
+                                 coordinates; node positions, macro and sheet terms and the
+                                 integer pixel base in FP64.  Far series: with the
+                                 hierarchical build in pairs of FP32 numbers (about 46 bits;
+                                 orders 12 to 32 in FP32 alone), with ML_BUILD_DIRECT in FP64;
+                                 c_1..c_p and the node's place within its pixel are then
+                                 rounded to FP32 */
 
 /* deposition modes (ml_field_desc.deposit) */
 #define ML_DEPOSIT_NGP 0      /* nearest grid point: uint32 ray counts N_ij (§3.2) */

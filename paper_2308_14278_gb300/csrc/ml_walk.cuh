@@ -1,5 +1,5 @@
-// The certified walk along a lattice row: shared by the counting kernels, the
-// cloud-in-cell forward and its adjoint.
+// The certified walk along a lattice row: shared by the counting kernels and the
+// cloud-in-cell forward.
 #pragma once
 
 #include "ml_task.cuh"
