@@ -1090,6 +1090,7 @@ ShootArgs make_args(const ml_field *f)
     }
     // (three rays and fewer are the rule's own nodes)
     a.piece_max = (float)std::max(3.0, floor(std::min(1e6, 0.15 * std::min(g.l1x, g.l1y) / g.l3x)));
+    a.carry_max = (unsigned)std::min<int64_t>(1 << 20, std::max<int64_t>(0, (1 << 23) - 1 - g.n2x));
     a.ipx_f = (float)(1.0 / g.dpx);
     a.ipy_f = (float)(1.0 / g.dpy);
     a.l3yx = g.l3y / g.l3x;

@@ -95,6 +95,7 @@ struct ShootArgs {
     float rc2;                      // close-pass radius^2 of near_sum_f32 (theta_E^2)
     float rc2u;                     // the same in lattice units (near_sum_lat)
     float piece_max;                // rays per piece of run_nodes: 0.15 level-1 cell widths
+    unsigned carry_max;             // longest run carried into a column: 2^20, and below 2^23 with its rays
     float l3yx_f;                   // l3y / l3x: a ray row in lattice units
     float yx_f;                     // dpx / dpy: y deflection per x deflection unit (pixels)
     double rho_y;                   // (d(macro_y)/d(theta_y) + kappa_*) * l3y / dpy

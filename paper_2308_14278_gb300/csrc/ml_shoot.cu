@@ -723,7 +723,7 @@ __device__ __forceinline__ void count_spans(const RowPoly<P> &rp, const SpanBoun
     // the run's first ray, as if all its rays lay in this column (an exact
     // float); carries that are long, or that could make a run of the 2^23 rays
     // that count_of no longer holds, are flushed first
-    if (rs.cnt > 1048576u || (float)rs.cnt + (uhi - ulo) >= 8388607.f) {
+    if (rs.cnt > a.carry_max) {
         run_flush(rs, a.map_u32, a.g.mnx, a.g.mny);
         rs.cnt = 0;
     }
