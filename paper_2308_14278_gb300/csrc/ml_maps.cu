@@ -751,13 +751,13 @@ cudaError_t launch_peak_stats(const uint32_t *N, int nx, int ny, int along, cons
 // register and is added once.  One thread and 4 (2h + 1)^2 atomics a sample
 // took 5.0 ms for 80 curves of 4096 samples of a 4-pixel source, bound by the
 // L2's atomics, N^2 atomics a sample 0.57 ms for 40 curves, this 0.28 ms
-// (1.5 against 4.5 ms at 16 pixels), bound by issue.  Where samples share few
-// pixels, narrow windows and samples far apart, the block adds N^2 products a
-// sample with atomics (400 x 16 samples 500 pixels apart at 0.5 pixels 202 -> 57
-// us, with the map's clearing).  The choice weighs warp steps: gathering 2.5 a row of the box and, for each of a
-// sample's rows, one per 96 columns of the samples that share it; scattering 3 per
-// 32 products.  By measurement over 250 spacings, widths and directions the lines
-// cross within 15 % of where the times do.
+// (1.5 against 4.5 ms at 16 pixels), bound by issue.  Where samples lie half a
+// window or more apart the block may add N^2 products a sample with atomics
+// instead (400 x 16 samples 500 pixels apart at 0.5 pixels 202 -> 57 us, with the
+// map's clearing).  The choice weighs warp steps: gathering 2.5 a row of the box
+// and, for each of a sample's rows, one per 96 columns of the samples that share
+// it; scattering 3 per 32 products.  By measurement over 250 spacings, widths and
+// directions the lines cross within 15 % of where the times do.
 constexpr int LCA_THREADS = 256;
 constexpr int LCA_CHUNK = 16;
 constexpr int LCA_COLS = 3;
@@ -814,8 +814,9 @@ __global__ void __launch_bounds__(LCA_THREADS) k_light_curves_adj(int mnx, int m
         const float gaps = (float)max(1, ns - 1), live = fminf((float)ns, (float)N * gaps / fmaxf((float)(d - c), 1.f) + 1.f);
         const float gather = 2.5f * (float)(d - c + N) +
                              (float)(ns * N) * ceilf(((float)N + (live - 1.f) * (float)(r - l) / gaps) * (1.f / 96.f));
-        // (samples in one window: gathered, their atomics would meet)
-        scatter = d + r > c + l && gather > 3.f / 32.f * (float)(ns * N * N);
+        // (only samples half a window apart: others' atomics meet, and their products
+        // would round one by one)
+        scatter = (float)(2 * max(d - c, r - l)) >= (float)N * gaps && gather > 3.f / 32.f * (float)(ns * N * N);
     }
     __syncthreads();
     if (scatter) {
@@ -940,10 +941,10 @@ cudaError_t launch_light_curves_adj(int mnx, int mny, const double *d_tracks, in
     const int64_t n = (int64_t)n_tracks * n_samples;
     if (e == cudaSuccess && n > 0) {
         // tracks per launch, within the grid's 2^31 - 1 blocks
-        // samples per thread for narrow windows, more than one once 75,000 threads are
+        // samples per thread for narrow windows, more than one once 30,000 threads are
         // busy (a million samples of 0.2 pixels on 300 x 200 pixels, where they meet:
         // 647 us scattered one by one)
-        const int64_t per = std::max<int64_t>(1, std::min<int64_t>(8, n / 75000));
+        const int64_t per = std::max<int64_t>(1, std::min<int64_t>(8, n / 30000));
         const int64_t blocks1 = h <= 1 ? (((n_samples + per - 1) / per) + 127) / 128 + 1 : (n_samples + LCA_CHUNK - 1) / LCA_CHUNK;
         const int64_t step = std::min<int64_t>(n_tracks, 0x7fffffff / blocks1);
         for (int64_t t = 0; t < n_tracks; t += step) {
