@@ -41,16 +41,14 @@ SMS, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 HBM_GBS_FALLBACK = 6790.0
 # DRAM bytes per ray of the certified counting kernel, from one ncu capture
 # per workload (dram__bytes_read.sum + dram__bytes_write.sum of one launch
-# over a centred slice of the lattice: 2e10 rays of the paper-scale map, level-2
-# (20, 10), and 2e9 of the Table-1 fold field, level-2 (20, 10), whose 84 MB map
-# stays in L2).  They were taken on the walk before its bound was taken once per
-# column; on the present sources the same launches move 209.2 + 252.6 MB (5 %
-# less) and 23.8 + 0 MB, so the figures are upper ends.  They hold for the kernel
-# sources whose code (comments and blank space left out, code_hash) has these
-# sha1 prefixes only.
-TRAFFIC_BYTES_PER_RAY = {"paper": (216.402944e6 + 269.967104e6) / 2.0e10,
-                         "fold": (23.782144e6 + 512.0) / 2.0e9}
-TRAFFIC_SOURCES = {"ml_shoot.cu": "4e7a0a4c", "ml_internal.cuh": "600f1be7", "ml_task.cuh": "891fab5e",
+# over a centred slice of the lattice at a grid that the autotuner picks: 2e10 rays
+# of the paper-scale map, level-1 cells 7.79 x 1.23 theta_E, level-2 (20, 5), and 2e9
+# of the Table-1 fold field, 19.91 x 19.91 theta_E, (5, 5), whose 84 MB map stays in
+# L2).  They hold for the kernel sources whose code (comments and blank space left
+# out, code_hash) has these sha1 prefixes only, and are taken anew when those change.
+TRAFFIC_BYTES_PER_RAY = {"paper": (197.566208e6 + 251.666688e6) / 2.0e10,
+                         "fold": (11.707136e6 + 1280.0) / 2.0e9}
+TRAFFIC_SOURCES = {"ml_shoot.cu": "2c29122c", "ml_internal.cuh": "de856d65", "ml_task.cuh": "891fab5e",
                    "ml_walk.cuh": "b83910bc"}
 
 
