@@ -669,8 +669,8 @@ std::unordered_map<uint64_t, GridChoice> g_measured;   // guarded by g_tune_mu
 // model's error is largest between fields of different kinds (walk lengths,
 // pixel runs), which the measurement settles; its cost is paid once per process
 // and field: three builds and up to twelve timed options, each of an eighth of the
-// lattice (at 1e11 rays; all of one below 2e9, a twenty-fifth beyond 4e11): 82 ms on
-// the paper-scale field, 223 ms on the Table-1 field.
+// lattice (at 1e11 rays; all of one below 2e9, a twenty-fifth beyond 4e11): 88 ms on
+// the paper-scale field, 237 ms on the Table-1 field.
 ml_status tune_grid(const ml_field_desc &d, const std::vector<double> &hx, const std::vector<double> &hy,
                     const std::vector<double> &hm, const double *dx, const double *dy, const double *dm,
                     cudaStream_t s, bool measure, GridChoice &best)

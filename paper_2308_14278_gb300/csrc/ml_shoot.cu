@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(FP64_THREADS) k_shoot_direct64(ShootArgs a)
 // NF_CHUNK rays of one level-2 column; four rays at a time.  Bound by the FP64
 // pipe: 2p + 10 per near lens + about 20 per ray instead of 4p + 16 per near lens
 // + about 40 and five 64-bit divisions: 1.2e7 rays at p = 10 took 2.84 ms, now
-// 1.15 ms.
+// 1.2 ms.
 constexpr int NF_CHUNK = 64;
 
 __global__ void __launch_bounds__(FP64_THREADS) k_shoot_nearfar64(ShootArgs a)
